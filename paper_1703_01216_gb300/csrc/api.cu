@@ -90,6 +90,49 @@ int ensure_wtab(Handle* H, const fr3d_sources* s, cudaStream_t st) {
   return FR3D_OK;
 }
 
+// Combination weights of the unfused row pass (FP64, and n = 512 in FP32): the same table in T, up to
+// kWeightBytes; *W = nullptr (V0 evaluated per voxel instead) when the table would be larger, cannot be
+// allocated, or is not there yet inside a stream capture.  A program that changes its sources on every call
+// rebuilds the table, which costs what the per-voxel evaluation costs.
+constexpr size_t kWeightBytes = 4ull << 30;
+template <typename T> int weights_or_null(Handle* H, const fr3d_sources* s, const T** W, cudaStream_t st) {
+  T*& tab = [H]() -> T*& {
+    if constexpr (sizeof(T) == 4) return H->wtab;
+    else return H->wtab64;
+  }();
+  std::vector<double>& key = sizeof(T) == 4 ? H->wtab_key : H->wtab64_key;
+  size_t& cap = sizeof(T) == 4 ? H->wtab_cap : H->wtab64_cap;
+  *W = nullptr;
+  if (tab && key == H->src_key) {
+    *W = tab;
+    return FR3D_OK;
+  }
+  const size_t need = sizeof(T) * (size_t)s->q * H->Mp * H->n * H->n;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  FR3D_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
+  if (need > kWeightBytes || cs != cudaStreamCaptureStatusNone) return FR3D_OK;
+  if (cap < need) {
+    if (tab) cudaFree(tab);
+    tab = nullptr;
+    cap = 0;
+    key.clear();
+    const cudaError_t e = cudaMalloc(&tab, need);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      tab = nullptr;
+      return FR3D_OK;
+    }
+    FR3D_CUDA_TRY(e);
+    cap = need;
+  }
+  key.clear();
+  if constexpr (sizeof(T) == 4) FR3D_TRY(build_wtab(H, tab, s->q, H->pts64, s->n_points, -s->A0 / kFourPi, st));
+  else FR3D_TRY(build_wtab64(H, tab, s->q, H->pts64, s->n_points, -s->A0 / kFourPi, st));
+  key = H->src_key;
+  *W = tab;
+  return FR3D_OK;
+}
+
 // ------------------------------------------------------------------ forward operator
 template <typename T>
 int fwd_impl(Handle* H, const T* zeta, int Q, T* U, cudaStream_t st) {
@@ -269,9 +312,17 @@ int invert_impl(Handle* H, const T* U, int Q, const fr3d_invert_opts* o, T* out,
   using C = typename Ops<T>::C;
   if constexpr (sizeof(T) == 4) {
     if (H->M > 1) {
-      if (o->output == FR3D_OUT_XI && fused_supported(H->n)) FR3D_TRY(ensure_wtab(H, o->sources, st));
+      const float* W = nullptr;
+      if (o->output == FR3D_OUT_XI) {
+        if (fused_supported(H->n)) {
+          FR3D_TRY(ensure_wtab(H, o->sources, st));
+          W = H->wtab;
+        } else {
+          FR3D_TRY(weights_or_null<float>(H, o->sources, &W, st));
+        }
+      }
       const SrcHost src = o->output == FR3D_OUT_XI ? src_host(H, FR3D_PREC_FP32, o->sources) : SrcHost{};
-      return invert_multi(H, U, Q, o, out, src, st);
+      return invert_multi(H, U, Q, o, out, src, W, st);
     }
   }
   C* Uh = reinterpret_cast<C*>((char*)H->ws + p.uh_off);
@@ -348,13 +399,18 @@ int invert_impl(Handle* H, const T* U, int Q, const fr3d_invert_opts* o, T* out,
     FR3D_TRY(build_dense64(H, st));
     A = H->A64d;
   }
+  const T* W = nullptr;
+  if (o->output == FR3D_OUT_XI) {
+    FR3D_TRY(weights_or_null<T>(H, o->sources, &W, st));
+    prof_mark(H, kStTable, st);
+  }
   // step 2 (solve) + step 3 (inverse DFT) + step 4 (xi = zeta / V0), by chunks of depths
   for (int j0 = 0; j0 < H->Mp; j0 += p.chunk) {
     const int nj = std::min(p.chunk, H->Mp - j0);
     FR3D_TRY(Ops<T>::col_solve1(H, Uh, Tb, A, D, aidx, nb, Q, j0, nj, st));
     prof_mark(H, kStColSolve, st);
     if (o->output == FR3D_OUT_XI)
-      FR3D_TRY(Ops<T>::row_c2r_xi(H, Tb, out, nj, Q, j0, src_host(H, o->precision, o->sources), st));
+      FR3D_TRY(Ops<T>::row_c2r_xi(H, Tb, out, nj, Q, j0, src_host(H, o->precision, o->sources), W, st));
     else
       FR3D_TRY(Ops<T>::row_c2r_plain(H, Tb, out, nj * Q, Q, j0, H->Mp, st));
     prof_mark(H, kStRowC2R, st);

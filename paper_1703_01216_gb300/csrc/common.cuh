@@ -79,6 +79,9 @@ struct Handle {
   float* wtab = nullptr;      // [Q][M'][n][n] V0_q / sum_q' V0_q'^2 for src_key (built on demand)
   std::vector<double> wtab_key;
   size_t wtab_cap = 0;
+  double* wtab64 = nullptr;   // the same in FP64 (FP64 calls)
+  std::vector<double> wtab64_key;
+  size_t wtab64_cap = 0;
   double* pts64 = nullptr;    // [Q*L*3]
   int src_cap = 0;
   // small device words

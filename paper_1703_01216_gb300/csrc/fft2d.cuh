@@ -246,21 +246,32 @@ __device__ __forceinline__ double v0_at(const Src64& s, int q, double x, double 
   return s.coef * acc;
 }
 
+// rows per CTA of the inverse row pass: half tiles where the combination holds accumulators
+template <typename T, int N, int MODE> constexpr int row_c2r_tile() {
+  constexpr int TY0 = RowTile<T, N>::v;
+  return (MODE != 0 && TY0 % 2 == 0) ? TY0 / 2 : TY0;
+}
+
 struct RowGeom {
   double x0, y0, h;  // voxel-centred grid x_a = x0 + (a + 1/2) h
 };
 
 // MODE 0 (plain): input plane ip -> output plane (ip % Q) * out_stride + j0 + ip / Q.
 // MODE 1 (xi):   output plane j0 + blockIdx.y <- sum over q of V0_q * (input plane blockIdx.y Q + q),
-//                divided by sum_q V0_q^2 (Algorithm 1 step 4, several q).
+//                divided by sum_q V0_q^2 (Algorithm 1 step 4, several q), V0_q evaluated per voxel.
+// MODE 2 (xi):   the same with the weights W_q = V0_q / sum_q' V0_q'^2 read from the table W
+//                ([q] planes of w_qs values, depth j0 + blockIdx.y), requested before the transform.
+// MODE 1 is bound by the point sources' reciprocal square roots, above all in FP64 (256^2 x 64, Q = 8, five
+// points: 9.5 of the call's 10.5 ms); MODE 2 reads one value per voxel and source instead: the FP64 call
+// takes 2.87 ms, the FP32 one at 512^2 x 51 depths, ten points, 0.556 ms (before 0.625).
 template <typename T, int N, int MODE>
 __global__ void __launch_bounds__(kThreads) k_row_c2r(const typename cpx<T>::t* __restrict__ in, T* __restrict__ out,
                                                      int Q, int j0, int out_stride,
                                                      typename SrcOf<T>::t src, RowGeom g, const T* __restrict__ zr,
-                                                     const typename cpx<T>::t* __restrict__ tw_half,
+                                                     const T* __restrict__ W, long w_qs,
                                                      const typename cpx<T>::t* __restrict__ tw_full) {
   using C = typename cpx<T>::t;
-  constexpr int L = N / 2, TY0 = RowTile<T, N>::v, TY = (MODE == 1 && TY0 % 2 == 0) ? TY0 / 2 : TY0;
+  constexpr int L = N / 2, TY = row_c2r_tile<T, N, MODE>();
   constexpr int SS = Smem<C, L>::ss;
   constexpr int EPT = (TY * L + kThreads - 1) / kThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -272,14 +283,23 @@ __global__ void __launch_bounds__(kThreads) k_row_c2r(const typename cpx<T>::t* 
   for (int e = tid; e < N; e += kThreads) tws[e] = __ldg(tw_full + e);
   build_passtw<L, 2, kThreads>(ptw, tw_full, tid);
   T num[EPT][2], den[EPT][2];
-  if (MODE == 1) {
+  if (MODE != 0) {
 #pragma unroll
     for (int i = 0; i < EPT; ++i) num[i][0] = num[i][1] = den[i][0] = den[i][1] = (T)0;
   }
-  const int nq = MODE == 1 ? Q : 1;
+  const int nq = MODE != 0 ? Q : 1;
   for (int q = 0; q < nq; ++q) {
-    const int ip = MODE == 1 ? blockIdx.y * Q + q : blockIdx.y;
+    const int ip = MODE != 0 ? blockIdx.y * Q + q : blockIdx.y;
     const C* s = in + ip * ps + y0;
+    C wv[EPT];
+    if (MODE == 2) {
+      const C* wp = reinterpret_cast<const C*>(W + q * w_qs + (long)(j0 + blockIdx.y) * N * N + (long)y0 * N);
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) {
+        const int e = tid + i * kThreads;
+        if (EPT * kThreads == TY * L || e < TY * L) wv[i] = __ldg(wp + e);
+      }
+    }
     for (int e = tid; e < TY * (L + 1); e += kThreads) {
       const int k = e / TY, r = e - k * TY;
       buf[r * SS + pidx<C>(k)] = s[(long)k * N + r];
@@ -311,6 +331,17 @@ __global__ void __launch_bounds__(kThreads) k_row_c2r(const typename cpx<T>::t* 
         const int r = e / L, m = e - r * L;
         oc[(long)r * L + m] = buf[r * SS + pidx<C>(m)];
       }
+    } else if (MODE == 2) {
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) {
+        const int e = tid + i * kThreads;
+        if (EPT * kThreads == TY * L || e < TY * L) {
+          const int r = e / L, m = e - r * L;
+          const C v = buf[r * SS + pidx<C>(m)];
+          num[i][0] += wv[i].x * v.x;
+          num[i][1] += wv[i].y * v.y;
+        }
+      }
     } else {
       const T z = zr[j0 + blockIdx.y];
       const T yy0 = (T)g.y0, xx0 = (T)g.x0, hh = (T)g.h;
@@ -332,7 +363,7 @@ __global__ void __launch_bounds__(kThreads) k_row_c2r(const typename cpx<T>::t* 
     }
     __syncthreads();
   }
-  if (MODE == 1) {
+  if (MODE != 0) {
     T* o = out + (long)(j0 + blockIdx.y) * N * N + (long)y0 * N;
     C* oc = reinterpret_cast<C*>(o);
 #pragma unroll
@@ -340,7 +371,7 @@ __global__ void __launch_bounds__(kThreads) k_row_c2r(const typename cpx<T>::t* 
       const int e = tid + i * kThreads;
       if (EPT * kThreads == TY * L || e < TY * L) {
         const int r = e / L, m = e - r * L;
-        oc[(long)r * L + m] = cmk(num[i][0] / den[i][0], num[i][1] / den[i][1]);
+        oc[(long)r * L + m] = MODE == 2 ? cmk(num[i][0], num[i][1]) : cmk(num[i][0] / den[i][0], num[i][1] / den[i][1]);
       }
     }
   }
@@ -360,10 +391,6 @@ template <int N> struct SmallTile {
   static constexpr int row = divisor_at_most(N, 8);
   static constexpr int col = 4;
 };
-template <typename T, int N, int MODE> constexpr int row_c2r_tile() {
-  constexpr int TY0 = RowTile<T, N>::v;
-  return (MODE == 1 && TY0 % 2 == 0) ? TY0 / 2 : TY0;
-}
 template <typename T, int N, int MODE> constexpr size_t row_c2r_smem() {
   using C = typename cpx<T>::t;
   return sizeof(C) * ((size_t)N + passtw_size<N / 2>() + (size_t)row_c2r_tile<T, N, MODE>() * Smem<C, N / 2>::ss);

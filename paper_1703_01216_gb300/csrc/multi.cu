@@ -565,7 +565,7 @@ int multi_alpha(Handle* H, const MultiWs& w, const double* alphas, int na, int r
 // Algorithm 1 for M > 1 (FP32 data and FFTs, FP64 eigen tables and residual sums).
 // The combination table (XI) is built by the caller.
 int invert_multi(Handle* H, const float* U, int Q, const fr3d_invert_opts* o, float* out, const SrcHost& src,
-                 cudaStream_t st) {
+                 const float* W, cudaStream_t st) {
   FR3D_TRY(ensure_multi_tables(H, st));
   const int nb = o->n_bands > 1 ? o->n_bands : 1;
   std::vector<double> count;
@@ -621,7 +621,7 @@ int invert_multi(Handle* H, const float* U, int Q, const fr3d_invert_opts* o, fl
   }
   prof_mark(H, kStColSolve, st);
   if (fused) {
-    FR3D_TRY(inv_fused_presolved_f32(H, w.Zs, H->wtab, out, Q, o->output, st));
+    FR3D_TRY(inv_fused_presolved_f32(H, w.Zs, W, out, Q, o->output, st));
     prof_mark(H, kStFused, st);
     H->last_launches = launches + 2;
     return FR3D_OK;
@@ -631,7 +631,7 @@ int invert_multi(Handle* H, const float* U, int Q, const fr3d_invert_opts* o, fl
   FR3D_TRY(Ops<float>::col_plain(H, w.Zs, w.Zs, Q * H->Mp, true, st));
   prof_mark(H, kStColInv, st);
   if (o->output == FR3D_OUT_XI)
-    FR3D_TRY(Ops<float>::row_c2r_xi(H, w.Zs, out, H->Mp, Q, 0, src, st));
+    FR3D_TRY(Ops<float>::row_c2r_xi(H, w.Zs, out, H->Mp, Q, 0, src, W, st));
   else
     FR3D_TRY(Ops<float>::row_c2r_plain(H, w.Zs, out, H->Mp * Q, Q, 0, H->Mp, st));
   prof_mark(H, kStRowC2R, st);

@@ -27,8 +27,9 @@ template <typename T> struct Ops {
   // row pass half spectrum -> real; input plane ip -> output plane (ip % Q) * out_stride + j0 + ip / Q
   static int row_c2r_plain(const Handle* H, const C* in, T* out, int nplanes, int Q, int j0, int out_stride,
                            cudaStream_t st);
-  // row pass with the combination xi = sum_q V0_q zeta_q / sum_q V0_q^2 for depths j0 .. j0 + nj - 1
-  static int row_c2r_xi(const Handle* H, const C* in, T* out, int nj, int Q, int j0, const SrcHost& src,
+  // row pass with the combination xi = sum_q V0_q zeta_q / sum_q V0_q^2 for depths j0 .. j0 + nj - 1;
+  // W: the combination weights [Q][M'][n][n], or null to evaluate V0 per voxel
+  static int row_c2r_xi(const Handle* H, const C* in, T* out, int nj, int Q, int j0, const SrcHost& src, const T* W,
                         cudaStream_t st);
   // U~[q][i] = (1/n^2) sum_j A[i][j] zeta~[q][j] for every half-spectrum bin
   static int contract_fwd(const Handle* H, const C* Zh, C* Uh, const T* A, int Q, cudaStream_t st);
@@ -67,6 +68,7 @@ int inv_queue_make_inst(void* dst, const FusedArgs& f, float2* T, int* cnt, int 
 int inv_queue_launch_table(const void* tab, int ninst, int* ctl, int* cnt_all, int ncnt, int total, cudaStream_t st);
 // W_q = V0_q / sum_q' V0_q'^2 on the R grid for the handle's cached sources
 int build_wtab(const Handle* H, float* W, int Q, const double* pts64, int L, double coef, cudaStream_t st);
+int build_wtab64(const Handle* H, double* W, int Q, const double* pts64, int L, double coef, cudaStream_t st);
 
 // alpha-rule partial sums buffer (per block, band and candidate)
 int ensure_partials(Handle* H);
@@ -84,9 +86,10 @@ int learned_alpha(Handle* H, const float2* Uh, int nplanes, int nb, double delta
 // choice, and the workspace bytes the inversion lays out from the start of the handle's workspace
 int ensure_multi_tables(Handle* H, cudaStream_t st);
 size_t multi_ws_bytes(const Handle* H, int Q);
-// src: the point sources of the combination (XI output; used at sizes without the fused inverse)
+// src, W: the point sources and the combination weights (XI output; W may be null at sizes without the fused
+// inverse: V0 is then evaluated per voxel)
 int invert_multi(Handle* H, const float* U, int Q, const fr3d_invert_opts* o, float* out, const SrcHost& src,
-                 cudaStream_t st);
+                 const float* W, cudaStream_t st);
 int choose_multi(Handle* H, const float* U, int Q, const double* alphas, int na, double delta, double tau,
                  int precision, int* aidx, double* residuals, int* info, cudaStream_t st);
 void band_thresholds(const Handle* H, const fr3d_invert_opts* o, int nb, double* thr2);

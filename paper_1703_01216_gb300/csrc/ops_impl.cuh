@@ -63,7 +63,7 @@ static int col_n(const Handle* H, const Op& op, int nplanes, cudaStream_t st) {
 
 template <typename T, int N, int MODE>
 static int row_c2r_n(const Handle* H, const typename cpx<T>::t* in, T* out, int nplanes, int Q, int j0,
-                     int out_stride, const SrcHost& src, cudaStream_t st) {
+                     int out_stride, const SrcHost& src, const T* W, cudaStream_t st) {
   constexpr size_t sm = row_c2r_smem<T, N, MODE>();
   auto kern = k_row_c2r<T, N, MODE>;
   FR3D_TRY(set_smem(kern, sm));
@@ -76,7 +76,7 @@ static int row_c2r_n(const Handle* H, const typename cpx<T>::t* in, T* out, int 
   if constexpr (sizeof(T) == 4) zr = H->zr32;
   else zr = H->zr64;
   dim3 grid(N / row_c2r_tile<T, N, MODE>(), nplanes);
-  kern<<<grid, kThreads, sm, st>>>(in, out, Q, j0, out_stride, s, g, zr, tw_of<T>(H, N / 2), tw_of<T>(H, N));
+  kern<<<grid, kThreads, sm, st>>>(in, out, Q, j0, out_stride, s, g, zr, W, (long)H->Mp * N * N, tw_of<T>(H, N));
   return cudaGetLastError() == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
 }
 
@@ -136,7 +136,7 @@ int Ops<T>::row_c2r_plain(const Handle* H, const C* in, T* out, int nplanes, int
   SrcHost none{nullptr, 0, 0.0};
   switch (H->n) {
 #define X(N) \
-  case N: return row_c2r_n<T, N, 0>(H, in, out, nplanes, Q, j0, out_stride, none, st);
+  case N: return row_c2r_n<T, N, 0>(H, in, out, nplanes, Q, j0, out_stride, none, nullptr, st);
     FR3D_FOR_EACH_N(X)
 #undef X
   }
@@ -144,11 +144,13 @@ int Ops<T>::row_c2r_plain(const Handle* H, const C* in, T* out, int nplanes, int
 }
 
 template <typename T>
-int Ops<T>::row_c2r_xi(const Handle* H, const C* in, T* out, int nj, int Q, int j0, const SrcHost& src,
+int Ops<T>::row_c2r_xi(const Handle* H, const C* in, T* out, int nj, int Q, int j0, const SrcHost& src, const T* W,
                        cudaStream_t st) {
   switch (H->n) {
-#define X(N) \
-  case N: return row_c2r_n<T, N, 1>(H, in, out, nj, Q, j0, 0, src, st);
+#define X(N)                                                                                      \
+  case N:                                                                                         \
+    return W ? row_c2r_n<T, N, 2>(H, in, out, nj, Q, j0, 0, src, W, st)                             \
+             : row_c2r_n<T, N, 1>(H, in, out, nj, Q, j0, 0, src, nullptr, st);
     FR3D_FOR_EACH_N(X)
 #undef X
   }
