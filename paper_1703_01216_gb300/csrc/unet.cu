@@ -34,12 +34,11 @@ constexpr int kL = 4;
 constexpr int kWidth[kL] = {16, 32, 64, 128};
 constexpr int kGuard = 128;
 constexpr int kNumConv = 15;
-constexpr long kWgRange = 4096;   // voxels per weight-gradient CTA
 
 struct Level {
   int D, H, W, Hp, Wp;
-  long Vp, Vs, p_first, p_last;
-  int ntiles;
+  long HW, Vp, Vs;
+  int q_first, q_last;   // interior positions of an (h, w) plane (with the halo between its rows)
 };
 
 Level make_level(int D, int H, int W) {
@@ -51,10 +50,9 @@ Level make_level(int D, int H, int W) {
   l.Wp = W + 2;
   l.Vp = (long)(D + 2) * l.Hp * l.Wp;
   l.Vs = l.Vp + kGuard;
-  const long hw = (long)l.Hp * l.Wp;
-  l.p_first = hw + l.Wp + 1;
-  l.p_last = l.Vp - 1 - (hw + l.Wp + 1);
-  l.ntiles = (int)((l.p_last - l.p_first + 128) / 128);
+  l.HW = (long)l.Hp * l.Wp;
+  l.q_first = l.Wp + 1;
+  l.q_last = (int)l.HW - 2 - l.Wp;
   return l;
 }
 
@@ -81,6 +79,8 @@ struct Layer {
   int out_t = 0, out_off = 0;
   int dgrad = 0;                  // 0 none, 1 with the leaky derivative of the input, 2 plain
   size_t img_f = 0, img_b = 0;    // byte offsets of the weight images
+  int ng_f = 0, ng_b = 0;         // output channels per CTA of the convolution and of its input gradient
+  WgradArgs wg{};                 // weight-gradient plan (the tensors are filled in per call)
 };
 
 }  // namespace
@@ -117,7 +117,9 @@ namespace {
 
 __device__ __forceinline__ float bfv(uint32_t u, int hi) { return __uint_as_float(hi ? (u & 0xFFFF0000u) : (u << 16)); }
 __device__ __forceinline__ uint32_t pk(float a, float b) {
-  return (uint32_t)tc::bf16_rn(a) | ((uint32_t)tc::bf16_rn(b) << 16);
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
 }
 __device__ __forceinline__ void unpack8(const uint4& q, float* f) {
   const uint32_t w[4] = {q.x, q.y, q.z, q.w};
@@ -318,21 +320,37 @@ __global__ void __launch_bounds__(kHeadThreads) k_head_forward(const unsigned ch
   }
 }
 
-// loss = mean_b e2_b / t2_b (FP64 over the block partials in order); keeps t2_b for the gradient
-__global__ void k_loss(const float* __restrict__ part, int nblk, int B, double* __restrict__ sums, float* __restrict__ loss) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double l = 0.0;
-  for (int b = 0; b < B; ++b) {
+// loss = mean_b e2_b / t2_b (FP64 over the block partials, one warp per sample, then the samples in order);
+// keeps t2_b for the gradient
+constexpr int kLossThreads = 256;
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
+  return v;
+}
+__global__ void __launch_bounds__(kLossThreads) k_loss(const float* __restrict__ part, int nblk, int B,
+                                                       double* __restrict__ sums, float* __restrict__ loss) {
+  const int lane = threadIdx.x & 31;
+  for (int b = threadIdx.x >> 5; b < B; b += kLossThreads / 32) {
     double e2 = 0.0, t2 = 0.0;
-    for (int k = 0; k < nblk; ++k) {
-      e2 += part[((long)b * nblk + k) * 2];
-      t2 += part[((long)b * nblk + k) * 2 + 1];
+    for (int k = lane; k < nblk; k += 32) {
+      const float2 v = reinterpret_cast<const float2*>(part)[(long)b * nblk + k];
+      e2 += v.x;
+      t2 += v.y;
     }
-    sums[2 * b] = e2;
-    sums[2 * b + 1] = t2;
-    l += e2 / t2;
+    e2 = warp_sum(e2);
+    t2 = warp_sum(t2);
+    if (lane == 0) {
+      sums[2 * b] = e2;
+      sums[2 * b + 1] = t2;
+    }
   }
-  if (loss) *loss = (float)(l / B);
+  __syncthreads();
+  if (threadIdx.x == 0 && loss) {
+    double l = 0.0;
+    for (int b = 0; b < B; ++b) l += sums[2 * b] / sums[2 * b + 1];
+    *loss = (float)(l / B);
+  }
 }
 
 // head backward: dy = 2 (y_s - t_s) / (B t2_b); gradient of the head input h (bf16(leaky'(h) bf16(w dy)))
@@ -385,101 +403,48 @@ __global__ void __launch_bounds__(kHeadThreads) k_head_backward(const unsigned c
   }
 }
 
-__global__ void k_head_grad_reduce(const float* __restrict__ part, int nblk, int B, float* __restrict__ g) {
-  const int c = threadIdx.x;
-  if (c >= 17) return;
+// one block per head parameter: the block partials in FP64, a fixed tree
+__global__ void __launch_bounds__(kLossThreads) k_head_grad_reduce(const float* __restrict__ part, int n, float* __restrict__ g) {
+  __shared__ double red[kLossThreads / 32];
+  const int c = blockIdx.x;
   double s = 0.0;
-  for (int b = 0; b < B; ++b)
-    for (int k = 0; k < nblk; ++k) s += part[((long)b * nblk + k) * 17 + c];
-  g[c] = (float)s;
-}
-
-// bias gradient partials: per chunk j and block, the sum over positions [p_first, p_last] of each of
-// the chunk's 8 channels (halo positions hold zeros)
-constexpr int kBiasThreads = 256;
-__global__ void __launch_bounds__(kBiasThreads) k_bias_partials(const unsigned char* __restrict__ G, int chunks, int off,
-                                                                long Vs, long p0, long p1, int B, float* __restrict__ part) {
-  __shared__ float red[8][kBiasThreads];
-  const int j = blockIdx.y;
-  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  const long span = p1 - p0 + 1;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < (long)B * span; i += (long)gridDim.x * blockDim.x) {
-    const int b = (int)(i / span);
-    const long p = p0 + (i - (long)b * span);
-    float f[8];
-    unpack8(*reinterpret_cast<const uint4*>(G + (((long)b * chunks + off + j) * Vs + p) * 16), f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] += f[k];
-  }
-#pragma unroll
-  for (int k = 0; k < 8; ++k) red[k][threadIdx.x] = acc[k];
+  for (int k = threadIdx.x; k < n; k += kLossThreads) s += part[(long)k * 17 + c];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int s = kBiasThreads / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kLossThreads / 32; ++w) s += red[w];
+    g[c] = (float)s;
+  }
+}
+
+// Weight images from the FP32 master (see unet_conv.cu): forward [group][e][c pair][f][a = 2, 1, 0][o of the
+// group][16 c] and input gradient [group][e][o pair][f][a = 2, 1, 0][c of the group][16 o] holding
+// W[o][c][2 - a][2 - e][2 - f], both as K-major core matrices [o / 8][2][8][8].
+__global__ void k_images(const float* __restrict__ w, int co, int ci, int ci_pad, int ngf, int ngb,
+                         uint16_t* __restrict__ fwd, uint16_t* __restrict__ bwd) {
+  const int total = 27 * co * ci_pad;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const int cc = i & 7, r = (i >> 3) & 7, h = (i >> 6) & 1;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x < 8) part[((long)j * gridDim.x + blockIdx.x) * 8 + threadIdx.x] = red[threadIdx.x][0];
-}
-
-__global__ void k_bias_reduce(const float* __restrict__ part, int nblk, int co, float* __restrict__ db) {
-  const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= co) return;
-  const int j = o / 8, k = o % 8;
-  double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += part[((long)j * nblk + b) * 8 + k];
-  db[o] = (float)s;
-}
-
-// weight gradient: canonical dW[o][c][tap] (c < ci) = sum over the ranges of the partials (fixed order)
-__global__ void k_wgrad_reduce(const float* __restrict__ part, long nranges, int co, int ci, int ci_pad,
-                               float* __restrict__ dW) {
-  const long total = (long)co * ci * 27;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const int tap = (int)(i % 27);
-    const long oc = i / 27;
-    const int c = (int)(oc % ci), o = (int)(oc / ci);
-    double s = 0.0;
-    for (long r = 0; r < nranges; ++r) s += part[((r * 27 + tap) * co + o) * (long)ci_pad + c];
-    dW[i] = (float)s;
-  }
-}
-
-// weight images from the FP32 master (see unet_conv.cu): forward [ae][c pair][f][o][2][8][8] and input
-// gradient [ae][o pair][f][c][2][8][8] holding W[o][c][2 - a][2 - e][2 - f]
-__global__ void k_images(const float* __restrict__ w, int co, int ci, int ci_pad, uint16_t* __restrict__ fwd,
-                         uint16_t* __restrict__ bwd) {
-  const long total = 27L * co * ci_pad;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    // forward image element i: ((((ae * cpairs + cp) * 3 + f) * co + o) * 16 + h * 8 + cc) with o = 8g + r
-    {
-      const int cc = (int)(i & 7), r = (int)((i >> 3) & 7), h = (int)((i >> 6) & 1);
-      long rest = i >> 7;                     // (((ae * cpairs + cp) * 3 + f) * (co / 8) + g)
-      const int g8 = (int)(rest % (co / 8));
-      rest /= co / 8;
-      const int f = (int)(rest % 3);
+    for (int dir = 0; dir < 2; ++dir) {
+      const int ng = dir ? ngb : ngf, pairs = (dir ? co : ci_pad) / 16;
+      int rest = i >> 7;
+      const int g8 = rest % (ng / 8);
+      rest /= ng / 8;
+      const int a = 2 - rest % 3;
       rest /= 3;
-      const int cpairs = ci_pad / 16;
-      const int cp = (int)(rest % cpairs), ae = (int)(rest / cpairs);
-      const int o = 8 * g8 + r, c = cp * 16 + h * 8 + cc;
-      const float v = c < ci ? w[((long)o * ci + c) * 27 + ae * 3 + f] : 0.f;
-      fwd[i] = tc::bf16_rn(v);
-    }
-    // input-gradient image element i: rows c (ci_pad), columns o (co)
-    {
-      const int cc = (int)(i & 7), r = (int)((i >> 3) & 7), h = (int)((i >> 6) & 1);
-      long rest = i >> 7;
-      const int g8 = (int)(rest % (ci_pad / 8));
-      rest /= ci_pad / 8;
-      const int f = (int)(rest % 3);
+      const int f = rest % 3;
       rest /= 3;
-      const int opairs = co / 16;
-      const int op = (int)(rest % opairs), ae = (int)(rest / opairs);
-      const int c = 8 * g8 + r, o = op * 16 + h * 8 + cc;
-      const int a = ae / 3, e = ae % 3;
-      const float v = c < ci ? w[((long)o * ci + c) * 27 + (2 - a) * 9 + (2 - e) * 3 + (2 - f)] : 0.f;
-      bwd[i] = tc::bf16_rn(v);
+      const int kp = rest % pairs;
+      rest /= pairs;
+      const int e = rest % 3, grp = rest / 3;
+      const int row = grp * ng + 8 * g8 + r, col = kp * 16 + h * 8 + cc;
+      if (dir == 0) {
+        fwd[i] = tc::bf16_rn(col < ci ? w[((long)row * ci + col) * 27 + a * 9 + e * 3 + f] : 0.f);
+      } else {
+        bwd[i] = tc::bf16_rn(row < ci ? w[((long)col * ci + row) * 27 + (2 - a) * 9 + (2 - e) * 3 + (2 - f)] : 0.f);
+      }
     }
   }
 }
@@ -502,7 +467,7 @@ int grid_for(long n, int threads = 256) { return (int)std::max<long>(1, std::min
 int build_images(Unet* U, cudaStream_t st) {
   for (int k = 0; k < kNumConv; ++k) {
     const Layer& Ly = U->layer[k];
-    k_images<<<grid_for(27L * Ly.co * Ly.ci_pad), 256, 0, st>>>(U->params + Ly.woff, Ly.co, Ly.ci, Ly.ci_pad,
+    k_images<<<grid_for(27L * Ly.co * Ly.ci_pad), 256, 0, st>>>(U->params + Ly.woff, Ly.co, Ly.ci, Ly.ci_pad, Ly.ng_f, Ly.ng_b,
                                                                  reinterpret_cast<uint16_t*>(U->imgs + Ly.img_f),
                                                                  reinterpret_cast<uint16_t*>(U->imgs + Ly.img_b));
   }
@@ -517,12 +482,11 @@ ConvArgs conv_args(const Unet* U, int lvl, int B) {
   a.D = L.D;
   a.H = L.H;
   a.W = L.W;
-  a.Hp = L.Hp;
   a.Wp = L.Wp;
+  a.HW = L.HW;
   a.Vs = L.Vs;
-  a.p_first = L.p_first;
-  a.p_last = L.p_last;
-  a.ntiles = L.ntiles;
+  a.q_first = L.q_first;
+  a.ntiles = conv_tiles(L.q_first, L.q_last);
   a.err = U->err;
   return a;
 }
@@ -536,6 +500,7 @@ int conv_forward(Unet* U, int k, int B, cudaStream_t st) {
   a.Cin = Ly.ci_pad;
   a.wimg = U->imgs + Ly.img_f;
   a.N = Ly.co;
+  a.Ng = Ly.ng_f;
   a.y = U->t[Ly.out_t];
   a.y_chunks = U->td[Ly.out_t].C / 8;
   a.y_off = Ly.out_off / 8;
@@ -546,40 +511,14 @@ int conv_forward(Unet* U, int k, int B, cudaStream_t st) {
 
 int conv_backward(Unet* U, int k, int B, cudaStream_t st) {
   const Layer& Ly = U->layer[k];
-  const Level& L = U->lv[Ly.lvl];
-  // weight gradient partials, then the ordered reduction into the canonical gradient
-  WgradArgs w{};
+  // weight and bias gradient: partial sums, then their ordered sum
+  WgradArgs w = Ly.wg;
   w.g = U->g[Ly.out_t];
-  w.g_chunks = U->td[Ly.out_t].C / 8;
-  w.g_off = Ly.out_off / 8;
-  w.Cout = Ly.co;
   w.x = U->t[Ly.in_t];
-  w.x_chunks = U->td[Ly.in_t].C / 8;
-  w.x_off = Ly.in_off / 8;
-  w.Cin = Ly.ci_pad;
-  w.ndw = 3 * Ly.co <= 128 ? 3 : 1;
   w.B = B;
-  w.Hp = L.Hp;
-  w.Wp = L.Wp;
-  w.Vs = L.Vs;
-  w.p_first = L.p_first;
-  w.p_last = L.p_last;
-  w.range = kWgRange;
-  w.ranges_per_sample = wgrad_ranges_per_sample(L.p_first, L.p_last, kWgRange);
   w.partials = U->partials;
   w.err = U->err;
-  const long nranges = (long)B * w.ranges_per_sample;
-  if ((size_t)(nranges * 27 * Ly.co * Ly.ci_pad) > U->partial_floats) return FR3D_ERR_UNSUPPORTED_SIZE;
-  FR3D_TRY(wgrad3_launch(w, st));
-  k_wgrad_reduce<<<grid_for((long)Ly.co * Ly.ci * 27), 256, 0, st>>>(U->partials, nranges, Ly.co, Ly.ci, Ly.ci_pad,
-                                                                        U->grads + Ly.woff);
-  // bias gradient
-  const int nblk = 64;
-  k_bias_partials<<<dim3(nblk, Ly.co / 8), kBiasThreads, 0, st>>>(U->g[Ly.out_t], U->td[Ly.out_t].C / 8,
-                                                                   Ly.out_off / 8, L.Vs, L.p_first, L.p_last, B,
-                                                                   U->red);
-  k_bias_reduce<<<1, 128, 0, st>>>(U->red, nblk, Ly.co, U->grads + Ly.woff + (long)Ly.co * Ly.ci * 27);
-  FR3D_CUDA_TRY(cudaGetLastError());
+  FR3D_TRY(wgrad3_launch(w, Ly.ci, U->grads + Ly.woff, U->grads + Ly.woff + (long)Ly.co * Ly.ci * 27, st));
   // input gradient
   if (Ly.dgrad) {
     ConvArgs a = conv_args(U, Ly.lvl, B);
@@ -589,6 +528,7 @@ int conv_backward(Unet* U, int k, int B, cudaStream_t st) {
     a.Cin = Ly.co;
     a.wimg = U->imgs + Ly.img_b;
     a.N = Ly.ci_pad;
+    a.Ng = Ly.ng_b;
     a.y = U->g[Ly.in_t];
     a.y_chunks = U->td[Ly.in_t].C / 8;
     a.y_off = Ly.in_off / 8;
@@ -639,10 +579,10 @@ int forward(Unet* U, const float* x, int B, const float* t, float* out, cudaStre
 int backward(Unet* U, const float* t, int B, float* loss, cudaStream_t st) {
   const Level& L0 = U->lv[0];
   const int nblk = 128;
-  k_loss<<<1, 32, 0, st>>>(U->red, nblk, B, U->lossbuf, loss);
+  k_loss<<<1, kLossThreads, 0, st>>>(U->red, nblk, B, U->lossbuf, loss);
   k_head_backward<<<dim3(nblk, B), kHeadThreads, 0, st>>>(U->t[T_D2], larg(L0), U->y, t, U->params + U->head_off,
                                                           U->in_scale, B, U->lossbuf, U->g[T_D2], U->red);
-  k_head_grad_reduce<<<1, 32, 0, st>>>(U->red, nblk, B, U->grads + U->head_off);
+  k_head_grad_reduce<<<17, kLossThreads, 0, st>>>(U->red, nblk * B, U->grads + U->head_off);
   FR3D_CUDA_TRY(cudaGetLastError());
   for (int l = 0; l <= kL - 2; ++l) {
     const int k = 9 + 2 * (kL - 2 - l);
@@ -787,14 +727,32 @@ extern "C" int fr3d_unet_create(int depth, int height, int width, int max_batch,
       Ly.img_b = ioff;
       ioff += (ib + 255) & ~(size_t)255;
       const Level& L = U->lv[Ly.lvl];
-      const size_t nr = (size_t)max_batch * wgrad_ranges_per_sample(L.p_first, L.p_last, kWgRange);
-      pmax = std::max(pmax, nr * 27 * Ly.co * Ly.ci_pad);
+      const int nt = conv_tiles(L.q_first, L.q_last);
+      Ly.ng_f = conv_group(Ly.ci_pad, Ly.co, L.D, nt, max_batch);
+      Ly.ng_b = conv_group(Ly.co, Ly.ci_pad, L.D, nt, max_batch);
+      WgradArgs& w = Ly.wg;
+      w.g_chunks = U->td[Ly.out_t].C / 8;
+      w.g_off = Ly.out_off / 8;
+      w.Cout = Ly.co;
+      w.x_chunks = U->td[Ly.in_t].C / 8;
+      w.x_off = Ly.in_off / 8;
+      w.Cin = Ly.ci_pad;
+      w.D = L.D;
+      w.Wp = L.Wp;
+      w.HW = L.HW;
+      w.Vs = L.Vs;
+      w.zero_pos = L.Vp;
+      w.q_first = L.q_first;
+      w.q_last = L.q_last;
+      if (!Ly.ng_f || !Ly.ng_b || wgrad_plan(&w, max_batch) != FR3D_OK) rc = FR3D_ERR_UNSUPPORTED_SIZE;
+      pmax = std::max(pmax, wgrad_partial_floats(w, max_batch));
     }
+    if (rc) break;
     U->head_off = off;
     U->n_params = off + kWidth[0] + 1;
     U->img_bytes = ioff;
     U->partial_floats = pmax;
-    U->red_floats = (size_t)std::max(128 * 17 * max_batch, 64 * 16 * 8);
+    U->red_floats = (size_t)128 * 17 * max_batch;
     const size_t np = (size_t)U->n_params;
     if (cudaMalloc(&U->params, np * 4) != cudaSuccess || cudaMalloc(&U->grads, np * 4) != cudaSuccess ||
         cudaMalloc(&U->m, np * 4) != cudaSuccess || cudaMalloc(&U->v, np * 4) != cudaSuccess ||

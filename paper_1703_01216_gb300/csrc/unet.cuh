@@ -15,36 +15,49 @@ enum ConvMode { kConvFwd = 0, kConvDgradMask = 1, kConvDgradPlain = 2 };
 struct ConvArgs {
   const unsigned char* x;
   int x_chunks, x_off, Cin;
-  const unsigned char* wimg;   // [9 (a, e)][Cin / 16][3 (f)][N][2 chunks][8][8] BF16, K-major core matrices
-  int N;
+  // [N / Ng groups][3 (e)][Cin / 16][3 (f)][3 (a = 2, 1, 0)][Ng / 8][2 chunks][8][8] BF16, K-major core matrices
+  const unsigned char* wimg;
+  int N, Ng;                   // output channels, and those of one CTA (conv_group)
   unsigned char* y;
   int y_chunks, y_off;
   const float* bias;           // kConvFwd: [N] (may be null)
   const unsigned char* mask;   // kConvDgradMask: the tensor whose leaky derivative multiplies the result
   int mask_chunks, mask_off;
   int mode;
-  int B, D, H, W, Hp, Wp;
-  long Vs, p_first, p_last;
-  int ntiles;                  // 128-position tiles per sample covering [p_first, p_last]
+  int B, D, H, W, Wp;
+  long HW, Vs;                 // voxels of a padded (h, w) plane, and of a padded volume with its guard
+  int q_first;                 // first interior position of a plane
+  int ntiles;                  // 128-position tiles of a plane (conv_tiles)
   int* err;                    // FR3D_INFO_TIMEOUT on a bounded wait that gave up (may be null)
+  int ngroups, nd, nchunks, stages, slog;   // set by conv3_launch (slog: log2 of the accumulator slots)
 };
 
-// Weight gradient partials: for every voxel range r, tap and (o, c): sum over the range of G[p][o] X[p + s][c].
+constexpr int kWgVox = 64;     // voxels (K) of a weight-gradient stage
+constexpr int kWgChain = 4096; // voxels at most that one FP32 accumulator of the weight gradient adds up
+// floats of one row of a weight-gradient partial: 27 / 3 taps x Cg input channels, the bias sum, padding
+__host__ __device__ constexpr int wgrad_row_floats(int Cg) { return 9 * Cg + 4; }
+
+// Weight gradient: partial sums per unit (sample, span of in-plane positions, depth chunk) and pair of
+// channel groups, then their ordered sum.
 struct WgradArgs {
   const unsigned char* g;      // output gradient (pre-activation), Cout channels
   int g_chunks, g_off, Cout;
   const unsigned char* x;      // layer input, Cin channels
   int x_chunks, x_off, Cin;
-  int ndw;                     // 3: the three f taps stacked in the rows (3 Cout <= 128); 1: one tap per CTA
-  int B, Hp, Wp;
-  long Vs, p_first, p_last, range;
-  int ranges_per_sample;
-  float* partials;             // [B * ranges_per_sample][27][Cout][Cin]
+  int B, D, Wp;
+  long HW, Vs, zero_pos;       // zero_pos: first voxel of the planes' zero guard
+  int q_first, q_last;         // interior positions of a plane (with the halo between them)
+  float* partials;             // [units][pairs][3 Og][wgrad_row_floats(Cg)]
   int* err;
+  int Og, Cg, n_og, n_cg, span, nspans, nd, nchunks, stages;   // wgrad_plan
 };
 
+int conv_tiles(int q_first, int q_last);
+int conv_group(int Cin, int N, int D, int ntiles, int B);
 int conv3_launch(const ConvArgs& a, cudaStream_t st);
-int wgrad3_launch(const WgradArgs& a, cudaStream_t st);
-int wgrad_ranges_per_sample(long p_first, long p_last, long range);
+int wgrad_plan(WgradArgs* a, int B);
+size_t wgrad_partial_floats(const WgradArgs& a, int B);
+// dW [Cout][ci][27] and db [Cout]; ci: the layer's unpadded input channels
+int wgrad3_launch(const WgradArgs& a, int ci, float* dW, float* db, cudaStream_t st);
 
 }  // namespace fr3d

@@ -9,15 +9,27 @@
 // (an MMA tile of M = 128 rows) and only the interior ones are stored.
 //
 // Forward and input-gradient kernel (k_conv3): D[p][n] = sum over taps and input channels of
-// X[p + s(tap)][c] * Wimg[tap][n][c].  Per (a, e) and 16 input channels one pipeline stage holds a slab of
-// 130 positions of two channel chunks (two bulk copies; the three f taps are the same slab with the
-// operand's start moved by 16 bytes) and the three taps' weights (one bulk copy of a prepared image):
-// three MMAs of K = 16.  The input gradient is the same kernel with the image of the flipped, transposed
-// weights (the adjoint of a correlation is the correlation with the flipped kernel).
+// X[p + s(tap)][c] * Wimg[tap][n][c], by plane sweeps.  A CTA keeps the weights of Ng output channels in
+// shared memory for its whole life and walks the depth of a 128-position tile of the (h, w) plane: every
+// input plane is loaded once per (e, 16 input channels) (a slab of 130 positions of two channel chunks; the
+// three f taps are the same slab with the operand's start moved by 16 bytes) and multiplied with the taps of
+// all three a at once, N = 3 Ng columns: they belong to the outputs of the three neighbouring planes, whose
+// accumulators ("slots" of Ng TMEM columns, zeroed when they are handed back) lie side by side in a ring.  One
+// CTA per SM runs up to four independent pipes (tiles), each with a producer warp, an MMA warp and four epilogue
+// warps that drain a plane's slot while the next planes run.
+//   Before, every (a, e) re-read the slab and the weights for each tile, with N = Ng columns per MMA: 188 us for
+//   16 -> 16 channels at 128^2 x 32, batch 8, now 78 us (tensors in and out of HBM: 41 us).  A single pipe takes
+//   197 us, two 115: an MMA of 48 columns needs 46 cycles of issue and operand reads, and what a pipe waits and
+//   issues between its stages is only hidden behind the other pipes' MMAs.
+//   The products of an output are accumulated in the order (a, e, channel pair, f) whatever Ng, depth chunk
+//   and grid, so the results do not depend on them, bit for bit.
 // Weight-gradient kernel (k_wgrad3): dW[tap][o][c] = sum_p G[p][o] X[p + s(tap)][c], a GEMM whose K is the
 // voxels: both operands come straight from CP planes, which hold 8 channels per 16 bytes, i.e. they are
-// MN-major operands (the instruction descriptor's transpose bits).  The rows stack the three f taps of a
-// (a, e) pair (each the output gradient shifted by one voxel) when 3 Cout <= 128.
+// MN-major operands (the instruction descriptor's transpose bits).  The rows stack the three f taps (the
+// output gradient shifted by one voxel) of Og <= 32 output channels, the columns the three e taps of Cg <= 48
+// input channels; the three a taps are three accumulators fed from the input planes d - 1, d, d + 1 of a ring,
+// so a plane sweep loads every input window once instead of once per a, and one CTA covers all 27 taps.  16
+// columns of ones behind the a = 1 windows make the bias gradient in the same MMAs.
 #include <math.h>
 
 #include <algorithm>
@@ -33,40 +45,29 @@ namespace {
 
 constexpr long kPolls = 1L << 22;
 constexpr uint32_t kSleepNs = 1000;   // suspend-time hint of the waits: a waiting thread parks (bound: kPolls * 1 us)
-constexpr int kConvStages = 4;
-constexpr int kSlabPos = 130;                   // positions of one (a, e) slab: 128 + the two f neighbours
+constexpr int kSlabPos = 130;                   // positions of one e slab: 128 + the two f neighbours
 constexpr int kSlabBytes = kSlabPos * 16;       // one channel chunk of a slab
+constexpr int kItemBytes = 2 * kSlabBytes;      // one (e, 16 channels) item: two chunks
+constexpr int kConvStageBytes = 3 * kItemBytes; // a stage: three consecutive items (3 Cin / 16 items per plane)
+constexpr int kConvMaxStages = 8;               // per pipe
+constexpr int kConvPipes = 4;                   // pipes of a CTA at most
+constexpr int kPipeThreads = 192;               // per pipe: four epilogue warps, a producer and an MMA warp
+constexpr int kTmemCols = 512;
+constexpr int kMaxSlots = kTmemCols / 16;
+constexpr size_t kMaxSmem = 227 * 1024;
 // MN-major shared-memory descriptor: byte strides between core matrices along MN (channel chunks) and
-// along K (groups of 8 voxels)
-constexpr uint32_t kMnStrideMN_LBO = 0;         // 0: the MN stride goes in the SBO field, the K stride in LBO (measured)
-
+// along K (groups of 8 voxels); the MN stride goes in the SBO field, the K stride in LBO (measured)
 __device__ __forceinline__ uint64_t desc_mn(uint32_t saddr, uint32_t mn_stride, uint32_t k_stride) {
-  return kMnStrideMN_LBO ? tc::desc_kmajor(saddr, mn_stride, k_stride) : tc::desc_kmajor(saddr, k_stride, mn_stride);
+  return tc::desc_kmajor(saddr, k_stride, mn_stride);
 }
 __host__ __device__ constexpr uint32_t idesc_mn(int M, int N) {
   return tc::idesc_bf16(M, N) | (1u << 15) | (1u << 16);
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int k = 0; k < 8; ++k) v[k] = __uint_as_float(r[k]);
-}
-
-__device__ __forceinline__ bool interior(long p, int Hp, int Wp, int D, int H, int W) {
-  const long hw = (long)Hp * Wp;
-  const int d = (int)(p / hw);
-  const long rem = p - (long)d * hw;
-  const int h = (int)(rem / Wp), w = (int)(rem - (long)h * Wp);
-  return d >= 1 && d <= D && h >= 1 && h <= H && w >= 1 && w <= W;
-}
-
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
-  return (uint32_t)tc::bf16_rn(a) | ((uint32_t)tc::bf16_rn(b) << 16);
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
 }
 __device__ __forceinline__ float lo16(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float hi16(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
@@ -79,317 +80,623 @@ __host__ __device__ __forceinline__ uint32_t tmem_cols(int n) {
   return c;
 }
 
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(bar)) : "memory");
+}
+
 // ------------------------------------------------------------------------------------------ k_conv3
-__global__ void __launch_bounds__(128) k_conv3(ConvArgs a) {
+// a unit of work: the depth chunk o0 .. o0 + cnt - 1 (padded plane indices) of the tile at q0 of sample b
+struct ConvUnit {
+  int b, q0, o0, cnt;
+  int kmin, kmax;   // input planes o0 - 1 + k, k in [kmin, kmax]: the zero halo planes at both ends are skipped
+};
+__device__ __forceinline__ ConvUnit conv_unit(const ConvArgs& a, int u) {
+  ConvUnit c;
+  const int ch = u % a.nchunks, r = u / a.nchunks;
+  c.b = r / a.ntiles;
+  c.q0 = a.q_first + (r - c.b * a.ntiles) * 128;
+  c.o0 = 1 + ch * a.nd;
+  c.cnt = min(a.nd, a.D + 1 - c.o0);
+  c.kmin = c.o0 == 1 ? 1 : 0;
+  c.kmax = c.o0 + c.cnt - 1 == a.D ? c.cnt : c.cnt + 1;
+  return c;
+}
+
+struct ConvPipe {
+  uint64_t full[kConvMaxStages], empty[kConvMaxStages], sdone[kMaxSlots], sfree[kMaxSlots], zeroed, drain;
+  int issued;
+};
+
+template <int PIPES>
+__global__ void __launch_bounds__(PIPES* kPipeThreads, 1) k_conv3(ConvArgs a) {
   extern __shared__ __align__(128) unsigned char sm[];
-  __shared__ __align__(8) uint64_t full[kConvStages], empty[kConvStages], done;
+  __shared__ __align__(8) ConvPipe pipes[PIPES];
+  __shared__ __align__(8) uint64_t wfull;
   __shared__ uint32_t tbase;
   __shared__ int sabort;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int N = a.N;
-  const int bBytes = 3 * N * 32;
-  const int stage = ((2 * kSlabBytes + bBytes) + 127) & ~127;
-  const int cpairs = a.Cin / 16, niter = 9 * cpairs;
-  const uint32_t ncols = tmem_cols(N);
-  if (tid == 0) {
-    for (int s = 0; s < kConvStages; ++s) {
-      tc::mbar_init(&full[s], 1);
-      tc::mbar_init(&empty[s], 1);
+  __shared__ float sbias[64];
+  // warps [0, 4 PIPES): epilogue (pipe = warp / 4; warp % 4 picks the 32 TMEM lanes it may read), then the
+  // producers, then the MMA warps
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int role = warp < 4 * PIPES ? 0 : (warp < 5 * PIPES ? 1 : 2);
+  const int pipe = role == 0 ? warp >> 2 : (role == 1 ? warp - 4 * PIPES : warp - 5 * PIPES);
+  ConvPipe& P = pipes[pipe];
+  uint64_t *full = P.full, *empty = P.empty, *sdone = P.sdone, *sfree = P.sfree;
+  const int Ng = a.Ng, cpairs = a.Cin / 16, S = a.stages, slog = a.slog, nslots = 1 << slog, smask = nslots - 1;
+  const int grp = blockIdx.x % a.ngroups;
+  // units go round the CTAs first and round their pipes next, so that the CTAs' shares differ by one unit at most
+  const int ctas = gridDim.x / a.ngroups, w0 = blockIdx.x / a.ngroups + pipe * ctas, wstep = ctas * PIPES;
+  const int nunits = a.B * a.ntiles * a.nchunks;
+  const uint32_t wbytes = (uint32_t)(27 * a.Cin * Ng * 2);
+  unsigned char* stages = sm + ((wbytes + 127) & ~127u) + (size_t)pipe * S * kConvStageBytes;
+  if (tid < PIPES) {
+    ConvPipe& Q = pipes[tid];
+    for (int s = 0; s < S; ++s) {
+      tc::mbar_init(&Q.full[s], 1);
+      tc::mbar_init(&Q.empty[s], 1);
     }
-    tc::mbar_init(&done, 1);
+    for (int s = 0; s < nslots; ++s) {
+      tc::mbar_init(&Q.sdone[s], 1);
+      tc::mbar_init(&Q.sfree[s], 4);
+    }
+    tc::mbar_init(&Q.zeroed, 4);
+    tc::mbar_init(&Q.drain, 1);
+    Q.issued = 0;
+    if (tid == 0) {
+      tc::mbar_init(&wfull, 1);
+      sabort = 0;
+    }
     tc::mbar_fence_init();
-    sabort = 0;
   }
-  if (warp == 0) tc::tmem_alloc(&tbase, ncols);
+  if (tid < Ng) sbias[tid] = a.bias ? a.bias[grp * Ng + tid] : 0.f;
+  if (warp == 0) tc::tmem_alloc(&tbase, kTmemCols);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = tbase;
-  const long HW = (long)a.Hp * a.Wp;
-  const uint32_t idesc = tc::idesc_bf16(128, N);
-  long g = 0;           // pipeline uses so far (all tiles of this CTA)
-  uint32_t tcount = 0;  // tiles so far
-  const long ntot = (long)a.B * a.ntiles;
-  for (long t = blockIdx.x; t < ntot; t += gridDim.x, ++tcount) {
-    const int b = (int)(t / a.ntiles);
-    const long p0 = a.p_first + (t - (long)b * a.ntiles) * 128;
-    if (tid == 0) {
-      // producer
-      for (int it = 0; it < niter && !flag(&sabort); ++it) {
-        const long gi = g + it;
-        const int s = (int)(gi % kConvStages);
-        const long use = gi / kConvStages;
-        if (use > 0 && !tc::mbar_wait_sleep(&empty[s], (uint32_t)((use - 1) & 1), kPolls, kSleepNs)) {
-          sabort = 1;
-          break;
+  const uint32_t tmem = tbase + pipe * (kTmemCols / PIPES);
+  if (role == 1) {
+    // producer: the group's weights once, then the slabs of every plane of every unit
+    if (pipe == 0) {
+      if (lane == 0) tc::mbar_arrive_expect_tx(&wfull, wbytes);
+      __syncwarp();
+      const unsigned char* wsrc = a.wimg + (size_t)grp * wbytes;
+      for (uint32_t o = lane * 8192u; o < wbytes; o += 32u * 8192u)
+        tc::bulk_g2s(sm + o, wsrc + o, min(8192u, wbytes - o), &wfull);
+    }
+    int s = 0, use = 0, stop = 0;
+    const int it = lane >> 1, h = lane & 1;
+    for (int u = w0; u < nunits && !stop; u += wstep) {
+      const ConvUnit c = conv_unit(a, u);
+      for (int k = c.kmin; k <= c.kmax && !stop; ++k) {
+        const long row = (long)(c.o0 - 1 + k) * a.HW + c.q0 - 1;
+        for (int st = 0; st < cpairs; ++st) {
+          if (lane == 0) {
+            stop = flag(&sabort);
+            if (!stop && use > 0 && !tc::mbar_wait_sleep(&empty[s], (uint32_t)((use - 1) & 1), kPolls, kSleepNs)) {
+              sabort = 1;
+              stop = 1;
+            }
+            if (!stop) {
+              tc::mbar_arrive_expect_tx(&full[s], kConvStageBytes);
+              ++P.issued;
+            }
+          }
+          stop = __shfl_sync(0xffffffffu, stop, 0);
+          __syncwarp();
+          if (stop) break;
+          if (lane < 6) {
+            const int i = 3 * st + it, e = i / cpairs, cp = i - e * cpairs;
+            const long chunk = (long)c.b * a.x_chunks + a.x_off + 2 * cp + h;
+            tc::bulk_g2s(stages + s * kConvStageBytes + it * kItemBytes + h * kSlabBytes,
+                         a.x + (chunk * a.Vs + row + (e - 1) * a.Wp) * 16, kSlabBytes, &full[s]);
+          }
+          if (++s == S) {
+            s = 0;
+            ++use;
+          }
         }
-        const int ae = it / cpairs, cp = it - ae * cpairs;
-        const long off = (long)(ae / 3 - 1) * HW + (long)(ae % 3 - 1) * a.Wp - 1;
-        unsigned char* st = sm + (size_t)s * stage;
-        tc::mbar_arrive_expect_tx(&full[s], (uint32_t)(2 * kSlabBytes + bBytes));
-        for (int h = 0; h < 2; ++h) {
-          const long chunk = (long)b * a.x_chunks + a.x_off + 2 * cp + h;
-          tc::bulk_g2s(st + h * kSlabBytes, a.x + (chunk * a.Vs + p0 + off) * 16, kSlabBytes, &full[s]);
-        }
-        tc::bulk_g2s(st + 2 * kSlabBytes, a.wimg + (size_t)it * bBytes, (uint32_t)bBytes, &full[s]);
       }
-    } else if (tid == 32) {
-      // MMA issuer
-      for (int it = 0; it < niter && !flag(&sabort); ++it) {
-        const long gi = g + it;
-        const int s = (int)(gi % kConvStages);
-        if (!tc::mbar_wait_sleep(&full[s], (uint32_t)((gi / kConvStages) & 1), kPolls, kSleepNs)) {
+    }
+  } else if (role == 2) {
+    // MMA warp: every value is the same in all its lanes (the tensor instructions take their descriptors from
+    // uniform registers; a single-lane branch cost 165 cycles per MMA), one elected lane issues
+    bool ok = tc::mbar_wait_sleep(&wfull, 0u, kPolls, kSleepNs) && tc::mbar_wait_sleep(&P.zeroed, 0u, kPolls, kSleepNs);
+    int s = 0, ph = 0, n0 = 0;
+    const uint32_t da0 = tc::smem_addr(stages) >> 4, db0 = tc::smem_addr(sm) >> 4;
+    const uint64_t dah = tc::desc_kmajor(0, kSlabBytes, 128), dbh = tc::desc_kmajor(0, 128, 256);
+    const uint32_t id1 = tc::idesc_bf16(128, Ng), dn = (uint32_t)(Ng >> 3) << 17;   // one more block of Ng columns
+    for (int u = w0; u < nunits && ok; u += wstep) {
+      const ConvUnit c = conv_unit(a, u);
+      for (int k = c.kmin; k <= c.kmax && ok; ++k) {
+        // the outputs this input plane feeds: r = k - 2 .. k (taps a = 2, 1, 0; weight blocks 0, 1, 2): one run of
+        // adjacent slots, or two where the ring wraps
+        const int r0 = max(0, k - 2), r1 = min(c.cnt - 1, k);
+        const int s0 = (n0 + r0) & smask;
+        if (k < c.cnt || k == c.kmin)   // slots touched for the first time: wait until they have been drained
+          for (int r = k == c.kmin ? r0 : k; r <= r1 && ok; ++r) {
+            const int n = n0 + r;
+            if (n > smask) ok = tc::mbar_wait_sleep(&sfree[n & smask], (uint32_t)(((n >> slog) - 1) & 1), kPolls, kSleepNs);
+          }
+        const int m0 = min(r1 - r0 + 1, nslots - s0), m1 = r1 - r0 + 1 - m0;
+        const uint32_t c0 = tmem + s0 * Ng, i0 = id1 + (m0 - 1) * dn, i1 = id1 + (m1 - 1) * dn;
+        const uint32_t b0 = (uint32_t)((r0 - (k - 2)) * 2 * Ng), b1 = b0 + m0 * 2 * Ng;
+        tc::fence_after_sync();
+        for (int st = 0; st < cpairs && ok; ++st) {
+          ok = tc::mbar_wait_sleep(&full[s], (uint32_t)ph, kPolls, kSleepNs);
+          if (!ok) break;
+          tc::fence_after_sync();
+          const uint32_t da = da0 + s * (kConvStageBytes / 16), db = db0 + st * 54 * Ng;
+          if (tc::elect_one()) {
+#pragma unroll
+            for (int x = 0; x < 9; ++x) {   // items x / 3, taps f = x % 3
+              const uint64_t dax = dah | (da + (x / 3) * (kItemBytes / 16) + x % 3);
+              tc::mma_bf16(c0, dax, dbh | (db + x * 6 * Ng + b0), i0, true);
+              if (m1 > 0) tc::mma_bf16(tmem, dax, dbh | (db + x * 6 * Ng + b1), i1, true);
+            }
+            tc::mma_commit(&empty[s]);
+          }
+          __syncwarp();
+          if (++s == S) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+        // outputs complete with this plane
+        if (ok && k >= 2 && tc::elect_one())
+          for (int r = k - 2; r < c.cnt && (r == k - 2 || k == c.kmax); ++r) tc::mma_commit(&sdone[(n0 + r) & smask]);
+        if (ok && k < 2 && k == c.kmax && tc::elect_one())
+          for (int r = 0; r < c.cnt; ++r) tc::mma_commit(&sdone[(n0 + r) & smask]);
+        __syncwarp();
+      }
+      n0 += c.cnt;
+      if (flag(&sabort)) ok = false;
+    }
+    if (!ok) sabort = 1;
+    if (tc::elect_one()) tc::mma_commit(&P.drain);
+    __syncwarp();
+  } else {
+    // epilogue: row = position q0 + row of the tile
+    const int row = tid & 127;
+    int n0 = 0;
+    bool ok = true;
+    const uint32_t tw = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    // every slot starts at zero, and is handed back as zeros
+    for (int j = 0; j < nslots * Ng; j += 16) tc::tmem_st16_zero(tw + j);
+    tc::tmem_st_wait();
+    tc::fence_before_sync();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&P.zeroed);
+    for (int u = w0; u < nunits && ok; u += wstep) {
+      const ConvUnit c = conv_unit(a, u);
+      const int q = c.q0 + row, hh = q / a.Wp, ww = q - hh * a.Wp;
+      const bool valid = hh >= 1 && hh <= a.H && ww >= 1 && ww <= a.W;
+      for (int r = 0; r < c.cnt; ++r) {
+        const int n = n0 + r, use = n >> slog, slot = n & smask;
+        const bool got = !flag(&sabort) && tc::mbar_wait_sleep(&sdone[slot], (uint32_t)(use & 1), kPolls, kSleepNs);
+        ok = __all_sync(0xffffffffu, got);
+        if (!ok) {
           sabort = 1;
           break;
         }
         tc::fence_after_sync();
-        const uint32_t st = tc::smem_addr(sm + (size_t)s * stage);
-        for (int f = 0; f < 3; ++f) {
-          const uint64_t da = tc::desc_kmajor(st + 16 * f, kSlabBytes, 128);
-          const uint64_t db = tc::desc_kmajor(st + 2 * kSlabBytes + f * N * 32, 128, 256);
-          tc::mma_bf16(tmem, da, db, idesc, it > 0 || f > 0);
-        }
-        tc::mma_commit(&empty[s]);
-      }
-      tc::mma_commit(&done);
-    }
-    g += niter;
-    __syncwarp();
-    const bool ok = tc::mbar_wait_sleep(&done, tcount & 1u, kPolls, kSleepNs);
-    if (!ok) sabort = 1;
-    tc::fence_after_sync();
-    __syncthreads();
-    if (sabort) break;
-    // epilogue: row tid = position p0 + tid
-    const long p = p0 + tid;
-    const bool valid = p <= a.p_last && interior(p, a.Hp, a.Wp, a.D, a.H, a.W);
-    const uint32_t tw = tmem + ((uint32_t)(warp * 32) << 16);
-    for (int j = 0; j < N / 8; ++j) {
-      float v[8];
-      tmem_ld8(tw + 8 * j, v);
-      if (!valid) continue;
-      if (a.mode == kConvFwd) {
+        const long p = (long)(c.o0 + r) * a.HW + q;
+        for (int j = 0; j < Ng / 8; j += 2) {
+          float v[16];
+          tc::tmem_ld16(tw + slot * Ng + 8 * j, v);
+          tc::tmem_st16_zero(tw + slot * Ng + 8 * j);
+          if (j + 2 >= Ng / 8) {   // the slot's last read: hand it back
+            tc::tmem_st_wait();
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sfree[slot]);
+          }
+          if (valid) {
+            const long jc = (long)grp * (Ng / 8) + j;
+            if (a.mode == kConvFwd) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float z = v[k] + (a.bias ? a.bias[8 * j + k] : 0.f);
-          v[k] = z > 0.f ? z : kLeaky * z;
-        }
-      } else if (a.mode == kConvDgradMask) {
-        const uint4 m = *reinterpret_cast<const uint4*>(
-            a.mask + (((long)b * a.mask_chunks + a.mask_off + j) * a.Vs + p) * 16);
-        const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
-        // the gradient is stored (rounded) first, then scaled by the leaky derivative and rounded again,
-        // as the two steps of the chain rule store it
+              for (int k = 0; k < 16; ++k) {
+                const float z = v[k] + sbias[8 * j + k];
+                v[k] = z > 0.f ? z : kLeaky * z;
+              }
+            } else if (a.mode == kConvDgradMask) {
+              // the gradient is stored (rounded) first, then scaled by the leaky derivative and rounded again,
+              // as the two steps of the chain rule store it
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          v[2 * k] = tc::bf16_val(tc::bf16_rn(v[2 * k]));
-          v[2 * k + 1] = tc::bf16_val(tc::bf16_rn(v[2 * k + 1]));
-          if (!(lo16(mw[k]) > 0.f)) v[2 * k] *= kLeaky;
-          if (!(hi16(mw[k]) > 0.f)) v[2 * k + 1] *= kLeaky;
+              for (int h = 0; h < 2; ++h) {
+                const uint4 m = __ldg(reinterpret_cast<const uint4*>(
+                    a.mask + (((long)c.b * a.mask_chunks + a.mask_off + jc + h) * a.Vs + p) * 16));
+                const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  float& lo = v[8 * h + 2 * k];
+                  float& hi = v[8 * h + 2 * k + 1];
+                  const uint32_t st = pack2(lo, hi);
+                  lo = lo16(st);
+                  hi = hi16(st);
+                  if (!(lo16(mw[k]) > 0.f)) lo *= kLeaky;
+                  if (!(hi16(mw[k]) > 0.f)) hi *= kLeaky;
+                }
+              }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              uint4 o;
+              o.x = pack2(v[8 * h], v[8 * h + 1]);
+              o.y = pack2(v[8 * h + 2], v[8 * h + 3]);
+              o.z = pack2(v[8 * h + 4], v[8 * h + 5]);
+              o.w = pack2(v[8 * h + 6], v[8 * h + 7]);
+              *reinterpret_cast<uint4*>(a.y + (((long)c.b * a.y_chunks + a.y_off + jc + h) * a.Vs + p) * 16) = o;
+            }
+          }
+          __syncwarp();
         }
       }
-      uint4 o;
-      o.x = pack2(v[0], v[1]);
-      o.y = pack2(v[2], v[3]);
-      o.z = pack2(v[4], v[5]);
-      o.w = pack2(v[6], v[7]);
-      *reinterpret_cast<uint4*>(a.y + (((long)b * a.y_chunks + a.y_off + j) * a.Vs + p) * 16) = o;
+      n0 += c.cnt;
     }
-    tc::fence_before_sync();
-    __syncthreads();
-  }
-  if (sabort) {
-    if (tid == 0 && a.err) atomicOr(a.err, FR3D_INFO_TIMEOUT);
-    tc::mbar_wait(&done, tcount & 1u, kPolls);   // give in-flight MMAs a bounded chance to finish
   }
   tc::fence_before_sync();
   __syncthreads();
+  if (sabort && tid < PIPES) {
+    // a bounded wait gave up: report it, and let the copies and MMAs in flight finish (bounded) before leaving
+    ConvPipe& Q = pipes[tid];
+    if (a.err) atomicOr(a.err, FR3D_INFO_TIMEOUT);
+    tc::mbar_wait(&wfull, 0u, kPolls);
+    for (int i = max(0, Q.issued - S); i < Q.issued; ++i) tc::mbar_wait(&Q.full[i % S], (uint32_t)((i / S) & 1), kPolls);
+    tc::mbar_wait(&Q.drain, 0u, kPolls);
+  }
+  __syncthreads();
   tc::fence_after_sync();
-  if (warp == 0) tc::tmem_dealloc(tmem, ncols);
+  if (warp == 0) tc::tmem_dealloc(tbase, kTmemCols);
 }
 
 // ------------------------------------------------------------------------------------------ k_wgrad3
-constexpr int kWgStages = 3;
-constexpr int kWgVox = 64;                      // voxels (K) per stage: four MMAs of K = 16 (a multiple of 16 dividing the range)
-constexpr int kWgPlane = kWgVox * 16;           // bytes of one channel chunk of a stage
+constexpr int kWgMaxStages = 8;
+constexpr int kWgThreads = 192;                 // warps 0-3 epilogue, 4 producer, 5 MMA
+constexpr int kWgPlane = kWgVox * 16;           // bytes of one window: kWgVox voxels of one channel chunk
 
-__global__ void __launch_bounds__(128) k_wgrad3(WgradArgs a) {
+// One CTA: the partial sums of one unit (sample, span of in-plane positions, depth chunk) for one pair of
+// channel groups.  A span is walked in sub-ranges of kWgVox positions, each swept through the depth.  Stage k
+// of a sweep holds the input plane g0 - 1 + k (three e windows per chunk, then 16 columns of ones) and, from
+// k = 2 on, the gradient plane g0 - 2 + k (three f windows per chunk): the MMAs of step k multiply that gradient
+// plane with the input planes of stages k - 2 (a = 0), k - 1 (a = 1, with the ones) and k (a = 2).  The 16 row
+// groups of an MMA reach past the 3 Og gradient rows into whatever lies behind them in shared memory: those
+// rows' accumulators are never read.
+// Bound (16 -> 16 channels at level 0): 12 window copies of 1 KB per 64 voxels from L2, and 3 x (4 KB + 1.5 KB)
+// of operand reads per 16 voxels, against 9 x 8 copies and 9 x 4.5 KB with one CTA per (a, e): 764 -> 223 us at
+// 128^2 x 32, batch 8, and the reduction, which used one thread per element, 224 -> 42 us.
+__global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
   extern __shared__ __align__(128) unsigned char sm[];
-  __shared__ __align__(8) uint64_t full[kWgStages], empty[kWgStages], done;
+  __shared__ __align__(8) uint64_t full[kWgMaxStages], empty[kWgMaxStages], done;
   __shared__ uint32_t tbase;
-  __shared__ int sabort;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int N = a.Cin;
-  const int gc = a.Cout / 8;                     // output-gradient chunks per f tap
-  const int rows_loaded = a.ndw * gc;            // row groups with data (the rest stay zero)
-  const int aBytes = 16 * kWgPlane;              // 128 rows
-  const int bBytes = (N / 8) * kWgPlane;
-  const int stage = aBytes + bBytes;
-  const uint32_t ncols = tmem_cols(N);
-  const int ntg = a.ndw == 3 ? 9 : 27;
-  const int tg = blockIdx.x % ntg;
-  const long r = blockIdx.x / ntg;
-  const int b = (int)(r / a.ranges_per_sample);
-  const long v0 = a.p_first + (r - (long)b * a.ranges_per_sample) * a.range;
-  const long v1 = min(v0 + a.range, a.p_last + 1);
-  const int nst = v1 > v0 ? (int)((v1 - v0 + kWgVox - 1) / kWgVox) : 0;
-  const int ae = a.ndw == 3 ? tg : tg / 3, fsel = a.ndw == 3 ? 0 : tg % 3;
-  const long HW = (long)a.Hp * a.Wp;
-  const long xoff = (long)(ae / 3 - 1) * HW + (long)(ae % 3 - 1) * a.Wp + (a.ndw == 3 ? 0 : fsel - 1);
-  // zero every stage once (the unused row groups of A are read as zeros)
-  for (int e = tid; e < kWgStages * stage / 16; e += 128) reinterpret_cast<uint4*>(sm)[e] = make_uint4(0, 0, 0, 0);
+  __shared__ int sabort, issued;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int S = a.stages;
+  const int nG = 3 * a.Og / 8, nX = 3 * a.Cg / 8;
+  const int stage = (nG + nX + 2) * kWgPlane;
+  const int N = 3 * a.Cg;
+  const uint32_t ncols = tmem_cols(3 * N + 16);
+  const int npairs = a.n_og * a.n_cg;
+  const int pair = blockIdx.x % npairs, unit = blockIdx.x / npairs;
+  const int og = pair / a.n_cg, cg = pair - og * a.n_cg;
+  const int ch = unit % a.nchunks, rest = unit / a.nchunks;
+  const int b = rest / a.nspans, sp = rest - b * a.nspans;
+  const int g0 = 1 + ch * a.nd, cnt = min(a.nd, a.D + 1 - g0);
+  const int v0 = a.q_first + sp * a.span, v1 = min(v0 + a.span, a.q_last + 1);   // in-plane positions [v0, v1)
+  // zeros everywhere once (the row groups past the gradient's), ones behind every stage's input windows
+  for (int e = tid; e < (S * stage + 2 * kWgPlane) / 16; e += kWgThreads) {
+    const int o = e * 16;
+    const uint32_t w = o < S * stage && o % stage >= (nG + nX) * kWgPlane ? 0x3F803F80u : 0u;
+    reinterpret_cast<uint4*>(sm)[e] = make_uint4(w, w, w, w);
+  }
   tc::fence_proxy_async();
   if (tid == 0) {
-    for (int s = 0; s < kWgStages; ++s) {
+    for (int s = 0; s < S; ++s) {
       tc::mbar_init(&full[s], 1);
       tc::mbar_init(&empty[s], 1);
     }
     tc::mbar_init(&done, 1);
     tc::mbar_fence_init();
     sabort = 0;
+    issued = 0;
   }
   if (warp == 0) tc::tmem_alloc(&tbase, ncols);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tbase;
-  const uint32_t idesc = idesc_mn(128, N);
-  if (warp == 0) {
-    // producer warp: lane 0 waits for the stage and posts its byte count, then the lanes issue the
-    // stage's copies (rows_loaded gradient chunks, N / 8 input chunks), one copy per lane
-    const int lane = tid & 31;
-    const int ncopy = rows_loaded + N / 8;
-    for (int it = 0; it < nst; ++it) {
-      const int s = it % kWgStages;
-      const int use = it / kWgStages;
-      int stop = 0;
-      if (lane == 0) {
-        stop = flag(&sabort);
-        if (!stop && use > 0 && !tc::mbar_wait_sleep(&empty[s], (uint32_t)((use - 1) & 1), kPolls, kSleepNs)) {
-          sabort = 1;
-          stop = 1;
+  if (warp == 4) {
+    // producer warp: lane 0 waits for the stage and posts its byte count, then each lane copies one window
+    // (the last K step of a span may end past it: the gradient's tail comes from the plane's zero guard)
+    const bool isg = lane < nG;
+    const int j = isg ? lane : lane - nG;
+    const int gc = (isg ? a.Og : a.Cg) / 8, t3 = j / gc, cc = j - t3 * gc;   // f or e, chunk in the group
+    const unsigned char* src = isg ? a.g + ((long)b * a.g_chunks + a.g_off + og * gc + cc) * a.Vs * 16
+                                   : a.x + ((long)b * a.x_chunks + a.x_off + cg * gc + cc) * a.Vs * 16;
+    const long shift = isg ? -(t3 - 1) : (long)(t3 - 1) * a.Wp;
+    int s = 0, use = 0, stop = 0;
+    for (int v = v0; v < v1 && !stop; v += kWgVox) {
+      const int rem = min(kWgVox, v1 - v), kv = (rem + 15) & ~15;
+      for (int k = 0; k < cnt + 2; ++k) {
+        if (lane == 0) {
+          stop = flag(&sabort);
+          if (!stop && use > 0 && !tc::mbar_wait_sleep(&empty[s], (uint32_t)((use - 1) & 1), kPolls, kSleepNs)) {
+            sabort = 1;
+            stop = 1;
+          }
+          if (!stop) {
+            tc::mbar_arrive_expect_tx(&full[s], (uint32_t)((nX + (k >= 2 ? nG : 0)) * kv * 16));
+            ++issued;
+          }
         }
-        if (!stop) tc::mbar_arrive_expect_tx(&full[s], (uint32_t)(ncopy * kWgPlane));
-      }
-      stop = __shfl_sync(0xffffffffu, stop, 0);
-      __syncwarp();   // the byte count is posted before any copy of the stage is issued
-      if (stop) break;
-      const long v = v0 + (long)it * kWgVox;
-      unsigned char* st = sm + (size_t)s * stage;
-      for (int k = lane; k < ncopy; k += 32) {
-        if (k < rows_loaded) {
-          // A: row group (fi, c) = output gradient chunk c at positions v - (fi - 1) (ndw = 3), or c at v
-          const int fi = k / gc, c = k - fi * gc;
-          const long pos = v - (a.ndw == 3 ? fi - 1 : 0);
-          const long chunk = (long)b * a.g_chunks + a.g_off + c;
-          tc::bulk_g2s(st + k * kWgPlane, a.g + (chunk * a.Vs + pos) * 16, kWgPlane, &full[s]);
-        } else {
-          // B: input chunk c at positions v + the (a, e[, f]) shift
-          const int c = k - rows_loaded;
-          const long chunk = (long)b * a.x_chunks + a.x_off + c;
-          tc::bulk_g2s(st + aBytes + c * kWgPlane, a.x + (chunk * a.Vs + v + xoff) * 16, kWgPlane, &full[s]);
+        stop = __shfl_sync(0xffffffffu, stop, 0);
+        __syncwarp();   // the byte count is posted before any copy of the stage is issued
+        if (stop) break;
+        unsigned char* dst = sm + s * stage + lane * kWgPlane;
+        if (isg) {
+          if (k >= 2) {
+            tc::bulk_g2s(dst, src + ((long)(g0 - 2 + k) * a.HW + v + shift) * 16, (uint32_t)(rem * 16), &full[s]);
+            if (kv > rem) tc::bulk_g2s(dst + rem * 16, src + a.zero_pos * 16, (uint32_t)((kv - rem) * 16), &full[s]);
+          }
+        } else if (lane < nG + nX) {
+          tc::bulk_g2s(dst, src + ((long)(g0 - 1 + k) * a.HW + v + shift) * 16, (uint32_t)(kv * 16), &full[s]);
+        }
+        if (++s == S) {
+          s = 0;
+          ++use;
         }
       }
     }
-  } else if (tid == 32) {
-    for (int it = 0; it < nst && !flag(&sabort); ++it) {
-      const int s = it % kWgStages;
-      if (!tc::mbar_wait_sleep(&full[s], (uint32_t)((it / kWgStages) & 1), kPolls, kSleepNs)) {
-        sabort = 1;
-        break;
+  } else if (warp == 5) {
+    // MMA warp: uniform values, one elected lane issues (as in k_conv3)
+    const uint32_t idn = idesc_mn(128, N), id1 = idesc_mn(128, N + 16);
+    const uint64_t dh = desc_mn(0, kWgPlane, 128);
+    const uint32_t d0 = tc::smem_addr(sm) >> 4, xoff = nG * kWgPlane / 16, st16 = stage / 16;
+    int s = 0, ph = 0;
+    bool ok = true, acc = false;
+    for (int v = v0; v < v1 && ok; v += kWgVox) {
+      const int ks = (min(kWgVox, v1 - v) + 15) / 16;
+      for (int k = 0; k < cnt + 2; ++k) {
+        ok = tc::mbar_wait_sleep(&full[s], (uint32_t)ph, kPolls, kSleepNs);
+        if (!ok) break;
+        if (k >= 2) {
+          tc::fence_after_sync();
+          const int s1 = s >= 1 ? s - 1 : s - 1 + S, s2 = s >= 2 ? s - 2 : s - 2 + S;
+          const uint32_t da = d0 + s * st16;
+          const uint32_t x0 = d0 + s2 * st16 + xoff, x1 = d0 + s1 * st16 + xoff, x2 = da + xoff;
+          if (tc::elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < kWgVox / 16; ++kk)
+              if (kk < ks) {
+                tc::mma_bf16(tmem, dh | (da + 16 * kk), dh | (x0 + 16 * kk), idn, acc || kk > 0);
+                tc::mma_bf16(tmem + N, dh | (da + 16 * kk), dh | (x2 + 16 * kk), idn, acc || kk > 0);
+                tc::mma_bf16(tmem + 2 * N, dh | (da + 16 * kk), dh | (x1 + 16 * kk), id1, acc || kk > 0);
+              }
+            tc::mma_commit(&empty[s2]);
+            if (k == cnt + 1) {
+              tc::mma_commit(&empty[s1]);
+              tc::mma_commit(&empty[s]);
+            }
+          }
+          acc = true;
+          __syncwarp();
+        }
+        if (++s == S) {
+          s = 0;
+          ph ^= 1;
+        }
       }
-      tc::fence_after_sync();
-      const uint32_t st = tc::smem_addr(sm + (size_t)s * stage);
-      for (int k = 0; k < kWgVox / 16; ++k) {
-        const uint64_t da = desc_mn(st + 256 * k, kWgPlane, 128);
-        const uint64_t db = desc_mn(st + aBytes + 256 * k, kWgPlane, 128);
-        tc::mma_bf16(tmem, da, db, idesc, it > 0 || k > 0);
-      }
-      tc::mma_commit(&empty[s]);
     }
-    tc::mma_commit(&done);
-  }
-  __syncwarp();
-  const bool ok = nst == 0 || tc::mbar_wait_sleep(&done, 0u, kPolls, kSleepNs);
-  if (!ok) sabort = 1;
-  tc::fence_after_sync();
-  __syncthreads();
-  // epilogue: row tid = (fi, o) of the stacked taps; partials [r][tap][o][c]
-  const uint32_t tw = tmem + ((uint32_t)(warp * 32) << 16);
-  const bool row_ok = tid < rows_loaded * 8 && !sabort;
-  const int fi = tid / a.Cout, o = tid - fi * a.Cout;
-  const int tap = a.ndw == 3 ? ae * 3 + fi : ae * 3 + fsel;
-  float* dst = a.partials + ((r * 27 + tap) * (long)a.Cout + o) * N;
-  for (int j = 0; j < N / 8; ++j) {
-    float v[8];
-    tmem_ld8(tw + 8 * j, v);
-    if (!row_ok) continue;
-    if (nst == 0)
-      for (int k = 0; k < 8; ++k) v[k] = 0.f;
-    *reinterpret_cast<float4*>(dst + 8 * j) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4*>(dst + 8 * j + 4) = make_float4(v[4], v[5], v[6], v[7]);
-  }
-  if (sabort) {
-    if (tid == 0 && a.err) atomicOr(a.err, FR3D_INFO_TIMEOUT);
-    if (nst > 0) tc::mbar_wait(&done, 0u, kPolls);
+    if (!ok) sabort = 1;
+    if (tc::elect_one()) tc::mma_commit(&done);
+    __syncwarp();
+  } else {
+    // epilogue: row tid = (f, o); columns [a = 0 | 2 | 1][e][c], then the ones
+    const bool got = tc::mbar_wait_sleep(&done, 0u, kPolls, kSleepNs);
+    if (!__all_sync(0xffffffffu, got)) sabort = 1;
+    tc::fence_after_sync();
+    const uint32_t tw = tmem + ((uint32_t)(warp * 32) << 16);
+    const int rs = wgrad_row_floats(a.Cg);
+    float* dst = a.partials + ((long)blockIdx.x * 3 * a.Og + tid) * rs;
+    for (int n = 0; n < 3 * N; n += 16) {
+      float v[16];
+      tc::tmem_ld16(tw + n, v);
+      if (tid < 3 * a.Og)
+#pragma unroll
+        for (int k = 0; k < 16; k += 4)
+          *reinterpret_cast<float4*>(dst + n + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+    }
+    float v[16];
+    tc::tmem_ld16(tw + 3 * N, v);
+    if (tid < 3 * a.Og) dst[3 * N] = v[0];
   }
   tc::fence_before_sync();
+  __syncthreads();
+  if (sabort && tid == 0) {
+    if (a.err) atomicOr(a.err, FR3D_INFO_TIMEOUT);
+    for (int i = max(0, issued - S); i < issued; ++i) tc::mbar_wait(&full[i % S], (uint32_t)((i / S) & 1), kPolls);
+    tc::mbar_wait(&done, 0u, kPolls);
+  }
   __syncthreads();
   tc::fence_after_sync();
   if (warp == 0) tc::tmem_dealloc(tmem, ncols);
 }
 
-std::mutex g_conv_mu;
-
-int launch_cfg(const void* kern, size_t smem, int ncols, int* occ_out) {
-  std::lock_guard<std::mutex> lock(g_conv_mu);
-  FR3D_TRY(smem_optin(kern, smem));
-  int occ = 0;
-  occ = resident_ctas(kern, 128, smem);
-  // the resident CTAs of an SM must not ask for more than its 512 TMEM columns together
-  const int cap = 512 / ncols;
-  while (occ > cap) {
-    smem += 8192;
-    FR3D_TRY(smem_optin(kern, smem));
-    occ = resident_ctas(kern, 128, smem);
+// dW[o][c][tap] (c < ci) and db[o]: the units' partial sums added in FP64 in a fixed order (8 threads per
+// element take every eighth unit, then the eight sums in order).  Bound by the partials' bytes.
+constexpr int kWgRedX = 32, kWgRedY = 8;
+__global__ void __launch_bounds__(kWgRedX* kWgRedY) k_wgrad_reduce(WgradArgs a, int nunits, int ci, float* __restrict__ dW,
+                                                                  float* __restrict__ db) {
+  __shared__ double red[kWgRedY][kWgRedX];
+  const int rs = wgrad_row_floats(a.Cg), N = 3 * a.Cg;
+  const int per = 3 * a.Og * rs, npairs = a.n_og * a.n_cg;
+  const int i = blockIdx.x * kWgRedX + threadIdx.x;
+  double s = 0.0;
+  if (i < per * npairs) {
+    const float* p = a.partials + i;
+    const long ustep = (long)per * npairs;
+#pragma unroll 8
+    for (int u = threadIdx.y; u < nunits; u += kWgRedY) s += (double)__ldg(p + u * ustep);
   }
-  if (occ < 1) return FR3D_ERR_UNSUPPORTED_SIZE;
-  *occ_out = occ;
-  return (int)smem;
+  red[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y != 0 || i >= per * npairs) return;
+  for (int y = 1; y < kWgRedY; ++y) s += red[y][threadIdx.x];
+  const int pair = i / per, m = (i - pair * per) / rs, n = i % rs;
+  const int og = pair / a.n_cg, cg = pair - og * a.n_cg;
+  const int f = m / a.Og, o = og * a.Og + m % a.Og;
+  if (n < 3 * N) {
+    const int part = n / N, e = (n % N) / a.Cg, c = cg * a.Cg + n % a.Cg;
+    const int ta = part == 0 ? 0 : 3 - part;
+    if (c < ci) dW[((long)o * ci + c) * 27 + ta * 9 + e * 3 + f] = (float)s;
+  } else if (n == 3 * N && f == 1 && cg == 0) {
+    db[o] = (float)s;
+  }
+}
+
+int sm_count(int* sms) {
+  int dev = 0;
+  FR3D_CUDA_TRY(cudaGetDevice(&dev));
+  FR3D_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
+  return FR3D_OK;
+}
+
+// input planes a depth chunk of nd outputs reads (the zero halo planes at the ends of the depth are skipped)
+int conv_planes(int D, int nd) { return nd >= D ? D : (2 * nd >= D ? nd + 1 : nd + 2); }
+
+// A way to run a convolution: output channels per CTA, pipes per CTA, stages per pipe, planes per depth chunk.
+struct ConvPlan {
+  int Ng = 0, pipes = 0, stages = 0, nd = 0;
+  double cost = 0;
+};
+size_t conv_weight_bytes(int Cin, int Ng) { return ((size_t)27 * Cin * Ng * 2 + 127) & ~(size_t)127; }
+constexpr size_t kSmemSlack = 3 * 1024;   // static shared memory and alignment kept out of the dynamic allocation
+
+// Cycles per MMA of N columns with c pipes of a CTA at work, fitted to measurements (N = 48, 96, 144): alone, the
+// waits and the issue of a pipe's stages are exposed; with four pipes the operand reads and the slabs' writes to
+// shared memory are what is left.  (16 -> 16 channels at 128^2 x 32, batch 8: 197 us with one pipe, 115 with two,
+// 78 with four.)
+double conv_mma_cycles(int N, int c) { return c == 1 ? 49 + 0.75 * N : (c == 2 ? 60 + 0.35 * N : 45 + 0.38 * N); }
+
+// The plan whose largest share takes the fewest cycles: units of a CTA x planes x MMAs x cycles per MMA.  Larger
+// groups read the slabs less often, smaller ones and shorter depth chunks spread a small volume over more SMs.
+// ng: only this group size (0: any).
+ConvPlan conv_plan(int Cin, int N, int D, int ntiles, int B, int ng, int sms) {
+  ConvPlan best;
+  const int cand[] = {64, 48, 32, 16};
+  for (int Ng : cand) {
+    if (N % Ng || (ng && Ng != ng)) continue;
+    const size_t wb = conv_weight_bytes(Cin, Ng);
+    if (wb > kMaxSmem - kSmemSlack) continue;
+    for (int pipes = kConvPipes; pipes >= 1; pipes >>= 1) {
+      if (4 * Ng > kTmemCols / pipes) continue;   // four slots: three live, one being drained
+      const int stages = (int)std::min<size_t>(kConvMaxStages, (kMaxSmem - kSmemSlack - wb) / (pipes * (size_t)kConvStageBytes));
+      if (stages < (pipes == 1 ? 4 : 3)) continue;
+      const int workers = std::max(1, sms / (N / Ng));
+      for (int nch = 1; nch <= std::min(D, 16); ++nch) {
+        const int nd = (D + nch - 1) / nch;
+        const long units = (long)B * ntiles * ((D + nd - 1) / nd);
+        const long share = (units + workers - 1) / workers;
+        const double mma = conv_mma_cycles(3 * Ng, (int)std::min<long>(pipes, share));
+        const double c = share * (conv_planes(D, nd) * (Cin / 16) * 9 * mma + 300);
+        if (!best.Ng || c < best.cost) best = ConvPlan{Ng, pipes, stages, nd, c};
+      }
+    }
+  }
+  return best;
+}
+
+template <int PIPES> int conv3_launch_t(const ConvArgs& a, int ctas, cudaStream_t st) {
+  // all of the SM's tensor memory is one CTA's: ask for more than half of its shared memory
+  const size_t smem = std::max(conv_weight_bytes(a.Cin, a.Ng) + (size_t)PIPES * a.stages * kConvStageBytes, (size_t)120 * 1024);
+  FR3D_TRY(smem_optin(reinterpret_cast<const void*>(k_conv3<PIPES>), smem));
+  k_conv3<PIPES><<<ctas, PIPES * kPipeThreads, smem, st>>>(a);
+  FR3D_CUDA_TRY(cudaGetLastError());
+  return FR3D_OK;
 }
 
 }  // namespace
 
-int conv3_launch(const ConvArgs& a, cudaStream_t st) {
-  if (a.Cin % 16 || a.N % 16 || a.N < 16 || a.N > 256) return FR3D_ERR_UNSUPPORTED_SIZE;
-  const int bBytes = 3 * a.N * 32;
-  const size_t stage = ((2 * kSlabBytes + bBytes) + 127) & ~127;
-  int occ = 0;
-  const int smem = launch_cfg(reinterpret_cast<const void*>(k_conv3), stage * kConvStages, (int)tmem_cols(a.N), &occ);
-  if (smem < 0) return smem;
-  int dev = 0, sms = 0;
-  FR3D_CUDA_TRY(cudaGetDevice(&dev));
-  FR3D_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const long ntot = (long)a.B * a.ntiles;
-  const int grid = (int)std::max<long>(1, std::min<long>(ntot, (long)occ * sms));
-  k_conv3<<<grid, 128, smem, st>>>(a);
-  FR3D_CUDA_TRY(cudaGetLastError());
+int conv_tiles(int q_first, int q_last) { return (q_last - q_first + 128) / 128; }
+
+int conv_group(int Cin, int N, int D, int ntiles, int B) {
+  int sms = 0;
+  if (sm_count(&sms) != FR3D_OK) return 0;
+  return conv_plan(Cin, N, D, ntiles, B, 0, sms).Ng;
+}
+
+int conv3_launch(const ConvArgs& args, cudaStream_t st) {
+  ConvArgs a = args;
+  if (a.Cin % 16 || a.Ng % 16 || a.Ng < 16 || a.Ng > 64 || a.N % a.Ng) return FR3D_ERR_UNSUPPORTED_SIZE;
+  int sms = 0;
+  FR3D_TRY(sm_count(&sms));
+  const ConvPlan p = conv_plan(a.Cin, a.N, a.D, a.ntiles, a.B, a.Ng, sms);
+  if (!p.Ng) return FR3D_ERR_UNSUPPORTED_SIZE;
+  a.ngroups = a.N / a.Ng;
+  a.nd = p.nd;
+  a.nchunks = (a.D + a.nd - 1) / a.nd;
+  a.stages = p.stages;
+  a.slog = 0;
+  while ((2 << a.slog) * a.Ng <= kTmemCols / p.pipes) ++a.slog;   // slots of a pipe's ring: a power of two
+  const long units = (long)a.B * a.ntiles * a.nchunks;
+  const long ctas = std::max<long>(1, std::min<long>(units, sms / a.ngroups));
+  switch (p.pipes) {
+    case 4: return conv3_launch_t<4>(a, (int)ctas * a.ngroups, st);
+    case 2: return conv3_launch_t<2>(a, (int)ctas * a.ngroups, st);
+    default: return conv3_launch_t<1>(a, (int)ctas * a.ngroups, st);
+  }
+}
+
+// Channel groups and units of a layer's weight gradient for batches up to B (fills Og .. nchunks, stages).
+// A unit's accumulators see at most kWgChain voxels, as many as one FP32 chain of the partial sums may have.
+int wgrad_plan(WgradArgs* a, int B) {
+  if (a->Cin % 16 || a->Cout % 16) return FR3D_ERR_UNSUPPORTED_SIZE;
+  a->Og = a->Cout % 32 == 0 ? 32 : 16;
+  a->Cg = a->Cin % 48 == 0 ? 48 : (a->Cin % 32 == 0 ? 32 : 16);
+  a->n_og = a->Cout / a->Og;
+  a->n_cg = a->Cin / a->Cg;
+  a->nd = std::min(a->D, kWgChain / kWgVox);
+  a->nchunks = (a->D + a->nd - 1) / a->nd;
+  a->nd = (a->D + a->nchunks - 1) / a->nchunks;
+  const int stage = (3 * a->Og / 8 + 3 * a->Cg / 8 + 2) * kWgPlane;
+  const bool two = tmem_cols(9 * a->Cg + 16) <= kTmemCols / 2;   // two CTAs per SM share the tensor memory
+  const size_t room = (two ? 112 * 1024 : kMaxSmem) - kSmemSlack - 2 * kWgPlane;
+  a->stages = (int)std::min<size_t>(kWgMaxStages, room / stage);
+  if (a->stages < 4) return FR3D_ERR_UNSUPPORTED_SIZE;
+  int sms = 0;
+  FR3D_TRY(sm_count(&sms));
+  const int slots = (two ? 2 : 1) * sms;
+  const int len = a->q_last - a->q_first + 1, npairs = a->n_og * a->n_cg;
+  double bc = 0;
+  a->span = 0;
+  for (int span = kWgVox; span * a->nd <= std::max(kWgChain, kWgVox * a->nd) && span < len + kWgVox; span += kWgVox) {
+    const long units = (long)B * a->nchunks * ((len + span - 1) / span);
+    const long rounds = (units * npairs + slots - 1) / slots;
+    // MMA and copy time of a unit against the bytes of the partials (written and read once), in cycles
+    const double c = (double)rounds * ((span / kWgVox) * (a->nd + 2) * 12.0 * (32 + 3 * a->Cg / 4) + 3000) +
+                     (double)units * npairs * 3 * a->Og * wgrad_row_floats(a->Cg) * 8 / 2500.0;
+    if (!a->span || c < bc) {
+      a->span = span;
+      bc = c;
+    }
+  }
+  a->nspans = (len + a->span - 1) / a->span;
   return FR3D_OK;
 }
 
-int wgrad3_launch(const WgradArgs& a, cudaStream_t st) {
-  if (a.Cin % 16 || a.Cin > 256 || a.Cout % 8 || a.ndw * a.Cout > 128) return FR3D_ERR_UNSUPPORTED_SIZE;
-  const size_t stage = 16 * kWgPlane + (a.Cin / 8) * kWgPlane;
-  int occ = 0;
-  const int smem = launch_cfg(reinterpret_cast<const void*>(k_wgrad3), stage * kWgStages, (int)tmem_cols(a.Cin), &occ);
-  if (smem < 0) return smem;
-  const int ntg = a.ndw == 3 ? 9 : 27;
-  const long grid = (long)ntg * a.B * a.ranges_per_sample;
-  k_wgrad3<<<(unsigned)grid, 128, smem, st>>>(a);
+size_t wgrad_partial_floats(const WgradArgs& a, int B) {
+  return (size_t)B * a.nspans * a.nchunks * a.n_og * a.n_cg * 3 * a.Og * wgrad_row_floats(a.Cg);
+}
+
+int wgrad3_launch(const WgradArgs& a, int ci, float* dW, float* db, cudaStream_t st) {
+  const int stage = (3 * a.Og / 8 + 3 * a.Cg / 8 + 2) * kWgPlane;
+  const size_t smem = (size_t)a.stages * stage + 2 * kWgPlane;
+  FR3D_TRY(smem_optin(reinterpret_cast<const void*>(k_wgrad3), smem));
+  const int units = a.B * a.nspans * a.nchunks, npairs = a.n_og * a.n_cg;
+  k_wgrad3<<<units * npairs, kWgThreads, smem, st>>>(a);
+  const int total = npairs * 3 * a.Og * wgrad_row_floats(a.Cg);
+  k_wgrad_reduce<<<(total + kWgRedX - 1) / kWgRedX, dim3(kWgRedX, kWgRedY), 0, st>>>(a, units, ci, dW, db);
   FR3D_CUDA_TRY(cudaGetLastError());
   return FR3D_OK;
 }
-
-int wgrad_ranges_per_sample(long p_first, long p_last, long range) { return (int)((p_last - p_first + range) / range); }
 
 }  // namespace fr3d
