@@ -298,25 +298,39 @@ __global__ void __launch_bounds__(kMThreads) k_alpha_m_partial(
   }
 }
 
-// Sum of the partials (fixed order), r^2 = sum / n^2, and the discrepancy choice per band (one warp
-// per band: ballots of r^2 <= thr, the largest index wins).
+// Sum of the partials (fixed order: every thread adds each S-th block, S = threads / sums, then the S sums in
+// order), r^2 = sum / n^2, and the discrepancy choice per band (one warp per band: ballots of r^2 <= thr, the largest
+// index wins).  One block of 1024 threads, so that the loads of a sum are S chains: with one chain per sum the 519
+// blocks of 512^2 took 58 us.
+constexpr int kMFinish = 1024;
 struct MThr {
   double t[FR3D_MAX_BANDS];
 };
-__global__ void __launch_bounds__(256) k_alpha_m_finish(const double* __restrict__ partials, int nblk, int nb, int na,
+__global__ void __launch_bounds__(kMFinish) k_alpha_m_finish(const double* __restrict__ partials, int nblk, int nb, int na,
                                                         double inv_n2, MThr thr, int* __restrict__ aidx,
                                                         double* __restrict__ res_out, int* __restrict__ info,
                                                         int keep) {
   __shared__ double r2[FR3D_MAX_BANDS * FR3D_MAX_ALPHAS];
   __shared__ int flg[FR3D_MAX_BANDS];
+  __shared__ double red[kMFinish];
   const int tid = threadIdx.x, O = nb * na;
-  for (int o = tid; o < O; o += blockDim.x) {
+  const int S = max(1, kMFinish / O);
+  for (int o0 = 0; o0 < O; o0 += kMFinish) {   // one round unless there are more sums than threads
+    const int o = o0 + tid % min(O, kMFinish), sub = tid / min(O, kMFinish);
     double s = 0.0;
-    for (int blk = 0; blk < nblk; ++blk) s += partials[(long)blk * O + o];
-    r2[o] = s * inv_n2;
-    if (res_out) res_out[o] = s * inv_n2;
+    if (o < O && sub < S) {
+#pragma unroll 8
+      for (int blk = sub; blk < nblk; blk += S) s += __ldg(partials + (long)blk * O + o);
+    }
+    red[tid] = s;
+    __syncthreads();
+    if (o < O && sub == 0) {
+      for (int q = 1; q < S; ++q) s += red[q * O + tid];
+      r2[o] = s * inv_n2;
+      if (res_out) res_out[o] = s * inv_n2;
+    }
+    __syncthreads();
   }
-  __syncthreads();
   const int warp = tid >> 5, lane = tid & 31;
   for (int b = warp; b < nb; b += blockDim.x / 32) {
     int best = -1, ok = 0, flags = 0;
@@ -553,7 +567,7 @@ int multi_alpha(Handle* H, const MultiWs& w, const double* alphas, int na, int r
   k_alpha_m_partial<<<nblk, kMThreads, 0, st>>>(H->mlam, w.Pc, H->M, H->C, H->cband, nb, al, H->s2, na, ra, H->partials);
   MThr t;
   for (int b = 0; b < nb; ++b) t.t[b] = thr2[b];
-  k_alpha_m_finish<<<1, 256, 0, st>>>(H->partials, nblk, nb, na, 1.0 / ((double)H->n * H->n), t, aidx, residuals,
+  k_alpha_m_finish<<<1, kMFinish, 0, st>>>(H->partials, nblk, nb, na, 1.0 / ((double)H->n * H->n), t, aidx, residuals,
                                       info, keep);
   FR3D_CUDA_TRY(cudaGetLastError());
   prof_mark(H, kStAlpha, st);
