@@ -134,15 +134,27 @@ template <typename T> int weights_or_null(Handle* H, const fr3d_sources* s, cons
 }
 
 // ------------------------------------------------------------------ forward operator
+// Sources go through the row pass and the contraction in groups whose row-transformed spectra stay in L2
+// (kFwdBytes; 256^2 x 64: four sources of 17 MB), and through the inverse passes together.  One source per launch left
+// the small stages with 8-33 CTAs: 40 launches and 396 us for eight sources at 256^2 x 64, now 6 launches.
+constexpr size_t kFwdBytes = 72ull << 20;
+constexpr int kMaxGridY = 65535;
+
 template <typename T>
 int fwd_impl(Handle* H, const T* zeta, int Q, T* U, cudaStream_t st) {
   using C = typename Ops<T>::C;
-  const int n = H->n;
+  const int n = H->n, M = H->M, Mp = H->Mp;
   const long ps = (long)(n / 2 + 1) * n;
-  const size_t zb = align_up(sizeof(C) * ps * H->Mp), ub = align_up(sizeof(C) * ps * H->M);
-  FR3D_TRY(ensure_ws(H, zb + ub));
+  const size_t per = sizeof(C) * ps * Mp;
+  const int g = (int)std::max<size_t>(1, std::min<size_t>(std::min(Q, kMaxGridY / std::max(M, Mp)), kFwdBytes / per));
+  const int chunks = M == 1 ? Ops<T>::contract_chunks(H, g) : 0;
+  // sources per inverse pass: all of them, unless their partials or the launch grid say otherwise
+  const int gs = (int)std::max<size_t>(g, std::min<size_t>(std::min(Q, kMaxGridY / M), kFwdBytes / (sizeof(C) * ps * std::max(M, chunks))));
+  const size_t zb = align_up(per * g), pb = align_up(sizeof(C) * ps * gs * chunks), ub = align_up(sizeof(C) * ps * gs * M);
+  FR3D_TRY(ensure_ws(H, zb + pb + ub));
   C* Zh = reinterpret_cast<C*>(H->ws);
-  C* Uh = reinterpret_cast<C*>((char*)H->ws + zb);
+  C* part = reinterpret_cast<C*>((char*)H->ws + zb);
+  C* Uh = reinterpret_cast<C*>((char*)H->ws + zb + pb);
   const T* A;
   if constexpr (sizeof(T) == 4) A = H->A32;
   else {
@@ -150,13 +162,24 @@ int fwd_impl(Handle* H, const T* zeta, int Q, T* U, cudaStream_t st) {
     A = H->A64d;
   }
   int launches = 0;
-  for (int q = 0; q < Q; ++q) {
-    FR3D_TRY(Ops<T>::row_r2c(H, zeta + (long)q * H->Mp * n * n, (long)n * n, Zh, H->Mp, st));
-    FR3D_TRY(Ops<T>::col_plain(H, Zh, Zh, H->Mp, false, st));
-    FR3D_TRY(Ops<T>::contract_fwd(H, Zh, Uh, A, 1, st));
-    FR3D_TRY(Ops<T>::col_plain(H, Uh, Uh, H->M, true, st));
-    FR3D_TRY(Ops<T>::row_c2r_plain(H, Uh, U + (long)q * H->M * n * n, H->M, 1, 0, 0, st));
-    launches += 5;
+  for (int q0 = 0; q0 < Q; q0 += gs) {
+    const int ns = std::min(gs, Q - q0);
+    for (int q = 0; q < ns; q += g) {
+      const int nq = std::min(g, ns - q);
+      FR3D_TRY(Ops<T>::row_r2c(H, zeta + (long)(q0 + q) * Mp * n * n, (long)n * n, Zh, nq * Mp, st));
+      if (M == 1) {
+        FR3D_TRY(Ops<T>::col_contract(H, Zh, part + q * ps, ps * ns, A, nq, chunks, st));
+        launches += 2;
+      } else {
+        FR3D_TRY(Ops<T>::col_plain(H, Zh, Zh, nq * Mp, false, st));
+        FR3D_TRY(Ops<T>::contract_fwd(H, Zh, Uh + (long)q * M * ps, A, nq, st));
+        launches += 3;
+      }
+    }
+    if (M == 1) FR3D_TRY(Ops<T>::col_sum(H, part, ps * ns, Uh, ns, chunks, st));
+    else FR3D_TRY(Ops<T>::col_plain(H, Uh, Uh, ns * M, true, st));
+    FR3D_TRY(Ops<T>::row_c2r_plain(H, Uh, U + (long)q0 * M * n * n, ns * M, 1, 0, 1, st));
+    launches += 2;
   }
   H->last_launches = launches;
   return FR3D_OK;

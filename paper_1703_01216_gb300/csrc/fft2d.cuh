@@ -81,39 +81,33 @@ struct TablePlanes {
   __device__ float2* dst(int p) const { return t[p].out; }
 };
 
-// in: planes of n x n reals; out: [plane][kx][y] complex.  One CTA transforms TY rows of a plane.
+// in: planes of n x n reals; out: [plane][kx][y] complex.  One CTA transforms TY rows of a plane: the first
+// radix pass is fed from global memory, and the split writes straight to the output (TY consecutive y per kx,
+// a segment of 8 TY bytes).  Bound by latency at few planes and by the memory traffic (4 B in, 4 B out per point)
+// at many: without the two staging trips through shared memory a CTA's 256^2 rows take 38 KB instead of 70 KB.
 template <typename T, int N, int TY, class PM>
 __global__ void __launch_bounds__(kThreads) k_row_r2c(PM pm, const typename cpx<T>::t* __restrict__ tw_full) {
   using C = typename cpx<T>::t;
-  constexpr int L = N / 2, SS = Smem<C, L>::ss, STS = TY + 1;
+  constexpr int L = N / 2, SS = Smem<C, L>::ss;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* tws = reinterpret_cast<C*>(smem_raw);       // exp(-2 pi i t / n), t < n
-  C* ptw = tws + N;                              // pass tables of the length-n/2 transform
+  C* tws = reinterpret_cast<C*>(smem_raw);       // exp(-2 pi i t / n), t <= n / 2
+  C* ptw = tws + L + 1;                          // pass tables of the length-n/2 transform
   C* buf = ptw + passtw_size<L>();
-  C* stg = buf + TY * SS;
   const int tid = threadIdx.x, plane = blockIdx.y, y0 = blockIdx.x * TY;
   const C* src = reinterpret_cast<const C*>(pm.src(plane) + (long)y0 * N);
-  for (int e = tid; e < N; e += kThreads) tws[e] = __ldg(tw_full + e);
+  for (int e = tid; e <= L; e += kThreads) tws[e] = __ldg(tw_full + e);
   build_passtw<L, 2, kThreads>(ptw, tw_full, tid);
-  batched_copy<TY * L, kThreads, 8>(
-      tid, [&](int e) { return __ldg(src + e); },
-      [&](int e, C v) { buf[(e / L) * SS + pidx<C>(e % L)] = v; });
-  __syncthreads();
-  fft_smem<L, false, TY, kThreads>(buf, SS, ptw, tid);
+  first_pass_from<L, false, TY, kThreads>(buf, SS, [&](int r, int t) { return __ldg(src + r * L + t); }, tid);
+  fft_passes<L, false, TY, kThreads, 1, Plan<L>::np, Plan<L>::radix(0)>(buf, SS, ptw, tid);
   const T half = (T)0.5;
+  C* dst = pm.dst(plane) + y0;
   for (int e = tid; e < TY * (L + 1); e += kThreads) {
     const int k = e / TY, r = e - k * TY;
     const C zk = buf[r * SS + pidx<C>(k == L ? 0 : k)];
     const C zc = cconj(buf[r * SS + pidx<C>(k == 0 ? 0 : L - k)]);
     const C E = cscale(cadd(zk, zc), half);
     const C O = cmul_mi<false>(cscale(csub(zk, zc), half));  // (Z[k] - conj Z[L-k]) / (2i)
-    stg[k * STS + r] = cadd(E, cmul(tws[k], O));  // X[k] = E[k] + w^k O[k]
-  }
-  __syncthreads();
-  C* dst = pm.dst(plane) + y0;
-  for (int e = tid; e < TY * (L + 1); e += kThreads) {
-    const int k = e / TY, r = e - k * TY;
-    dst[(long)k * N + r] = stg[k * STS + r];
+    dst[(long)k * N + r] = cadd(E, cmul(tws[k], O));  // X[k] = E[k] + w^k O[k]
   }
 }
 
@@ -170,6 +164,102 @@ struct ColTable {
   __device__ float2* dst(int p) const { return t[p].out; }
   __device__ float2 load(int, int, int, float2 v) const { return v; }
 };
+
+constexpr int kMaxChunks = 8;   // depth chunks of the forward contraction at most
+// inverse column pass over the sum of S <= kMaxChunks partial spectra, p and p + stride, ..., scaled by `scale`
+template <typename T> struct ColSum {
+  using C = typename cpx<T>::t;
+  const C* in;        // [S][planes][H1][n]
+  C* out;             // [planes][H1][n]
+  long ps, stride;
+  int S, n;
+  T scale;
+  __device__ void begin(int) {}
+  __device__ const C* src(int p) const { return in + p * ps; }
+  __device__ C* dst(int p) const { return out + p * ps; }
+  __device__ C load(int p, int kx, int ky, C v) const {
+    const C* q = in + p * ps + (long)kx * n + ky;
+    C u[kMaxChunks - 1];   // every partial requested before the first is added
+#pragma unroll
+    for (int s = 1; s < kMaxChunks; ++s) u[s - 1] = s < S ? __ldg(q + s * stride) : cmk((T)0, (T)0);
+#pragma unroll
+    for (int s = 1; s < kMaxChunks; ++s) v = cadd(v, u[s - 1]);
+    return cscale(v, scale);
+  }
+};
+
+// ---------------------------------------------------------------- forward column pass + contraction (M = 1)
+// Partial sums over a chunk of depths of A_j(k) zeta~_j(k) (Eq. (5)-(6) with one observation depth): a CTA
+// transforms TC columns of every depth's plane in turn and keeps the weighted sum of their outputs in registers,
+// so the transformed columns are never written.  Z: [q][M'][H1][n] row-transformed spectra; out: [q][H1][n], the
+// chunks out_cs apart.
+// Grid: column tiles x q x depth chunks.  One radix-16 butterfly per thread at n = 256 (kContractThreads).
+constexpr int kContractThreads = 128;
+template <typename T, int N> struct ContractTile {
+  static constexpr int v0 = (sizeof(T) == 4 ? 2048 : 1024) / N;
+  static constexpr int v1 = v0 < 1 ? 1 : v0;
+  static constexpr int v = v1 > N / 2 + 1 ? N / 2 + 1 : v1;
+};
+template <typename T, int N, int TC>
+__global__ void __launch_bounds__(kContractThreads) k_col_contract(const typename cpx<T>::t* __restrict__ Z,
+                                                                   typename cpx<T>::t* __restrict__ out,
+                                                                   const T* __restrict__ A, int Mp, int chunk, long out_cs,
+                                                                   const typename cpx<T>::t* __restrict__ tw) {
+  using C = typename cpx<T>::t;
+  using LP = LastPass<N>;
+  constexpr int NT = kContractThreads, SS = Smem<C, N>::ss, H1 = N / 2 + 1, NP = Plan<N>::np;
+  constexpr int R = LP::R, BPS = LP::BPS, NB = TC * BPS, K = (NB + NT - 1) / NT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* ptw = reinterpret_cast<C*>(smem_raw);
+  C* buf = ptw + passtw_size<N>();
+  const int tid = threadIdx.x, c0 = blockIdx.x * TC, q = blockIdx.y;
+  const long ps = (long)H1 * N;
+  const int j0 = blockIdx.z * chunk, j1 = min(j0 + chunk, Mp);
+  build_passtw<N, 1, NT>(ptw, tw, tid);
+  C acc[K][R];
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[k][r] = cmk((T)0, (T)0);
+  for (int j = j0; j < j1; ++j) {
+    const C* src = Z + ((long)q * Mp + j) * ps + (long)c0 * N;
+    const T* a = A + (long)j * ps + (long)c0 * N;
+    T w[K][R];   // requested before the transform
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int b = tid + k * NT, s = b / BPS, t = b - s * BPS;
+#pragma unroll
+      for (int r = 0; r < R; ++r) w[k][r] = (b < NB && c0 + s < H1) ? __ldg(a + s * N + t + r * LP::NS) : (T)0;
+    }
+    first_pass_from<N, false, TC, NT>(
+        buf, SS, [&](int s, int t) { return c0 + s < H1 ? __ldg(src + s * N + t) : cmk((T)0, (T)0); }, tid);
+    fft_passes<N, false, TC, NT, 1, NP - 1, Plan<N>::radix(0)>(buf, SS, ptw, tid);
+    auto add = [&](int, int, C v, int k, int r) {
+      acc[k][r].x = fma_p(w[k][r], v.x, acc[k][r].x);
+      acc[k][r].y = fma_p(w[k][r], v.y, acc[k][r].y);
+    };
+    if constexpr (NP > 1) {
+      last_pass_to<N, false, TC, NT>(buf, SS, ptw, add, tid);
+    } else {   // a single pass: its outputs are in the buffer already
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const int b = tid + k * NT;
+        if (b < NB)
+#pragma unroll
+          for (int r = 0; r < R; ++r) add(b, r, buf[b * SS + pidx<C>(r)], k, r);
+      }
+    }
+    __syncthreads();   // the next depth's first pass overwrites the buffer
+  }
+  C* dst = out + blockIdx.z * out_cs + q * ps + (long)c0 * N;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int b = tid + k * NT, s = b / BPS, t = b - s * BPS;
+    if (b < NB && c0 + s < H1)
+#pragma unroll
+      for (int r = 0; r < R; ++r) dst[s * N + t + r * LP::NS] = acc[k][r];
+  }
+}
 
 // Solve for M = 1 fused into the inverse column pass (Eq. (6) with a single observation depth):
 // zeta~_j(k) = A_j(k) U~_q(k) / (n^2 (||A(k)||^2 + alpha s^2)).  Output plane p = jc Q + q holds
@@ -264,14 +354,14 @@ struct RowGeom {
 // MODE 1 is bound by the point sources' reciprocal square roots, above all in FP64 (256^2 x 64, Q = 8, five
 // points: 9.5 of the call's 10.5 ms); MODE 2 reads one value per voxel and source instead: the FP64 call
 // takes 2.87 ms, the FP32 one at 512^2 x 51 depths, ten points, 0.556 ms (before 0.625).
-template <typename T, int N, int MODE>
+template <typename T, int N, int MODE, int TY>
 __global__ void __launch_bounds__(kThreads) k_row_c2r(const typename cpx<T>::t* __restrict__ in, T* __restrict__ out,
                                                      int Q, int j0, int out_stride,
                                                      typename SrcOf<T>::t src, RowGeom g, const T* __restrict__ zr,
                                                      const T* __restrict__ W, long w_qs,
                                                      const typename cpx<T>::t* __restrict__ tw_full) {
   using C = typename cpx<T>::t;
-  constexpr int L = N / 2, TY = row_c2r_tile<T, N, MODE>();
+  constexpr int L = N / 2;
   constexpr int SS = Smem<C, L>::ss;
   constexpr int EPT = (TY * L + kThreads - 1) / kThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -380,7 +470,7 @@ __global__ void __launch_bounds__(kThreads) k_row_c2r(const typename cpx<T>::t* 
 template <typename T, int N, int TY> constexpr size_t row_r2c_smem() {
   using C = typename cpx<T>::t;
   constexpr int L = N / 2;
-  return sizeof(C) * ((size_t)N + passtw_size<L>() + (size_t)TY * Smem<C, L>::ss + (size_t)(L + 1) * (TY + 1));
+  return sizeof(C) * ((size_t)(L + 1) + passtw_size<L>() + (size_t)TY * Smem<C, L>::ss);
 }
 template <typename T, int N, int TC> constexpr size_t col_smem() {
   using C = typename cpx<T>::t;
@@ -391,9 +481,9 @@ template <int N> struct SmallTile {
   static constexpr int row = divisor_at_most(N, 8);
   static constexpr int col = 4;
 };
-template <typename T, int N, int MODE> constexpr size_t row_c2r_smem() {
+template <typename T, int N, int TY> constexpr size_t row_c2r_smem() {
   using C = typename cpx<T>::t;
-  return sizeof(C) * ((size_t)N + passtw_size<N / 2>() + (size_t)row_c2r_tile<T, N, MODE>() * Smem<C, N / 2>::ss);
+  return sizeof(C) * ((size_t)N + passtw_size<N / 2>() + (size_t)TY * Smem<C, N / 2>::ss);
 }
 
 }  // namespace fr3d

@@ -33,6 +33,12 @@ template <typename T> struct Ops {
                         cudaStream_t st);
   // U~[q][i] = (1/n^2) sum_j A[i][j] zeta~[q][j] for every half-spectrum bin
   static int contract_fwd(const Handle* H, const C* Zh, C* Uh, const T* A, int Q, cudaStream_t st);
+  // M = 1: the same from the row-transformed planes of Q sources, as partial sums of `chunks` depth chunks (part:
+  // chunks part_cs apart, [Q][n/2+1][n] each), and their sum with the inverse column pass, ready for the row pass
+  static int contract_chunks(const Handle* H, int Q);
+  static int col_contract(const Handle* H, const C* Zh, C* part, long part_cs, const T* A, int Q, int chunks,
+                          cudaStream_t st);
+  static int col_sum(const Handle* H, const C* part, long part_cs, C* Uh, int Q, int chunks, cudaStream_t st);
   // zeta[q][j] = xi[j] * V0_q
   static int zeta_from_xi(const Handle* H, const T* xi, T* zeta, int Q, const SrcHost& src, cudaStream_t st);
   // discrepancy choice over the cached alpha tables (M = 1), per band (nb = 1: whole spectrum);

@@ -61,11 +61,11 @@ static int col_n(const Handle* H, const Op& op, int nplanes, cudaStream_t st) {
   return col_t<T, N, INV, Op, TC>(H, op, nplanes, st);
 }
 
-template <typename T, int N, int MODE>
-static int row_c2r_n(const Handle* H, const typename cpx<T>::t* in, T* out, int nplanes, int Q, int j0,
+template <typename T, int N, int MODE, int TY>
+static int row_c2r_t(const Handle* H, const typename cpx<T>::t* in, T* out, int nplanes, int Q, int j0,
                      int out_stride, const SrcHost& src, const T* W, cudaStream_t st) {
-  constexpr size_t sm = row_c2r_smem<T, N, MODE>();
-  auto kern = k_row_c2r<T, N, MODE>;
+  constexpr size_t sm = row_c2r_smem<T, N, TY>();
+  auto kern = k_row_c2r<T, N, MODE, TY>;
   FR3D_TRY(set_smem(kern, sm));
   typename SrcOf<T>::t s;
   s.pts = reinterpret_cast<decltype(s.pts)>(src.pts);
@@ -75,9 +75,21 @@ static int row_c2r_n(const Handle* H, const typename cpx<T>::t* in, T* out, int 
   const T* zr;
   if constexpr (sizeof(T) == 4) zr = H->zr32;
   else zr = H->zr64;
-  dim3 grid(N / row_c2r_tile<T, N, MODE>(), nplanes);
+  dim3 grid(N / TY, nplanes);
   kern<<<grid, kThreads, sm, st>>>(in, out, Q, j0, out_stride, s, g, zr, W, (long)H->Mp * N * N, tw_of<T>(H, N));
   return cudaGetLastError() == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
+}
+
+template <typename T, int N, int MODE>
+static int row_c2r_n(const Handle* H, const typename cpx<T>::t* in, T* out, int nplanes, int Q, int j0,
+                     int out_stride, const SrcHost& src, const T* W, cudaStream_t st) {
+  constexpr int TY = row_c2r_tile<T, N, MODE>();
+  // few planes: small tiles put more CTAs in flight (the forward operator's eight planes of 256^2: 64 CTAs of 32
+  // rows take 12.6 us, 256 of 8 rows 5)
+  if constexpr (MODE == 0 && SmallTile<N>::row < TY)
+    if ((long)nplanes * (N / TY) < kSmallGrid)
+      return row_c2r_t<T, N, MODE, SmallTile<N>::row>(H, in, out, nplanes, Q, j0, out_stride, src, W, st);
+  return row_c2r_t<T, N, MODE, TY>(H, in, out, nplanes, Q, j0, out_stride, src, W, st);
 }
 
 template <typename T>
@@ -189,6 +201,54 @@ int Ops<T>::contract_fwd(const Handle* H, const C* Zh, C* Uh, const T* A, int Q,
   const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 16);
   k_contract_fwd<T, C><<<blocks, 256, 0, st>>>(Zh, Uh, A, Q, H->M, H->Mp, ps, (T)(1.0 / ((double)H->n * H->n)));
   return cudaGetLastError() == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
+}
+
+template <typename T, int N>
+static int col_contract_n(const Handle* H, const typename cpx<T>::t* Zh, typename cpx<T>::t* part, long part_cs,
+                          const T* A, int Q, int chunks, cudaStream_t st) {
+  constexpr int TC = ContractTile<T, N>::v;
+  constexpr size_t sm = col_smem<T, N, TC>();
+  auto kern = k_col_contract<T, N, TC>;
+  FR3D_TRY(set_smem(kern, sm));
+  const dim3 grid((N / 2 + TC) / TC, Q, chunks);
+  kern<<<grid, kContractThreads, sm, st>>>(Zh, part, A, H->Mp, (H->Mp + chunks - 1) / chunks, part_cs, tw_of<T>(H, N));
+  return cudaGetLastError() == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
+}
+
+// Depth chunks of the contraction: enough CTAs to fill the SMs (five each at n = 256), at least four depths each, no
+// empty chunk; more partials than kMaxChunks cost the sum more than the extra CTAs give (16 chunks: 17 us).
+template <typename T>
+int Ops<T>::contract_chunks(const Handle* H, int Q) {
+  int tc = (sizeof(T) == 4 ? 2048 : 1024) / H->n;
+  tc = std::max(1, std::min(tc, H->n / 2 + 1));
+  const int ctas = ((H->n / 2 + tc) / tc) * Q;
+  const int want = std::max(1, std::min({(5 * 152 + ctas - 1) / ctas, H->Mp / 4, kMaxChunks}));
+  const int per = (H->Mp + want - 1) / want;
+  return (H->Mp + per - 1) / per;
+}
+
+template <typename T>
+int Ops<T>::col_contract(const Handle* H, const C* Zh, C* part, long part_cs, const T* A, int Q, int chunks,
+                         cudaStream_t st) {
+  switch (H->n) {
+#define X(N) \
+  case N: return col_contract_n<T, N>(H, Zh, part, part_cs, A, Q, chunks, st);
+    FR3D_FOR_EACH_N(X)
+#undef X
+  }
+  return FR3D_ERR_UNSUPPORTED_SIZE;
+}
+
+template <typename T>
+int Ops<T>::col_sum(const Handle* H, const C* part, long part_cs, C* Uh, int Q, int chunks, cudaStream_t st) {
+  const ColSum<T> op{part, Uh, (long)(H->n / 2 + 1) * H->n, part_cs, chunks, H->n, (T)(1.0 / ((double)H->n * H->n))};
+  switch (H->n) {
+#define X(N) \
+  case N: return col_n<T, N, true>(H, op, Q, st);
+    FR3D_FOR_EACH_N(X)
+#undef X
+  }
+  return FR3D_ERR_UNSUPPORTED_SIZE;
 }
 
 // ---------------------------------------------------------------- zeta = xi V0 (Sec. 2)
