@@ -68,9 +68,9 @@ struct Group {
   int nplanes = 0, nclusters = 0;
   int var = -1;   // inverse variant (-1: not chosen yet; 5: the tile queue)
   size_t off_planes = 0, off_fused = 0, off_map = 0;
-  // the tile queue over the group's instances (n = 256, xi output, plan form): its descriptor table in
+  // the tile queue over the group's instances (a supported size, xi output, plan form): its descriptor table in
   // the plan's tables, its counters and intermediates in the plan's queue buffer
-  int qn = 0, qtotal = 0, qncnt = 0;
+  int qn = 0, qdepths = 0;
   size_t off_queue = 0;
   int* qctl = nullptr;
   int* qcnt = nullptr;
@@ -239,25 +239,25 @@ void build_descriptors(const fr3d_instance* inst, const std::map<int, std::vecto
     g.nclusters = (int)map.size();
     if (qbuf && queue_group(g.n, inst[kv.second[0]].opts->output)) {
       // [4 launch counters][2 M' depth counters per instance][intermediates, 256-byte aligned]
-      int ncnt = 0;
-      for (int idx : kv.second) ncnt += 2 * inst[idx].handle->h.Mp;
+      int depths = 0;
+      for (int idx : kv.second) depths += inst[idx].handle->h.Mp;
       g.qctl = reinterpret_cast<int*>(qbuf);
       g.qcnt = g.qctl + 4;
-      unsigned char* tp = qbuf + al(sizeof(int) * (4 + (size_t)ncnt));
+      unsigned char* tp = qbuf + al(sizeof(int) * (4 + 2 * (size_t)depths));
       std::vector<unsigned char> qt(inv_queue_inst_bytes() * kv.second.size());
-      int tick = 0, c = 0, k = 0;
+      int d = 0, k = 0;
       for (int idx : kv.second) {
         const fr3d_instance& I = inst[idx];
         const int mp = I.handle->h.Mp;
-        tick += inv_queue_make_inst(qt.data() + k * inv_queue_inst_bytes(), fa[k], reinterpret_cast<float2*>(tp),
-                                    g.qcnt + c, mp, tick);
+        inv_queue_make_inst(qt.data() + k * inv_queue_inst_bytes(), fa[k], reinterpret_cast<float2*>(tp),
+                            g.qcnt + 2 * d, mp, d);
         tp += al(inv2_scratch_bytes(g.n, I.Q, mp));
-        c += 2 * mp;
+        d += mp;
         ++k;
       }
+      qbuf = tp;   // the next group's part
       g.qn = k;
-      g.qtotal = tick;
-      g.qncnt = ncnt;
+      g.qdepths = depths;
       g.off_queue = put(qt.data(), qt.size());
     }
     g.off_planes = put(planes.data(), planes.size() * sizeof(PlanePtr));
@@ -269,7 +269,7 @@ void build_descriptors(const fr3d_instance* inst, const std::map<int, std::vecto
   ap.off = alph.empty() ? 0 : put(alph.data(), alph.size() * sizeof(AlphaInst));
 }
 
-// bytes of the plan's queue buffer (the tile queue of its n = 256 group, xi output), 0 if none
+// bytes of the plan's queue buffer (the tile queues of its groups of a supported size, xi output), 0 if none
 size_t queue_bytes(const fr3d_instance* inst, const std::map<int, std::vector<int>>& by_n) {
   size_t b = 0;
   for (auto& kv : by_n) {
@@ -285,7 +285,7 @@ size_t queue_bytes(const fr3d_instance* inst, const std::map<int, std::vector<in
 // the inverse of a group: the tile queue (variant 5, where the plan has one) or a fused tile variant
 int run_inverse(const Group& g, const unsigned char* dev, int output, int v, cudaStream_t st) {
   if (v == 5 && g.qn > 0)
-    return inv_queue_launch_table(dev + g.off_queue, g.qn, g.qctl, g.qcnt, g.qncnt, g.qtotal, st);
+    return inv_queue_launch_table(g.n, dev + g.off_queue, g.qn, g.qctl, g.qcnt, g.qdepths, st);
   return inv_fused_batched_f32(g.n, fused_of(g, dev), map_of(g, dev), g.nclusters, output, std::min(v, 3), st);
 }
 
@@ -312,9 +312,15 @@ extern "C" int fr3d_batch_create(const fr3d_instance* inst, int n, fr3d_batch** 
   b.output = inst[0].opts->output;
   const size_t qb = queue_bytes(inst, by_n);
   if (qb > 0) {
-    FR3D_CUDA_TRY(cudaMalloc(&b.qbuf, qb));
-    cudaError_t e = cudaMemsetAsync(b.qbuf, 0, qb, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaError_t e = cudaMalloc(&b.qbuf, qb);
+    if (e == cudaErrorMemoryAllocation) {   // no room for the intermediates: the plan runs the fused tiles
+      cudaGetLastError();
+      b.qbuf = nullptr;
+      e = cudaSuccess;
+    } else if (e == cudaSuccess) {
+      e = cudaMemsetAsync(b.qbuf, 0, qb, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    }
     if (e != cudaSuccess) {
       cudaFree(b.qbuf);
       return FR3D_ERR_CUDA;

@@ -1,4 +1,4 @@
-// Batched mixed-radix (2, 3, 4, 8, 16) complex FFTs on shared memory.
+// Batched mixed-radix (2, 3, 4, 6, 8, 12, 16) complex FFTs on shared memory.
 //
 // Every 2D transform of Algorithm 1 (steps 1 and 3) is built from one
 // primitive: a CTA transforms NSEQ sequences of compile-time length L held in
@@ -158,7 +158,39 @@ template <bool INV> struct Dft<16, INV> {
   template <typename C> static __device__ __forceinline__ void run(C* v) { DftDif<16, INV>::run(v); }
 };
 
-// Radix schedule per transform length (product of the radices = L, applied first to last).
+// 6 = 2 x 3 and 12 = 3 x 4 points by the prime-factor map (no twiddles): input n = N2 n1 + N1 n2, output
+// k = N2 (N2^-1 mod N1) k1 + N1 (N1^-1 mod N2) k2, both mod N1 N2
+template <int N1, int N2, int E1, int E2, bool INV> struct DftPfa {
+  template <typename C> static __device__ __forceinline__ void run(C* v) {
+    constexpr int N = N1 * N2;
+    C u[N2][N1];
+#pragma unroll
+    for (int b = 0; b < N2; ++b) {
+#pragma unroll
+      for (int a = 0; a < N1; ++a) u[b][a] = v[(N2 * a + N1 * b) % N];
+      Dft<N1, INV>::run(u[b]);
+    }
+#pragma unroll
+    for (int a = 0; a < N1; ++a) {
+      C w[N2];
+#pragma unroll
+      for (int b = 0; b < N2; ++b) w[b] = u[b][a];
+      Dft<N2, INV>::run(w);
+#pragma unroll
+      for (int b = 0; b < N2; ++b) v[(E1 * a + E2 * b) % N] = w[b];
+    }
+  }
+};
+template <bool INV> struct Dft<6, INV> {
+  template <typename C> static __device__ __forceinline__ void run(C* v) { DftPfa<2, 3, 3, 4, INV>::run(v); }
+};
+template <bool INV> struct Dft<12, INV> {
+  template <typename C> static __device__ __forceinline__ void run(C* v) { DftPfa<3, 4, 4, 9, INV>::run(v); }
+};
+
+// Radix schedule per transform length (product of the radices = L, applied first to last).  Two passes up to 256: with
+// 16 x 4 x 3 and 8 x 4 x 3 for 192 and 96 the fused inverse spilled up to 0.9 KB per thread and took 137 us for 64
+// depths and 8 sources at n = 192, now 120 us.
 template <int L> struct Plan;
 #define FR3D_PLAN(L_, NP_, R0_, R1_, R2_)                                        \
   template <> struct Plan<L_> {                                                \
@@ -170,11 +202,11 @@ FR3D_PLAN(12, 2, 4, 3, 1)
 FR3D_PLAN(16, 1, 16, 1, 1)
 FR3D_PLAN(24, 2, 8, 3, 1)
 FR3D_PLAN(32, 2, 8, 4, 1)
-FR3D_PLAN(48, 2, 16, 3, 1)
+FR3D_PLAN(48, 2, 6, 8, 1)
 FR3D_PLAN(64, 2, 8, 8, 1)
-FR3D_PLAN(96, 3, 8, 4, 3)
+FR3D_PLAN(96, 2, 12, 8, 1)
 FR3D_PLAN(128, 2, 16, 8, 1)
-FR3D_PLAN(192, 3, 16, 4, 3)
+FR3D_PLAN(192, 2, 16, 12, 1)
 FR3D_PLAN(256, 2, 16, 16, 1)
 FR3D_PLAN(384, 3, 16, 8, 3)
 FR3D_PLAN(512, 3, 8, 8, 8)

@@ -49,9 +49,9 @@ template <int N> struct FusedCfg;
 template <> struct FusedCfg<16> : FusedCfgBase { static constexpr int CL = 1, NT = 128, RB = 16, MINB = 4; };
 template <> struct FusedCfg<24> : FusedCfgBase { static constexpr int CL = 1, NT = 96, RB = 24, MINB = 4; };
 template <> struct FusedCfg<32> : FusedCfgBase { static constexpr int CL = 1, NT = 128, RB = 32, MINB = 4; };
-template <> struct FusedCfg<48> : FusedCfgBase { static constexpr int CL = 1, NT = 128, RB = 48, MINB = 3; };
+template <> struct FusedCfg<48> : FusedCfgBase { static constexpr int CL = 1, NT = 128, RB = 48, MINB = 2; };
 template <> struct FusedCfg<64> : FusedCfgBase { static constexpr int CL = 2, NT = 256, RB = 32, MINB = 2; };
-template <> struct FusedCfg<96> : FusedCfgBase { static constexpr int CL = 2, NT = 256, RB = 48, MINB = 2; };
+template <> struct FusedCfg<96> : FusedCfgBase { static constexpr int CL = 2, NT = 256, RB = 48, MINB = 1; };
 template <> struct FusedCfg<128> : FusedCfgBase { static constexpr int CL = 4, NT = 256, RB = 32, MINB = 2; };
 template <> struct FusedCfg<192> : FusedCfgBase { static constexpr int CL = 8, NT = 256, RB = 8, MINB = 2; };
 template <> struct FusedCfg<256> : FusedCfgBase { static constexpr int CL = 8, NT = 256, RB = 16, MINB = 2; };

@@ -19,19 +19,21 @@ namespace fr3d {
 
 namespace {
 
-constexpr int kColThreads = 256;
 constexpr int kRowThreads = 128;
-constexpr int kRB = 8;   // rows per block of pass 2
 
 template <int N> struct Inv2Geom {
   static constexpr int L = N / 2;
   static constexpr int CA = L <= 16 ? L : (L % 16 == 0 ? 16 : 12);   // columns per block of pass 1
+  // n = 96 transforms its columns in 8 + 12 and its rows in 8 + 6 butterflies: 128 threads and 16 rows per block keep
+  // them busy (with 256 threads and 8 rows, 64 depths and 8 sources took 39.7 us)
+  static constexpr int CTH = N == 96 ? 128 : 256;   // threads of pass 1
+  static constexpr int RB = N == 96 ? 16 : 8;       // rows per block of pass 2
   static constexpr int SSC = PaddedLen<N, float2>::v + 1;            // odd: transposed reads free of conflicts
   static constexpr int SSR = PaddedLen<L, float2>::v;
   static constexpr int PTC = passtw_size<N>() > 0 ? passtw_size<N>() : 1;
   static constexpr int PTR = passtw_size<L>() > 0 ? passtw_size<L>() : 1;
   static constexpr size_t smem_col = sizeof(float2) * ((size_t)CA * SSC + PTC);
-  static constexpr size_t smem_row = sizeof(float2) * ((size_t)kRB * SSR + N + PTR);
+  static constexpr size_t smem_row = sizeof(float2) * ((size_t)RB * SSR + N + PTR);
 };
 
 struct Inv2Args {
@@ -50,7 +52,7 @@ struct Inv2Args {
 };
 
 template <int N>
-__global__ void __launch_bounds__(kColThreads) k_inv2_col(Inv2Args a) {
+__global__ void __launch_bounds__(Inv2Geom<N>::CTH) k_inv2_col(Inv2Args a) {
   using G = Inv2Geom<N>;
   constexpr int L = G::L, CA = G::CA, SSC = G::SSC;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -62,7 +64,7 @@ __global__ void __launch_bounds__(kColThreads) k_inv2_col(Inv2Args a) {
   const int q = plane / a.nj, jl = plane - q * a.nj, j = a.j0 + jl;
   const int c0 = blockIdx.y * CA;
   const long ps = (long)(L + 1) * N;
-  build_passtw<N, 1, kColThreads>(ptc, a.tw_n, tid);
+  build_passtw<N, 1, G::CTH>(ptc, a.tw_n, tid);
   pdl_wait();
   if (tid < a.nb) s_aidx[tid] = min(max(a.aidx[tid], 0), a.na - 1);
   __syncthreads();
@@ -86,12 +88,12 @@ __global__ void __launch_bounds__(kColThreads) k_inv2_col(Inv2Args a) {
     }
     return v;
   };
-  first_pass_from<N, true, CA, kColThreads>(colbuf, SSC, ldc, tid);
-  fft_passes<N, true, CA, kColThreads, 1, Plan<N>::np, Plan<N>::radix(0)>(colbuf, SSC, ptc, tid);
+  first_pass_from<N, true, CA, G::CTH>(colbuf, SSC, ldc, tid);
+  fft_passes<N, true, CA, G::CTH, 1, Plan<N>::np, Plan<N>::radix(0)>(colbuf, SSC, ptc, tid);
   // rows of T: CA consecutive columns per row y (coalesced writes; the odd stride keeps the reads of
   // consecutive columns in distinct banks)
   float2* Tp = a.T + (long)plane * N * L;
-  for (int e = tid; e < CA * N; e += kColThreads) {
+  for (int e = tid; e < CA * N; e += G::CTH) {
     const int y = e / CA, s = e - y * CA;
     Tp[(long)y * L + c0 + s] = colbuf[s * SSC + pidx<float2>(y)];
   }
@@ -100,7 +102,7 @@ __global__ void __launch_bounds__(kColThreads) k_inv2_col(Inv2Args a) {
 template <int N, int MODE>
 __global__ void __launch_bounds__(kRowThreads) k_inv2_row(Inv2Args a) {
   using G = Inv2Geom<N>;
-  constexpr int L = G::L, SSR = G::SSR;
+  constexpr int L = G::L, SSR = G::SSR, kRB = G::RB;
   using LP = LastPass<L>;
   constexpr int NBF = kRB * LP::BPS;                       // butterflies of the last pass
   constexpr int KR = (NBF + kRowThreads - 1) / kRowThreads;
@@ -210,10 +212,10 @@ int inv2_launch_n(const Inv2Args& a, bool xi, cudaStream_t st) {
   FR3D_TRY(smem_optin(reinterpret_cast<const void*>(k_inv2_col<N>), G::smem_col));
   const void* rk = xi ? reinterpret_cast<const void*>(k_inv2_row<N, 1>) : reinterpret_cast<const void*>(k_inv2_row<N, 0>);
   FR3D_TRY(smem_optin(rk, G::smem_row));
-  k_inv2_col<N><<<dim3(a.Q * a.nj, G::L / G::CA), kColThreads, G::smem_col, st>>>(a);
+  k_inv2_col<N><<<dim3(a.Q * a.nj, G::L / G::CA), G::CTH, G::smem_col, st>>>(a);
   FR3D_CUDA_TRY(cudaGetLastError());
-  if (xi) k_inv2_row<N, 1><<<dim3(a.nj, N / kRB), kRowThreads, G::smem_row, st>>>(a);
-  else k_inv2_row<N, 0><<<dim3(a.nj, N / kRB), kRowThreads, G::smem_row, st>>>(a);
+  if (xi) k_inv2_row<N, 1><<<dim3(a.nj, N / G::RB), kRowThreads, G::smem_row, st>>>(a);
+  else k_inv2_row<N, 0><<<dim3(a.nj, N / G::RB), kRowThreads, G::smem_row, st>>>(a);
   FR3D_CUDA_TRY(cudaGetLastError());
   return FR3D_OK;
 }

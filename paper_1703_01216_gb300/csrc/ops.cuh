@@ -59,19 +59,19 @@ int inv_fused_f32(const Handle* H, const float2* Uh, const float* Dd, const int*
 struct FusedArgs;
 size_t inv2_scratch_bytes(int n, int Q, int nj);
 int inv2_launch(int n, bool xi, const FusedArgs& f, int nj, float2* T, cudaStream_t st);
-// The persistent tile-queue inverse (inv_queue.cu): n = 256, xi output, U~ input (no solved spectra).
-// T: the two-pass intermediate (inv2_scratch_bytes); ctl: inv_queue_ctl_ints(nj, Q) ints, zeroed once at
+// The persistent tile-queue inverse (inv_queue.cu): n = 96, 128, 192, 256, xi output, U~ input (no solved
+// spectra).  T: the two-pass intermediate (inv2_scratch_bytes); ctl: inv_queue_ctl_ints(nj, Q) ints, zeroed once at
 // allocation (every launch leaves them zeroed).
 bool inv_queue_supported(int n, bool xi);
 size_t inv_queue_ctl_ints(int nj, int Q);
 int inv_queue_launch(int n, const FusedArgs& f, int nj, float2* T, int* ctl, cudaStream_t st);
-// The same queue over several instances of n = 256 in one launch: every instance's descriptor (written to
-// host memory by inv_queue_make_inst, which returns the instance's ticket count; tick0 = the tickets of the
-// instances before it) in a device table; ctl: 4 zeroed ints; cnt_all: ncnt zeroed ints holding every
-// instance's 2 nj counters (cnt); total = all tickets.  The launch leaves ctl and cnt_all zeroed.
+// The same queue over several instances of one size in one launch: every instance's descriptor (written to
+// host memory by inv_queue_make_inst; d0 = the depths of the instances before it) in a device table; ctl: 4
+// zeroed ints; cnt_all: the 2 nj zeroed counters (cnt) of every instance; depths: all of them.  The launch leaves ctl
+// and cnt_all zeroed.
 size_t inv_queue_inst_bytes();
-int inv_queue_make_inst(void* dst, const FusedArgs& f, float2* T, int* cnt, int nj, int tick0);
-int inv_queue_launch_table(const void* tab, int ninst, int* ctl, int* cnt_all, int ncnt, int total, cudaStream_t st);
+void inv_queue_make_inst(void* dst, const FusedArgs& f, float2* T, int* cnt, int nj, int d0);
+int inv_queue_launch_table(int n, const void* tab, int ninst, int* ctl, int* cnt_all, int depths, cudaStream_t st);
 // W_q = V0_q / sum_q' V0_q'^2 on the R grid for the handle's cached sources
 int build_wtab(const Handle* H, float* W, int Q, const double* pts64, int L, double coef, cudaStream_t st);
 int build_wtab64(const Handle* H, double* W, int Q, const double* pts64, int L, double coef, cudaStream_t st);
