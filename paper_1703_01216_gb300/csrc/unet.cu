@@ -117,9 +117,7 @@ namespace {
 
 __device__ __forceinline__ float bfv(uint32_t u, int hi) { return __uint_as_float(hi ? (u & 0xFFFF0000u) : (u << 16)); }
 __device__ __forceinline__ uint32_t pk(float a, float b) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
-  return r;
+  return (uint32_t)tc::bf16_rn(a) | ((uint32_t)tc::bf16_rn(b) << 16);
 }
 __device__ __forceinline__ void unpack8(const uint4& q, float* f) {
   const uint32_t w[4] = {q.x, q.y, q.z, q.w};
