@@ -31,11 +31,11 @@ struct AlphaInst {
   double inv_n2;   // 1 / n^2
   long ps;         // plane stride of the data spectra, (n/2 + 1) n
   int n, Cn;       // grid size and its frequency classes
-  int nplanes, na, nb, bstart, nblk;
+  int nplanes, na, nb, bstart, nblk, gsize;
 };
 
 // The alpha rule of every instance of a plan, all grid sizes, in one launch.  Each instance owns
-// alpha_blocks(Cn) consecutive blocks of the grid (the table is ordered by first block) and its own
+// consecutive blocks of the grid, one per 64 classes (the table is ordered by first block), and its own
 // partial sums and tickets.  A plan's grid is many waves of blocks, each a chain of dependent
 // steps, so four blocks per SM (64 registers, a 64-byte spill) run faster than two at 98 registers.
 __global__ void __launch_bounds__(256, 4) k_alpha_batched(const AlphaInst* __restrict__ inst, int ninst) {
@@ -46,8 +46,9 @@ __global__ void __launch_bounds__(256, 4) k_alpha_batched(const AlphaInst* __res
     else hi = mid - 1;
   }
   const AlphaInst a = inst[lo];
-  alpha_choose_body<float2>(a.Uh, a.ps, a.nplanes, a.n, a.Cn, a.Ft, a.na, a.thr2, a.cband, a.nb, a.inv_n2, a.partials,
-                            a.counter, a.aidx, a.res, a.info, a.tickets, (int)blockIdx.x - a.bstart, a.nblk);
+  alpha_choose_body<8>(a.Uh, a.ps, a.nplanes, a.n, a.Cn, a.Ft, a.na, a.thr2, a.cband, a.nb, a.inv_n2, a.partials,
+                            a.counter, a.aidx, a.res, a.info, a.tickets, (int)blockIdx.x - a.bstart, a.nblk, kAlphaCPB,
+                       a.gsize);
 }
 
 int inv_fused_batched_f32(int n, const FusedArgs* inst, const int2* map, int nclusters, int output, int variant,
@@ -225,7 +226,8 @@ void build_descriptors(const fr3d_instance* inst, const std::map<int, std::vecto
         a.nplanes = I.Q;
         a.na = I.opts->n_alpha;
         a.bstart = ap.nblk;
-        a.nblk = alpha_blocks(H->C);
+        a.nblk = alpha_blocks(H->C, kAlphaCPB);
+        a.gsize = alpha_group(a.nblk, a.nb * a.na);
         ap.nblk += a.nblk;
         ap.max_na = std::max(ap.max_na, a.na);
         alph.push_back(a);

@@ -146,6 +146,24 @@ struct Handle {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
+// Launch, with pdl = true with programmatic stream serialisation: the kernel may start once every block of the kernel before it in
+// the stream has released it or exited; it must call pdl_wait() in every thread before it touches what that kernel
+// (or, through that kernel's own wait, an earlier one) reads or writes.
+template <typename... P, typename... A>
+int launch_on(bool pdl, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...) == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
+}
+
 // launch-count bookkeeping (host)
 struct Launches {
   int n = 0;

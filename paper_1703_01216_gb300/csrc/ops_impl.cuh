@@ -30,8 +30,7 @@ static int row_r2c_t(const Handle* H, const PM& pm, int nplanes, cudaStream_t st
   auto kern = k_row_r2c<T, N, TY, PM>;
   FR3D_TRY(set_smem(kern, sm));
   dim3 grid(N / TY, nplanes);
-  kern<<<grid, kThreads, sm, st>>>(pm, tw_of<T>(H, N));
-  return cudaGetLastError() == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
+  return launch_on(true, kern, grid, kThreads, sm, st, pm, tw_of<T>(H, N));
 }
 
 template <typename T, int N>
@@ -49,8 +48,7 @@ static int col_t(const Handle* H, const Op& op, int nplanes, cudaStream_t st) {
   auto kern = k_col_fft<T, N, INV, Op, TC>;
   FR3D_TRY(set_smem(kern, sm));
   dim3 grid((N / 2 + 1 + TC - 1) / TC, nplanes);
-  kern<<<grid, kThreads, sm, st>>>(op, tw_of<T>(H, N));
-  return cudaGetLastError() == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
+  return launch_on(true, kern, grid, kThreads, sm, st, op, tw_of<T>(H, N));
 }
 
 template <typename T, int N, bool INV, class Op>
@@ -76,8 +74,8 @@ static int row_c2r_t(const Handle* H, const typename cpx<T>::t* in, T* out, int 
   if constexpr (sizeof(T) == 4) zr = H->zr32;
   else zr = H->zr64;
   dim3 grid(N / TY, nplanes);
-  kern<<<grid, kThreads, sm, st>>>(in, out, Q, j0, out_stride, s, g, zr, W, (long)H->Mp * N * N, tw_of<T>(H, N));
-  return cudaGetLastError() == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
+  return launch_on(true, kern, grid, kThreads, sm, st, in, out, Q, j0, out_stride, s, g, zr, W, (long)H->Mp * N * N,
+                   tw_of<T>(H, N));
 }
 
 template <typename T, int N, int MODE>
@@ -211,8 +209,8 @@ static int col_contract_n(const Handle* H, const typename cpx<T>::t* Zh, typenam
   auto kern = k_col_contract<T, N, TC>;
   FR3D_TRY(set_smem(kern, sm));
   const dim3 grid((N / 2 + TC) / TC, Q, chunks);
-  kern<<<grid, kContractThreads, sm, st>>>(Zh, part, A, H->Mp, (H->Mp + chunks - 1) / chunks, part_cs, tw_of<T>(H, N));
-  return cudaGetLastError() == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
+  return launch_on(true, kern, grid, kContractThreads, sm, st, Zh, part, A, H->Mp, (H->Mp + chunks - 1) / chunks, part_cs,
+                   tw_of<T>(H, N));
 }
 
 // Depth chunks of the contraction: enough CTAs to fill the SMs (five each at n = 256), at least four depths each, no
@@ -295,42 +293,100 @@ __device__ __forceinline__ void class_pq(int c, int& p, int& q) {
 __device__ __forceinline__ double sq_abs(float2 v) { return (double)fmaf(v.x, v.x, v.y * v.y); }
 __device__ __forceinline__ double sq_abs(double2 v) { return fma(v.x, v.x, v.y * v.y); }
 
-constexpr int kAlphaCPB = 64;  // classes per block
-constexpr int kAlphaSplit = 4; // threads per class in the power gather
-constexpr int kAlphaGroup = 8;   // blocks per group of the two-level reduction
-static_assert(kAlphaCPB == 64 && kAlphaGroup == 8,
-              "ensure_partials sizes the partial-sum buffer for 64 classes per block and 8 blocks per group");
-static_assert(256 / kAlphaSplit >= kAlphaCPB, "every class of a block has its gather threads");
+constexpr int kAlphaThreads = 256;
+constexpr int kAlphaCPB = 64;      // classes per block at most
+constexpr int kAlphaFill = 160;    // blocks that fill the chip (about one per SM)
 
 // Per band b of frequency classes (one band: the whole spectrum),
 //   r_b^2(alpha_k) = n^-2 sum_{c in b} Ft[c][k] P[c]  (Parseval; M = 1 closed form of the residual),
 // with P[c] the data power of class c: every stored half-spectrum bin of the class, weighted 1 on
 // the kx = 0 and kx = n/2 columns and 2 elsewhere (their mirror bins are not stored), summed over
 // planes.  The discrepancy rule picks, per band, the largest alpha_k with r_b^2 <= thr2.t[b].
-// Deterministic: fixed-order partial sums per block; per group of kAlphaGroup consecutive blocks, in
-// block order, by the group's last block to finish (an atomic ticket per group); over the groups, in
-// group order, by the last group to finish.  The tickets leave the blocks free to land on distinct
-// SMs (an 8-block cluster per group placed two blocks on some SMs and added two cluster barriers).
+// The kernel is a chain of dependent steps (6 MB at 256^2, 8 sources, 64 candidates, about 1 us of HBM time), so the
+// steps are kept short: the classes per block weigh the FP64 products of a block (64 classes and 64 candidates take
+// 1 us) against the sums of more blocks (alpha_cpb), a block's filter slab is fetched by asynchronous copies before the data
+// transform has finished (programmatic launch; the slab depends on the handle only), and the
+// block sums are reduced in one or two levels of tickets (alpha_group).
+// Deterministic: fixed-order sums of a block's classes; block sums in a fixed interleaved order.
 // FP64 runs at a small fraction of the FP32 rate on this GPU, so the serial parts avoid FP64 chains:
 // the choice is a warp ballot per band rather than a loop over candidates.
 struct BandThr {
   double t[FR3D_MAX_BANDS];
 };
 
-// blocks of the alpha rule for Cn classes: one per kAlphaCPB classes
-inline int alpha_blocks(int Cn) { return (Cn + kAlphaCPB - 1) / kAlphaCPB; }
-__host__ __device__ inline int alpha_groups(int nblk) { return (nblk + kAlphaGroup - 1) / kAlphaGroup; }
+inline int alpha_blocks(int Cn, int cpb) { return (Cn + cpb - 1) / cpb; }
+// Blocks per group of the reduction's first level.  One SM adds two FP64 numbers per cycle: up to 2048 numbers the last
+// block adds them all (a second level costs about 2600 cycles of fences and tickets), above that about sqrt(blocks)
+// groups share the work (132 blocks of 64 sums in one level: 4200 cycles; in 11 groups of 12: 384 + 352).
+inline int alpha_group(int nblk, int O) {
+  if (nblk * O <= 2048) return nblk;
+  int g = 8;
+  while (g * g < nblk) ++g;
+  return g;
+}
+// Classes per block for a single call (a multiple of 8 up to 64, at most kAlphaFill blocks unless 64 classes need
+// more): the fewest FP64 cycles of the products of a block and of the reduction of the blocks' sums.
+inline int alpha_cpb(int Cn, int na, int nb) {
+  const int O = na * nb;
+  int best = kAlphaCPB;
+  long bc = -1;
+  for (int c = kAlphaCPB; c >= 8; c -= 8) {
+    const int nblk = alpha_blocks(Cn, c), g = alpha_group(nblk, O), ngr = (nblk + g - 1) / g;
+    if (nblk > kAlphaFill && c < kAlphaCPB) break;
+    const long cost = (long)c * na / 2 + (ngr == 1 ? (long)nblk * O / 2 : 2600 + (long)(g + ngr) * O / 2);
+    if (bc < 0 || cost < bc) {
+      bc = cost;
+      best = c;
+    }
+  }
+  return best;
+}
 // the group tickets of the alpha rule in the handle's partial-sum buffer (tables.cu)
 unsigned* alpha_tickets(const Handle* H);
 
-template <typename C>
+__device__ __forceinline__ void cp_async(void* dst, const void* src, bool wide) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if (wide) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+
+// Sum of cnt vectors of O values, O apart: thread (t, o) adds every TPO-th vector (B loads in flight), the TPO sums of
+// an o are added in order and handed to emit(o, sum).  red: kAlphaThreads doubles.
+template <int B, class Em>
+__device__ __forceinline__ void alpha_reduce(const double* __restrict__ src, int cnt, int O, double* red, Em emit, int tid) {
+  const int Ow = min(O, kAlphaThreads), TPO = kAlphaThreads / Ow;
+  const int ol = tid % Ow, t = tid / Ow;
+  for (int o0 = 0; o0 < O; o0 += Ow) {
+    const int o = o0 + ol;
+    double s = 0.0;
+    if (o < O && t < TPO) {
+      for (int q0 = t; q0 < cnt; q0 += B * TPO) {
+        double v[B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) v[i] = __ldcg(src + (long)min(q0 + i * TPO, cnt - 1) * O + o);
+#pragma unroll
+        for (int i = 0; i < B; ++i)
+          if (q0 + i * TPO < cnt) s += v[i];   // (adding the zeros would cost the FP64 pipe as much)
+      }
+    }
+    red[tid] = s;
+    __syncthreads();
+    if (t == 0 && o < O) {
+      for (int k = 1; k < TPO; ++k) s += red[k * Ow + ol];
+      emit(o, s);
+    }
+    __syncthreads();
+  }
+}
+
+template <int B, typename C>
 __device__ __forceinline__ void alpha_choose_body(const C* __restrict__ Uh, long ps, int nplanes, int n, int Cn,
                                                   const double* __restrict__ Ft, int na, const BandThr& thr2,
                                                   const unsigned char* __restrict__ cband, int nb, double inv_n2,
                                                   double* __restrict__ partials, unsigned* __restrict__ counter,
                                                   int* __restrict__ aidx, double* __restrict__ res_out,
                                                   int* __restrict__ info, unsigned* __restrict__ gticket, int blk,
-                                                  int nblk) {
+                                                  int nblk, int cpb, int gsize) {
   // partials: [nblk][O] block sums, then [groups][O] group sums; gticket: one ticket per group
   // (alpha_tickets); counter: the ticket over the groups.  Every ticket is zero between launches.
   // Accumulation types: the class power P[c] is summed in the data's precision (at most 4 nplanes
@@ -338,140 +394,107 @@ __device__ __forceinline__ void alpha_choose_body(const C* __restrict__ Uh, long
   using A = typename std::conditional<std::is_same<C, float2>::value, float, double>::type;
   __shared__ double sP[kAlphaCPB];
   __shared__ unsigned char sB[kAlphaCPB];
-  __shared__ int present[FR3D_MAX_BANDS];
-  __shared__ double red[256];
+  __shared__ unsigned present;
+  __shared__ double red[kAlphaThreads];
   __shared__ double sPart[FR3D_MAX_BANDS * FR3D_MAX_ALPHAS];   // this block's sums; later the r^2 curves
   __shared__ int flg[FR3D_MAX_BANDS];
   __shared__ bool last;
-  extern __shared__ double sF[];             // [kAlphaCPB][na] slab of Ft for this block's classes
+  extern __shared__ __align__(16) double sF[];   // [cpb][na] slab of Ft for this block's classes
   const int tid = threadIdx.x;
-  const int c0 = blk * kAlphaCPB;
-  const int nF = max(0, min(kAlphaCPB, Cn - c0)) * na;
-  const double* slab = Ft + (long)c0 * na;
-  const int O = nb * na;
-  if (tid < FR3D_MAX_BANDS) present[tid] = 0;
-  // one round of global loads: this thread's share of the class powers and of the filter slab
-  const int cl = tid / kAlphaSplit, sub = tid % kAlphaSplit, c = c0 + cl;
-  const bool own = cl < kAlphaCPB;            // threads past the block's classes gather nothing
-  int kxs[4] = {0, 0, 0, 0}, kys[4] = {0, 0, 0, 0}, nm = 0;
-  if (own && c < Cn) {
-    int p, q;
-    class_pq(c, p, q);
-    // members (kx, ky) of the class in the half spectrum
-    kxs[nm] = p; kys[nm++] = q;
-    if (q != 0 && 2 * q != n) { kxs[nm] = p; kys[nm++] = n - q; }
-    if (p != q) {
-      kxs[nm] = q; kys[nm++] = p;
-      if (p != 0 && 2 * p != n) { kxs[nm] = q; kys[nm++] = n - p; }
-    }
+  const int c0 = blk * cpb, ncl = min(cpb, Cn - c0), O = nb * na;
+  {
+    const double* slab = Ft + (long)c0 * na;   // 16-byte aligned: c0 is a multiple of 8
+    const int nF = ncl * na;
+    for (int e = 2 * tid; e < nF; e += 2 * kAlphaThreads) cp_async(sF + e, slab + e, e + 1 < nF);
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  double f[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const int e = tid + i * 256;
-    f[i] = e < nF ? __ldg(slab + e) : 0.0;
-  }
+  if (tid == 0) present = 0;
+  for (int o = tid; o < O; o += kAlphaThreads) sPart[o] = 0.0;
+  // class powers: `split` adjacent lanes per class share its (member, plane) items; member m of class (p, q):
+  // (p, q), (p, n - q), (q, p), (q, n - p), where they are distinct stored bins
+  const int split = 1 << (31 - __clz(kAlphaThreads / cpb)), cl = tid / split, sub = tid % split, c = c0 + cl;
+  int p = 0, q = 0;
+  if (cl < ncl) class_pq(c, p, q);
+  const bool mirq = q != 0 && 2 * q != n, mirp = p != 0 && 2 * p != n;
+  const A wp = (p == 0 || 2 * p == n) ? A(1) : A(2), wq = (q == 0 || 2 * q == n) ? A(1) : A(2);
+  pdl_wait();   // the data spectra
   A acc = 0;
-  for (int pl0 = sub; pl0 < nplanes; pl0 += 2 * kAlphaSplit) {
-    A s[4][2];
+  if (cl < ncl)
+    for (int i0 = sub; i0 < 4 * nplanes; i0 += 8 * split) {
+      C v[8];
+      A w[8];   // 0: no such item (it reads the class's first bin instead: no branch between the loads)
 #pragma unroll
-    for (int mi = 0; mi < 4; ++mi)
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int pl = pl0 + u * kAlphaSplit;
-        const C v = (mi < nm && pl < nplanes) ? __ldg(Uh + pl * ps + (long)kxs[mi] * n + kys[mi]) : C{0, 0};
-        s[mi][u] = v.x * v.x + v.y * v.y;
+      for (int u = 0; u < 8; ++u) {
+        const int i = i0 + u * split, m = i & 3, pl = i >> 2;
+        const bool has = pl < nplanes && (m == 0 || (m == 1 && mirq) || (m == 2 && p != q) || (m == 3 && p != q && mirp));
+        const int kx = m < 2 ? p : q, ky = m == 0 ? q : (m == 1 ? n - q : (m == 2 ? p : n - p));
+        v[u] = __ldcg(Uh + (has ? pl * ps + (long)kx * n + ky : (long)p * n + q));
+        w[u] = has ? (m < 2 ? wp : wq) : A(0);
       }
 #pragma unroll
-    for (int mi = 0; mi < 4; ++mi)
-      if (mi < nm) acc += ((kxs[mi] == 0 || 2 * kxs[mi] == n) ? A(1) : A(2)) * (s[mi][0] + s[mi][1]);
-  }
-  // the kAlphaSplit threads of a class are adjacent lanes: combine them in a fixed order
-#pragma unroll
-  for (int m = 1; m < kAlphaSplit; m <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, m);
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const int e = tid + i * 256;
-    if (e < nF) sF[e] = f[i];
-  }
-  // slabs longer than 16 loads per thread (more than 64 candidates) finish here
-  for (int e = tid + 16 * 256; e < nF; e += 256) sF[e] = __ldg(slab + e);
-  if (sub == 0 && own) {
-    sP[cl] = (double)acc;
-    const int b = (c < Cn && nb > 1) ? (int)cband[c] : 0;
-    sB[cl] = (unsigned char)b;
-    if (c < Cn) present[b] = 1;
-  }
-  __syncthreads();
-  // per band: this block's sums of F[c][k] P[c] (S threads per candidate, fixed order)
-  const int S = 256 / na;
-  for (int b = 0; b < nb; ++b) {
-    if (present[b]) {
-      if (tid < S * na) {
-        const int k = tid % na, sb = tid / na;
-        double a2 = 0.0;
-        for (int cc = sb; cc < kAlphaCPB; cc += S)
-          if (c0 + cc < Cn && sB[cc] == b) a2 = fma(sF[cc * na + k], sP[cc], a2);
-        red[tid] = a2;
-      }
-      __syncthreads();
+      for (int u = 0; u < 8; ++u)
+        if (w[u] != A(0)) acc += w[u] * (v[u].x * v[u].x + v[u].y * v[u].y);
     }
+  for (int m = 1; m < split; m <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, m);   // fixed order
+  __syncthreads();   // present and the zeros
+  if (sub == 0 && cl < ncl) {
+    sP[cl] = (double)acc;
+    const int b = nb > 1 ? (int)cband[c] : 0;
+    sB[cl] = (unsigned char)b;
+    if (nb > 1) atomicOr(&present, 1u << b);
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  // per band of this block: the sums of F[c][k] P[c] (S threads per candidate, fixed order)
+  const int S = kAlphaThreads / na, kc = tid % na, sb = tid / na;
+  for (unsigned bands = nb > 1 ? present : 1u; bands; bands &= bands - 1) {
+    const int b = __ffs(bands) - 1;
+    double a2 = 0.0;
+    if (sb < S) {
+#pragma unroll 4
+      for (int cc = sb; cc < ncl; cc += S)
+        if (nb == 1 || sB[cc] == b) a2 = fma(sF[cc * na + kc], sP[cc], a2);
+    }
+    red[tid] = a2;
+    __syncthreads();
     if (tid < na) {
-      double s = 0.0;
-      if (present[b])
-        for (int sb = 0; sb < S; ++sb) s += red[sb * na + tid];
-      sPart[b * na + tid] = s;
+      for (int k = 1; k < S; ++k) a2 += red[k * na + tid];
+      sPart[b * na + tid] = a2;
     }
     __syncthreads();
   }
-  // level 1: this block's sums, then a ticket of its group; the group's last block adds the group's
-  // block sums in block order
-  const int ngr = alpha_groups(nblk);
-  double* gpart = partials + (long)nblk * O;
-  for (int o = tid; o < O; o += 256) partials[(long)blk * O + o] = sPart[o];
+  for (int o = tid; o < O; o += kAlphaThreads) partials[(long)blk * O + o] = sPart[o];
+  // level 1: a ticket of the block's group; the group's last block adds the group's block sums
+  const int ngr = (nblk + gsize - 1) / gsize, g = blk / gsize, gsz = min(gsize, nblk - g * gsize);
   __threadfence();
   __syncthreads();
-  const int g = blk / kAlphaGroup;
-  const int gsz = min(kAlphaGroup, nblk - g * kAlphaGroup);
   if (tid == 0) last = atomicAdd(gticket + g, 1u) == (unsigned)(gsz - 1);
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int o = tid; o < O; o += 256) {
-    double v[kAlphaGroup];
-#pragma unroll
-    for (int q = 0; q < kAlphaGroup; ++q) v[q] = q < gsz ? __ldcg(partials + (long)(g * kAlphaGroup + q) * O + o) : 0.0;
-    double s = 0.0;
-#pragma unroll
-    for (int q = 0; q < kAlphaGroup; ++q)
-      if (q < gsz) s += v[q];
-    gpart[(long)g * O + o] = s;
-  }
-  // level 2: a ticket over the groups
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    gticket[g] = 0u;
-    last = atomicAdd(counter, 1u) == (unsigned)(ngr - 1);
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  // every other block has finished: let a programmatically launched successor start its set-up
-  pdl_release();
-  // the last group: r^2 per (band, candidate) over the group sums (24 loads in flight per round)
-  for (int o = tid; o < O; o += 256) {
-    double s = 0.0;
-    for (int g0 = 0; g0 < ngr; g0 += 24) {
-      double v[24];
-#pragma unroll
-      for (int i = 0; i < 24; ++i) v[i] = g0 + i < ngr ? __ldcg(gpart + (long)(g0 + i) * O + o) : 0.0;
-#pragma unroll
-      for (int i = 0; i < 24; ++i) s += v[i];
-    }
+  if (tid == 0) gticket[g] = 0u;
+  auto final_sum = [&](int o, double s) {
     s *= inv_n2;
     sPart[o] = s;
     if (res_out) res_out[o] = s;
+  };
+  const double* mine = partials + (long)g * gsize * O;
+  if (ngr == 1) {
+    pdl_release();   // every other block has finished: a programmatic successor may start its set-up
+    alpha_reduce<B>(mine, gsz, O, red, final_sum, tid);
+  } else {
+    // level 2: a ticket over the groups; the last group adds the group sums
+    double* gpart = partials + (long)nblk * O;
+    alpha_reduce<B>(mine, gsz, O, red, [&](int o, double s) { gpart[(long)g * O + o] = s; }, tid);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(counter, 1u) == (unsigned)(ngr - 1);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    pdl_release();
+    alpha_reduce<B>(gpart, ngr, O, red, final_sum, tid);
+    if (tid == 0) *counter = 0u;
   }
   __syncthreads();
   // choice per band, one warp per band: ballots of r^2 <= thr over the candidates, largest index wins
@@ -508,35 +531,32 @@ __device__ __forceinline__ void alpha_choose_body(const C* __restrict__ Uh, long
     int flags = 0;
     for (int b = 0; b < nb; ++b) flags |= flg[b];
     if (info) *info = flags;
-    *counter = 0u;
   }
 }
 
 template <typename C>
-__global__ void __launch_bounds__(256) k_alpha_choose(const C* __restrict__ Uh, long ps, int nplanes, int n, int Cn,
-                                                      const double* __restrict__ Ft, int na, BandThr thr2,
-                                                      const unsigned char* __restrict__ cband, int nb, double inv_n2,
-                                                      double* __restrict__ partials, unsigned* __restrict__ counter,
-                                                      int* __restrict__ aidx, double* __restrict__ res_out,
-                                                      int* __restrict__ info, unsigned* __restrict__ gticket) {
-  alpha_choose_body(Uh, ps, nplanes, n, Cn, Ft, na, thr2, cband, nb, inv_n2, partials, counter, aidx, res_out, info,
-                    gticket, (int)blockIdx.x, (int)gridDim.x);
+__global__ void __launch_bounds__(kAlphaThreads) k_alpha_choose(
+    const C* __restrict__ Uh, long ps, int nplanes, int n, int Cn, const double* __restrict__ Ft, int na, BandThr thr2,
+    const unsigned char* __restrict__ cband, int nb, double inv_n2, double* __restrict__ partials,
+    unsigned* __restrict__ counter, int* __restrict__ aidx, double* __restrict__ res_out, int* __restrict__ info,
+    unsigned* __restrict__ gticket, int cpb, int gsize) {
+  alpha_choose_body<16>(Uh, ps, nplanes, n, Cn, Ft, na, thr2, cband, nb, inv_n2, partials, counter, aidx, res_out, info,
+                        gticket, (int)blockIdx.x, (int)gridDim.x, cpb, gsize);
 }
 
 template <typename T>
 int Ops<T>::alpha_choose(Handle* H, const C* Uh, int nplanes, int n_alpha, const double* thr2, int nb, int* aidx,
                          double* residuals, int* info, cudaStream_t st) {
-  const int blocks = alpha_blocks(H->C);
+  const int cpb = alpha_cpb(H->C, n_alpha, nb), blocks = alpha_blocks(H->C, cpb);
   FR3D_TRY(ensure_partials(H));
   const long ps = (long)(H->n / 2 + 1) * H->n;
-  const size_t sm = sizeof(double) * kAlphaCPB * n_alpha;
+  const size_t sm = sizeof(double) * cpb * n_alpha;
   FR3D_TRY(set_smem(k_alpha_choose<C>, sm));
   BandThr t;
   for (int b = 0; b < nb; ++b) t.t[b] = thr2[b];
-  k_alpha_choose<C><<<blocks, 256, sm, st>>>(Uh, ps, nplanes, H->n, H->C, H->Ft, n_alpha, t, H->cband, nb,
-                                            1.0 / ((double)H->n * H->n), H->partials, H->counter, aidx, residuals,
-                                            info, alpha_tickets(H));
-  return cudaGetLastError() == cudaSuccess ? FR3D_OK : FR3D_ERR_CUDA;
+  return launch_on(true, k_alpha_choose<C>, dim3(blocks), kAlphaThreads, sm, st, Uh, ps, nplanes, H->n, H->C, H->Ft, n_alpha,
+                    t, H->cband, nb, 1.0 / ((double)H->n * H->n), H->partials, H->counter, aidx, residuals, info,
+                    alpha_tickets(H), cpb, alpha_group(blocks, nb * n_alpha));
 }
 
 }  // namespace fr3d

@@ -100,19 +100,20 @@ int alpha_tables(Handle* H, const double* alphas, int n_alpha, int ra, cudaStrea
 }
 
 // The handle's partial-sum buffer: data, then the alpha rule's group tickets at a fixed offset.
-// Data: the alpha rule's [blocks][O] block sums and [groups][O] group sums (blocks of 64 classes,
-// groups of 8 blocks, O <= FR3D_MAX_ALPHAS * FR3D_MAX_BANDS); the M > 1 rule's [blocks of 64
+// Data: the alpha rule's [blocks][O] block sums and [groups][O] group sums (blocks of 8 to 64 classes: at most 160, or
+// one per 64 classes; O <= FR3D_MAX_ALPHAS * FR3D_MAX_BANDS); the M > 1 rule's [blocks of 64
 // classes][bands][alphas]; the learned rule's at most 2 * 152 blocks of FR3D_MAX_BANDS sums.
 // Tickets: one unsigned per group, zero between launches (zeroed here, reset by the launch that
 // used them).
+static long max_partial_blocks(int C) { return std::max((C + 63) / 64, std::min(160, (C + 7) / 8)); }
 static long partial_data_doubles(int C) {
-  const long blocks = (C + 63) / 64, groups = (blocks + 7) / 8;
+  const long blocks = max_partial_blocks(C), groups = (blocks + 7) / 8;
   return std::max((blocks + groups) * (long)FR3D_MAX_ALPHAS * FR3D_MAX_BANDS, 2L * 152 * FR3D_MAX_BANDS);
 }
 
 int ensure_partials(Handle* H) {
   const long data = partial_data_doubles(H->C);
-  const long groups = ((H->C + 63) / 64 + 7) / 8;
+  const long groups = (max_partial_blocks(H->C) + 7) / 8;
   const long need = data + (groups + 1) / 2;
   if (H->partial_cap >= need) return FR3D_OK;
   if (H->partials) cudaFree(H->partials);
