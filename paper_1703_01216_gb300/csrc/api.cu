@@ -247,21 +247,23 @@ int choose_impl(Handle* H, const T* U, int Q, const double* alphas, int n_alpha,
 struct InvertPlan {
   size_t uh_off, t_off, uin_off, out_off, total;
   int chunk;
+  bool bins;   // M > 1: the spectra in bin order (multi.cu)
 };
 
 template <typename T>
-InvertPlan plan_invert(const Handle* H, int Q, bool host_io, int output) {
+InvertPlan plan_invert(const Handle* H, int Q, bool host_io, int output, bool bins = false) {
   using C = typename Ops<T>::C;
   const int n = H->n;
   const size_t ps_b = sizeof(C) * (size_t)(n / 2 + 1) * n;
   InvertPlan p;
   p.uh_off = 0;
+  p.bins = bins;
   size_t off = align_up(ps_b * Q * H->M);
   const size_t per_j = ps_b * Q;
   const bool fused = sizeof(T) == 4 && fused_supported(n);
   const bool multi = sizeof(T) == 4 && H->M > 1;      // the M > 1 path lays out its own workspace first
   int chunk = fused ? 0 : (int)std::max<size_t>(1, std::min<size_t>(H->Mp, kChunkBytes / per_j));
-  if (multi) off = multi_ws_bytes(H, Q);
+  if (multi) off = multi_ws_bytes(H, Q, bins);
   if (fused || multi) {
     p.chunk = H->Mp;
     p.t_off = off;
@@ -289,6 +291,20 @@ InvertPlan plan_invert(const Handle* H, int Q, bool host_io, int output) {
   }
   p.total = off;
   return p;
+}
+
+// The plan with its workspace allocated; M > 1 goes to plane order where there is no room for bin order (which
+// takes |M - M'| Q half spectra more).
+template <typename T>
+int reserve_invert(Handle* H, int Q, bool host_io, int output, InvertPlan* p) {
+  const bool bins = sizeof(T) == 4 && H->M > 1 && multi_bins(H);
+  *p = plan_invert<T>(H, Q, host_io, output, bins);
+  const int rc = ensure_ws(H, p->total);
+  if (rc != FR3D_ERR_OOM || !bins) return rc;
+  cudaGetLastError();
+  H->no_bins = true;
+  *p = plan_invert<T>(H, Q, host_io, output, false);
+  return ensure_ws(H, p->total);
 }
 
 int check_invert_args(Handle* H, int Q, const fr3d_invert_opts* o) {
@@ -345,7 +361,7 @@ int invert_impl(Handle* H, const T* U, int Q, const fr3d_invert_opts* o, T* out,
         }
       }
       const SrcHost src = o->output == FR3D_OUT_XI ? src_host(H, FR3D_PREC_FP32, o->sources) : SrcHost{};
-      return invert_multi(H, U, Q, o, out, src, W, st);
+      return invert_multi(H, U, Q, o, out, src, W, p.bins, st);
     }
   }
   C* Uh = reinterpret_cast<C*>((char*)H->ws + p.uh_off);
@@ -545,8 +561,8 @@ extern "C" int fr3d_invert(fr3d_handle* h, const void* U, int Q, const fr3d_inve
     FR3D_TRY(fr3d::ensure_ws(H, p.total));
     return fr3d::invert_impl<double>(H, (const double*)U, Q, opts, (double*)out, p, st);
   }
-  const fr3d::InvertPlan p = fr3d::plan_invert<float>(H, Q, false, opts->output);
-  FR3D_TRY(fr3d::ensure_ws(H, p.total));
+  fr3d::InvertPlan p;
+  FR3D_TRY(fr3d::reserve_invert<float>(H, Q, false, opts->output, &p));
   return fr3d::invert_impl<float>(H, (const float*)U, Q, opts, (float*)out, p, st);
 }
 
@@ -570,8 +586,8 @@ static void* host_mapped_alias(const void* p, size_t bytes) {
 template <typename T>
 static int invert_host_t(Handle* H, const void* U_host, int Q, const fr3d_invert_opts* o, void* out_host,
                          cudaStream_t st) {
-  const fr3d::InvertPlan p = fr3d::plan_invert<T>(H, Q, true, o->output);
-  FR3D_TRY(fr3d::ensure_ws(H, p.total));
+  fr3d::InvertPlan p;
+  FR3D_TRY(fr3d::reserve_invert<T>(H, Q, true, o->output, &p));
   const int n = H->n;
   T* Ud = reinterpret_cast<T*>((char*)H->ws + p.uin_off);
   T* Od = reinterpret_cast<T*>((char*)H->ws + p.out_off);

@@ -116,6 +116,7 @@ struct Handle {
   // workspace
   void* ws = nullptr;
   size_t ws_bytes = 0;
+  bool no_bins = false;              // bin order did not fit once: the layout stays (captured work keeps its workspace)
   int last_launches = 0;
   // fused-inverse tile variant of the last call, and the autotuner's timings (ms) if it ran
   int fused_var = 0;

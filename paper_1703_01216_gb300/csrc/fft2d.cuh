@@ -157,6 +157,45 @@ __global__ void __launch_bounds__(kThreads) k_col_fft(Op op, const typename cpx<
   }
 }
 
+// Column pass between plane order [plane][kx][ky] and bin order [kx][ky][plane] (the per-class products of several
+// observation depths read and write whole records): one CTA transforms the column kx of PB planes, so the bin-ordered
+// side moves in segments of PB values (64 bytes at n = 512) and the plane-ordered side in whole columns.
+template <int N, bool INV, int PB>
+__global__ void __launch_bounds__(kThreads) k_col_bins(const float2* in, float2* out, int nplanes,
+                                                       const float2* __restrict__ tw) {
+  using C = float2;
+  constexpr int SS = Smem<C, N>::ss;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* ptw = reinterpret_cast<C*>(smem_raw);
+  C* buf = ptw + passtw_size<N>();
+  const int tid = threadIdx.x, kx = blockIdx.x, p0 = blockIdx.y * PB, np = min(PB, nplanes - p0);
+  const long ps = (long)(N / 2 + 1) * N;
+  build_passtw<N, 1, kThreads>(ptw, tw, tid);
+  pdl_wait();
+  const C* planes = in + p0 * ps + (long)kx * N;   // (forward)
+  const long rec = (long)kx * N * nplanes + p0;
+  batched_copy<PB * N, kThreads, 8>(
+      tid,
+      [&](int e) {
+        const int pl = INV ? e % PB : e / N, ky = INV ? e / PB : e % N;
+        if (pl >= np) return cmk(0.f, 0.f);
+        return INV ? in[rec + (long)ky * nplanes + pl] : planes[pl * ps + ky];
+      },
+      [&](int e, C v) {
+        const int pl = INV ? e % PB : e / N, ky = INV ? e / PB : e % N;
+        buf[pl * SS + pidx<C>(ky)] = v;
+      });
+  __syncthreads();
+  fft_smem<N, INV, PB, kThreads>(buf, SS, ptw, tid);
+  for (int e = tid; e < PB * N; e += kThreads) {
+    const int pl = INV ? e / N : e % PB, ky = INV ? e % N : e / PB;
+    if (pl >= np) continue;
+    const C v = buf[pl * SS + pidx<C>(ky)];
+    if (INV) out[(p0 + pl) * ps + (long)kx * N + ky] = v;
+    else out[rec + (long)ky * nplanes + pl] = v;
+  }
+}
+
 // plain forward/inverse column pass, plane p -> plane p
 template <typename T> struct ColPlain {
   using C = typename cpx<T>::t;

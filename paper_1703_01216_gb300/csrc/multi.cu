@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(256) k_class_eig(const double* __restrict__ A6
 
 // Projection p = U_c^T U~ in place for every member bin and plane set q, and the class powers
 // P_ci = sum over members and q of wt |p_i|^2 (FP32 terms in a fixed order, stored in FP64).
-// Uh planes are [q][i] (plane q M + i).  One warp per class: the class's member values of a plane set
+// Uh holds value (bin, q, i) at the strides sp.  One warp per class: the class's member values of a plane set
 // are gathered into the warp's shared-memory slice, lane l owns components i = l, l + 32, and the
 // eigenvector table (stored [k][i]) streams from global memory in coalesced rows, each element
 // feeding every member.  Classes own disjoint bins, so the in-place writes never meet another
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) k_class_eig(const double* __restrict__ A6
 constexpr int kPerCta = 8;                      // warps (classes) per CTA
 constexpr int kRows = (kMaxM + 31) / 32;        // components (or depths) per lane
 constexpr int kBatch = 4;                       // table rows per batch of the double-buffered stream
-__global__ void __launch_bounds__(256) k_project(float2* __restrict__ Uh, long ps, int Q, int M, int n, int Cn,
+__global__ void __launch_bounds__(256) k_project(float2* __restrict__ Uh, SpecStride sp, int Q, int M, int n, int Cn,
                                                  const float* __restrict__ Ut, double* __restrict__ Pc) {
   __shared__ float2 xs[kPerCta][4 * kMaxM];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(256) k_project(float2* __restrict__ Uh, long p
     load(0, 0);   // the first batch is in flight during the gather
     for (int e = lane; e < nm * M; e += 32) {
       const int m = e / M, k = e - m * M;
-      x[e] = Uh[((long)q * M + k) * ps + bin[m]];
+      x[e] = Uh[bin[m] * sp.b + q * sp.q + k * sp.k];
     }
     __syncwarp();
     float2 y[kRows][4];
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(256) k_project(float2* __restrict__ Uh, long p
 #pragma unroll
         for (int m = 0; m < 4; ++m)
           if (m < nm) {
-            Uh[((long)q * M + i) * ps + bin[m]] = y[r][m];
+            Uh[bin[m] * sp.b + q * sp.q + i * sp.k] = y[r][m];
             pw[r] = fmaf(wts[m], y[r][m].x * y[r][m].x + y[r][m].y * y[r][m].y, pw[r]);
           }
       }
@@ -367,17 +367,17 @@ __global__ void __launch_bounds__(kMFinish) k_alpha_m_finish(const double* __res
 }
 
 // zeta~_j(bin, q) = sum_i W_c[i][j] g_i p_i(bin, q) / n^2 with g_i of the class's band alpha, written to
-// the spectra Zs [q][j][bin] (jq = 0: the fused inverse's order) or [j][q][bin] (jq = 1: the order of the
-// two-pass inverse).  One warp per class: the scaled projected data g_i p_i of the members
+// the spectra Zs at the strides sz (planes [q][j] for the fused inverse, [j][q] for the two-pass inverse, or bin
+// order).  One warp per class: the scaled projected data g_i p_i of the members
 // for one q sit in the warp's shared-memory slice, lane l owns depths j = j0 + l, j0 + l + 32 of a
 // 64-depth chunk, and W_c (stored [i][j]) streams from global memory in coalesced rows, each element
 // feeding every member.
-__global__ void __launch_bounds__(256) k_solve_m(const float2* __restrict__ P, long ps, int Q, int M, int Mp, int n,
+__global__ void __launch_bounds__(256) k_solve_m(const float2* __restrict__ P, SpecStride sp, int Q, int M, int Mp, int n,
                                                  int Cn, const double* __restrict__ lam, const float* __restrict__ W,
                                                  const unsigned char* __restrict__ cband, int nb,
                                                  const int* __restrict__ aidx, int na, MAlphas al,
                                                  const double* __restrict__ s2, int ra, double inv_n2,
-                                                 float2* __restrict__ Zs, int jq) {
+                                                 float2* __restrict__ Zs, SpecStride sz) {
   constexpr int kJ = 2;   // depths per lane in a chunk of 64
   __shared__ float2 xs[kPerCta][4 * kMaxM];
   __shared__ float gs[kPerCta][kMaxM];
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(256) k_solve_m(const float2* __restrict__ P, l
   for (int q = 0; q < Q; ++q) {
     for (int e = lane; e < nm * M; e += 32) {
       const int m = e / M, i = e - m * M;
-      const float2 v = P[((long)q * M + i) * ps + bin[m]];
+      const float2 v = P[bin[m] * sp.b + q * sp.q + i * sp.k];
       x[e] = make_float2(v.x * g[i], v.y * g[i]);
     }
     __syncwarp();
@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(256) k_solve_m(const float2* __restrict__ P, l
         if (jj < Mp)
 #pragma unroll
           for (int m = 0; m < 4; ++m)
-            if (m < nm) Zs[(jq ? (long)jj * Q + q : (long)q * Mp + jj) * ps + bin[m]] = z[t][m];
+            if (m < nm) Zs[bin[m] * sz.b + q * sz.q + jj * sz.k] = z[t][m];
       }
     }
     __syncwarp();   // the x reads are done before the next q is gathered
@@ -510,47 +510,70 @@ int ensure_multi_tables(Handle* H, cudaStream_t st) {
   return FR3D_OK;
 }
 
-// workspace of invert_multi: data spectra [Q][M], solved spectra [Q][M'], class powers [C][M]
-size_t multi_ws_bytes(const Handle* H, int Q) {
-  const size_t ps = (size_t)(H->n / 2 + 1) * H->n;
-  auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  return up(sizeof(float2) * ps * Q * H->M) + up(sizeof(float2) * ps * Q * H->Mp) + up(sizeof(double) * H->C * H->M);
-}
-
 namespace {
-
-struct MultiWs {
-  float2* Uh;   // [Q][M] half spectra, projected in place
-  float2* Zs;   // [Q][M'] solved spectra
-  double* Pc;   // [C][M] class powers
-};
 
 size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-int multi_ws(Handle* H, int Q, bool with_zs, MultiWs* w) {
+// From this grid on the spectra of the per-class products are kept in bin order (a class member's components
+// adjacent), written by the forward column pass and read by the inverse one: a class gathers and scatters
+// whole records instead of 8-byte values a plane apart, each of which cost a 32-byte sector.  Below it the fused
+// inverse on plane-ordered spectra saves two launches.  Whole inversions: 512^2, M = M' = 51, 516 us in plane order
+// and 449 in bin order (projection 169 -> 131, solve 168 -> 120, the column passes + 6 each); 256^2, M = 40,
+// M' = 64, split BF16, 187 -> 167.
+constexpr int kBinsMinN = 192;
+
+struct MultiWs {
+  bool bins;
+  float2* Uh;     // half spectra of the data at the strides su, projected in place
+  float2* Zs;     // solved spectra at the strides sz; bin order: first the planes of the forward row pass
+  float2* rows;   // planes of the inverse row pass: Zs, or (bin order) in the place of Uh
+  double* Pc;     // [C][M] class powers
+  SpecStride su, sz;
+  size_t total;
+};
+
+// layout from the start of the handle's workspace; base: null to get the size alone
+MultiWs multi_layout(const Handle* H, int Q, bool with_zs, bool bins, char* base) {
   const long ps = (long)(H->n / 2 + 1) * H->n;
-  const size_t ub = up256(sizeof(float2) * ps * Q * H->M);
-  const size_t zb = with_zs ? up256(sizeof(float2) * ps * Q * H->Mp) : 0;
-  const size_t pb = up256(sizeof(double) * H->C * H->M);
-  FR3D_TRY(ensure_ws(H, std::max(ub + zb + pb, with_zs ? multi_ws_bytes(H, Q) : 0)));
-  w->Uh = reinterpret_cast<float2*>(H->ws);
-  w->Zs = with_zs ? reinterpret_cast<float2*>((char*)H->ws + ub) : nullptr;
-  w->Pc = reinterpret_cast<double*>((char*)H->ws + ub + zb);
-  return FR3D_OK;
+  size_t ub = up256(sizeof(float2) * ps * Q * H->M);
+  size_t zb = with_zs ? up256(sizeof(float2) * ps * Q * H->Mp) : 0;
+  if (bins) ub = zb = std::max(ub, zb);   // the column passes are out of place: each part holds planes and records in turn
+  MultiWs w;
+  w.bins = bins;
+  w.Uh = reinterpret_cast<float2*>(base);
+  w.Zs = zb ? reinterpret_cast<float2*>(base + ub) : nullptr;
+  w.rows = bins ? w.Uh : w.Zs;
+  w.Pc = reinterpret_cast<double*>(base + ub + zb);
+  // bin order: records [q][i] of the data and [j][q] of the solved spectra (the two-pass inverse's plane order)
+  w.su = bins ? SpecStride{(long)Q * H->M, H->M, 1} : SpecStride{1, H->M * ps, ps};
+  w.sz = bins ? SpecStride{(long)Q * H->Mp, 1, Q}
+              : (fused_supported(H->n) ? SpecStride{1, H->Mp * ps, ps} : SpecStride{1, ps, Q * ps});
+  w.total = ub + zb + up256(sizeof(double) * H->C * H->M);
+  return w;
 }
+
+}  // namespace
+
+bool multi_bins(const Handle* H) { return H->n >= kBinsMinN && !H->no_bins; }
+
+// workspace of invert_multi: data spectra [Q][M], solved spectra [Q][M'], class powers [C][M]
+size_t multi_ws_bytes(const Handle* H, int Q, bool bins) { return multi_layout(H, Q, true, bins, nullptr).total; }
+
+namespace {
 
 // data spectra of every (q, i) plane and their projection onto the class eigenvectors
 int multi_data(Handle* H, const float* U, int Q, const MultiWs& w, int precision, int* info, int* launches,
                cudaStream_t st) {
-  const long ps = (long)(H->n / 2 + 1) * H->n;
-  FR3D_TRY(Ops<float>::row_r2c(H, U, (long)H->n * H->n, w.Uh, Q * H->M, st));
+  float2* rows = w.bins ? w.Zs : w.Uh;
+  FR3D_TRY(Ops<float>::row_r2c(H, U, (long)H->n * H->n, rows, Q * H->M, st));
   prof_mark(H, kStRowR2C, st);
-  FR3D_TRY(Ops<float>::col_plain(H, w.Uh, w.Uh, Q * H->M, false, st));
+  if (w.bins) FR3D_TRY(Ops<float>::col_to_bins(H, rows, w.Uh, Q * H->M, st));
+  else FR3D_TRY(Ops<float>::col_plain(H, w.Uh, w.Uh, Q * H->M, false, st));
   prof_mark(H, kStColFwd, st);
   if (tc_precision(precision)) {
-    FR3D_TRY(tc_project(H, w.Uh, Q, w.Pc, precision == FR3D_PREC_BF16X3, info, st));
+    FR3D_TRY(tc_project(H, w.Uh, w.su, Q, w.Pc, precision == FR3D_PREC_BF16X3, info, st));
   } else {
-    k_project<<<(H->C + kPerCta - 1) / kPerCta, 32 * kPerCta, 0, st>>>(w.Uh, ps, Q, H->M, H->n, H->C, H->mUt, w.Pc);
+    k_project<<<(H->C + kPerCta - 1) / kPerCta, 32 * kPerCta, 0, st>>>(w.Uh, w.su, Q, H->M, H->n, H->C, H->mUt, w.Pc);
     FR3D_CUDA_TRY(cudaGetLastError());
   }
   prof_mark(H, kStOther, st);
@@ -579,13 +602,13 @@ int multi_alpha(Handle* H, const MultiWs& w, const double* alphas, int na, int r
 // Algorithm 1 for M > 1 (FP32 data and FFTs, FP64 eigen tables and residual sums).
 // The combination table (XI) is built by the caller.
 int invert_multi(Handle* H, const float* U, int Q, const fr3d_invert_opts* o, float* out, const SrcHost& src,
-                 const float* W, cudaStream_t st) {
+                 const float* W, bool bins, cudaStream_t st) {
   FR3D_TRY(ensure_multi_tables(H, st));
   const int nb = o->n_bands > 1 ? o->n_bands : 1;
   std::vector<double> count;
   FR3D_TRY(ensure_bands(H, nb, &count));
-  MultiWs w;
-  FR3D_TRY(multi_ws(H, Q, true, &w));
+  FR3D_TRY(ensure_ws(H, multi_ws_bytes(H, Q, bins)));
+  const MultiWs w = multi_layout(H, Q, true, bins, (char*)H->ws);
   const bool tcp = tc_precision(o->precision);
   if (tcp) {
     FR3D_TRY(ensure_tc_tables(H, 0, st));
@@ -621,16 +644,15 @@ int invert_multi(Handle* H, const float* U, int Q, const fr3d_invert_opts* o, fl
       if (o->info && !tcp) FR3D_CUDA_TRY(cudaMemsetAsync(o->info, 0, sizeof(int), st));
     }
   }
-  const long ps = (long)(H->n / 2 + 1) * H->n;
   const int na = o->alpha_mode == FR3D_ALPHA_FIXED ? 1 : o->n_alpha;
-  const bool fused = fused_supported(H->n);
+  const bool fused = fused_supported(H->n) && !bins;
   if (tcp) {
-    FR3D_TRY(tc_solve(H, w.Uh, Q, aidx, al.a, na, o->ra, nb, w.Zs, fused ? 0 : 1, o->precision == FR3D_PREC_BF16X3,
-                      o->info, st));
+    FR3D_TRY(tc_solve(H, w.Uh, w.su, Q, aidx, al.a, na, o->ra, nb, w.Zs, w.sz, o->precision == FR3D_PREC_BF16X3, o->info,
+                      st));
   } else {
     k_solve_m<<<(H->C + kPerCta - 1) / kPerCta, 32 * kPerCta, 0, st>>>(
-        w.Uh, ps, Q, H->M, H->Mp, H->n, H->C, H->mlam, H->mW, H->cband, nb, aidx, na, al, H->s2, o->ra,
-        1.0 / ((double)H->n * H->n), w.Zs, fused ? 0 : 1);
+        w.Uh, w.su, Q, H->M, H->Mp, H->n, H->C, H->mlam, H->mW, H->cband, nb, aidx, na, al, H->s2, o->ra,
+        1.0 / ((double)H->n * H->n), w.Zs, w.sz);
     FR3D_CUDA_TRY(cudaGetLastError());
   }
   prof_mark(H, kStColSolve, st);
@@ -640,14 +662,15 @@ int invert_multi(Handle* H, const float* U, int Q, const fr3d_invert_opts* o, fl
     H->last_launches = launches + 2;
     return FR3D_OK;
   }
-  // other sizes: the inverse column pass in place, then the row pass with the source combination (XI)
-  // or per source (ZETA); the solved spectra already carry 1/n^2
-  FR3D_TRY(Ops<float>::col_plain(H, w.Zs, w.Zs, Q * H->Mp, true, st));
+  // otherwise the inverse column pass (from bin order, or in place), then the row pass with the source combination
+  // (XI) or per source (ZETA); the solved spectra already carry 1/n^2
+  if (bins) FR3D_TRY(Ops<float>::col_from_bins(H, w.Zs, w.rows, Q * H->Mp, st));
+  else FR3D_TRY(Ops<float>::col_plain(H, w.Zs, w.Zs, Q * H->Mp, true, st));
   prof_mark(H, kStColInv, st);
   if (o->output == FR3D_OUT_XI)
-    FR3D_TRY(Ops<float>::row_c2r_xi(H, w.Zs, out, H->Mp, Q, 0, src, W, st));
+    FR3D_TRY(Ops<float>::row_c2r_xi(H, w.rows, out, H->Mp, Q, 0, src, W, st));
   else
-    FR3D_TRY(Ops<float>::row_c2r_plain(H, w.Zs, out, H->Mp * Q, Q, 0, H->Mp, st));
+    FR3D_TRY(Ops<float>::row_c2r_plain(H, w.rows, out, H->Mp * Q, Q, 0, H->Mp, st));
   prof_mark(H, kStRowC2R, st);
   H->last_launches = launches + 3;
   return FR3D_OK;
@@ -660,8 +683,17 @@ int choose_multi(Handle* H, const float* U, int Q, const double* alphas, int na,
   FR3D_TRY(ensure_bands(H, 1, nullptr));
   const bool tcp = tc_precision(precision);
   if (tcp) FR3D_TRY(ensure_tc_tables(H, 0, st));
-  MultiWs w;
-  FR3D_TRY(multi_ws(H, Q, false, &w));
+  // bin order needs a second part for the planes of the row pass; plane order where there is no room for it
+  bool bins = multi_bins(H);
+  int rc = ensure_ws(H, multi_layout(H, Q, bins, bins, nullptr).total);
+  if (rc == FR3D_ERR_OOM && bins) {
+    cudaGetLastError();
+    H->no_bins = true;
+    bins = false;
+    rc = ensure_ws(H, multi_layout(H, Q, false, false, nullptr).total);
+  }
+  FR3D_TRY(rc);
+  const MultiWs w = multi_layout(H, Q, bins, bins, (char*)H->ws);
   int launches = 0;
   prof_begin(H, st);
   if (tcp && info) {

@@ -21,6 +21,9 @@ template <typename T> struct Ops {
   static int row_r2c(const Handle* H, const T* in, long in_ps, C* out, int nplanes, cudaStream_t st);
   // column pass in place/out of place, plain
   static int col_plain(const Handle* H, const C* in, C* out, int nplanes, bool inverse, cudaStream_t st);
+  // column passes between plane order and bin order (out of place): forward, planes -> [bin][nplanes]; inverse, back
+  static int col_to_bins(const Handle* H, const C* planes, C* bins, int nplanes, cudaStream_t st);
+  static int col_from_bins(const Handle* H, const C* bins, C* planes, int nplanes, cudaStream_t st);
   // inverse column pass with the M = 1 Tikhonov weights; output planes jc * Q + q, jc < nj
   static int col_solve1(const Handle* H, const C* Uh, C* out, const T* A, const T* D, const int* aidx, int nb,
                         int Q, int j0, int nj, cudaStream_t st);
@@ -91,11 +94,12 @@ int learned_alpha(Handle* H, const float2* Uh, int nplanes, int nb, double delta
 // several observation depths (multi.cu): eigen tables of every class, the inversion and the alpha
 // choice, and the workspace bytes the inversion lays out from the start of the handle's workspace
 int ensure_multi_tables(Handle* H, cudaStream_t st);
-size_t multi_ws_bytes(const Handle* H, int Q);
+bool multi_bins(const Handle* H);   // the spectra in bin order where there is room
+size_t multi_ws_bytes(const Handle* H, int Q, bool bins);
 // src, W: the point sources and the combination weights (XI output; W may be null at sizes without the fused
 // inverse: V0 is then evaluated per voxel)
 int invert_multi(Handle* H, const float* U, int Q, const fr3d_invert_opts* o, float* out, const SrcHost& src,
-                 const float* W, cudaStream_t st);
+                 const float* W, bool bins, cudaStream_t st);
 int choose_multi(Handle* H, const float* U, int Q, const double* alphas, int na, double delta, double tau,
                  int precision, int* aidx, double* residuals, int* info, cudaStream_t st);
 void band_thresholds(const Handle* H, const fr3d_invert_opts* o, int nb, double* thr2);
@@ -103,14 +107,19 @@ void band_thresholds(const Handle* H, const fr3d_invert_opts* o, int nb, double*
 int inv_fused_presolved_f32(const Handle* H, const float2* Zs, const float* W, float* out, int Q, int output,
                             cudaStream_t st);
 
+// Where the value of (frequency bin, source q, component k) of a set of spectra lies: bin * b + q * q + k * k.
+// Plane order ([q][k] or [k][q] planes of bins) or bin order ([bin] records of Q K values).
+struct SpecStride {
+  long b, q, k;
+};
 // per-class dense products on the tensor cores (tc_contract.cu; M > 1, BF16 operands, FP32 accumulation;
 // split = the hi + lo form of FR3D_PREC_BF16X3)
 bool tc_precision(int precision);
 int tc_max_q();
 int ensure_tc_tables(Handle* H, int kind, cudaStream_t st);
-int tc_project(Handle* H, float2* Uh, int Q, double* Pc, bool split, int* info, cudaStream_t st);
-int tc_solve(Handle* H, const float2* P, int Q, const int* aidx, const double* alphas, int na, int ra, int nb,
-             float2* Zs, int jq, bool split, int* info, cudaStream_t st);
+int tc_project(Handle* H, float2* Uh, SpecStride sp, int Q, double* Pc, bool split, int* info, cudaStream_t st);
+int tc_solve(Handle* H, const float2* P, SpecStride sp, int Q, const int* aidx, const double* alphas, int na, int ra,
+             int nb, float2* Zs, SpecStride sz, bool split, int* info, cudaStream_t st);
 int tc_forward(Handle* H, const float2* Zh, float2* Uh, bool split, cudaStream_t st);
 
 // right-hand side of Eq. (7) (rhs.cu): the density sum_l 1/|x' - x_l| on the box Pi, and the combination

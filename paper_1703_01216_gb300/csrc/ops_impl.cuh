@@ -114,6 +114,35 @@ int Ops<T>::col_plain(const Handle* H, const C* in, C* out, int nplanes, bool in
   return FR3D_ERR_UNSUPPORTED_SIZE;
 }
 
+// the sizes of bin-ordered spectra (multi.cu)
+template <typename T, bool INV>
+static int col_bins(const Handle* H, const typename cpx<T>::t* in, typename cpx<T>::t* out, int nplanes, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    switch (H->n) {
+#define X(N)                                                                                                       \
+  case N: {                                                                                                        \
+    constexpr int PB = ColTile<float, N>::v;                                                                       \
+    constexpr size_t sm = col_smem<float, N, PB>();                                                                \
+    auto kern = k_col_bins<N, INV, PB>;                                                                            \
+    FR3D_TRY(set_smem(kern, sm));                                                                                  \
+    return launch_on(true, kern, dim3(N / 2 + 1, (nplanes + PB - 1) / PB), kThreads, sm, st, in, out, nplanes,     \
+                     tw_of<float>(H, N));                                                                          \
+  }
+      X(192) X(256) X(384) X(512)
+#undef X
+    }
+  }
+  return FR3D_ERR_UNSUPPORTED_SIZE;
+}
+template <typename T>
+int Ops<T>::col_to_bins(const Handle* H, const C* planes, C* bins, int nplanes, cudaStream_t st) {
+  return col_bins<T, false>(H, planes, bins, nplanes, st);
+}
+template <typename T>
+int Ops<T>::col_from_bins(const Handle* H, const C* bins, C* planes, int nplanes, cudaStream_t st) {
+  return col_bins<T, true>(H, bins, planes, nplanes, st);
+}
+
 template <typename T>
 int Ops<T>::col_solve1(const Handle* H, const C* Uh, C* out, const T* A, const T* D, const int* aidx, int nb, int Q,
                        int j0, int nj, cudaStream_t st) {

@@ -46,10 +46,9 @@ struct TcArgs {
   int Kc;               // 8-column chunks of the contraction index in a table row group
   int R, K;             // output rows per column and contraction length (<= 64 each)
   int C, n, Q;
-  long ps;              // half-spectrum plane stride (bins)
-  const float2* in;     // right-hand-side planes, plane q * K + k
-  float2* out;          // output planes, q * R + r (jq = 0) or r * Q + q (jq = 1)
-  int jq;
+  const float2* in;     // right-hand sides, value (bin, q, k) at the strides si
+  float2* out;          // outputs, value (bin, q, r) at the strides so
+  SpecStride si, so;
   int scale;            // TcScale
   float cscale;         // kScaleConst factor
   const double* lam;    // kScaleSolve: [C][K] eigenvalues
@@ -225,7 +224,7 @@ __global__ void __launch_bounds__(kTcCtaThreads) k_tc_contract(TcArgs a, TcAlpha
         for (int u = 0; u < 8; ++u) {
           const int k = 8 * kc + u;
           const bool ok = live && k < a.K;
-          v[u] = ok ? __ldg(a.in + ((long)q * a.K + k) * a.ps + bin) : make_float2(0.f, 0.f);
+          v[u] = ok ? __ldg(a.in + bin * a.si.b + q * a.si.q + k * a.si.k) : make_float2(0.f, 0.f);
           lv[u] = (ok && a.scale == kScaleSolve) ? __ldg(a.lam + (long)c * a.K + k) : 0.0;
         }
         double t = 0.0;
@@ -321,8 +320,7 @@ __global__ void __launch_bounds__(kTcCtaThreads) k_tc_contract(TcArgs a, TcAlpha
           if (c >= 0 && r < a.R) {
             for (int m = 0; m < I.nm[s]; ++m) {
               const float2 y = make_float2(v[2 * m], v[2 * m + 1]);
-              const long plane = a.jq ? (long)r * a.Q + q : (long)q * a.R + r;
-              a.out[plane * a.ps + I.bin[s][m]] = y;
+              a.out[I.bin[s][m] * a.so.b + q * a.so.q + r * a.so.k] = y;
               pw = fmaf(I.wt[s][m], y.x * y.x + y.y * y.y, pw);
             }
           }
@@ -460,7 +458,6 @@ TcArgs base_args(const Handle* H, int kind, bool split, int Q) {
   a.C = H->C;
   a.n = H->n;
   a.Q = Q;
-  a.ps = (long)(H->n / 2 + 1) * H->n;
   a.inv_n2 = (float)(1.0 / ((double)H->n * H->n));
   return a;
 }
@@ -469,30 +466,32 @@ TcArgs base_args(const Handle* H, int kind, bool split, int Q) {
 
 int tc_max_q() { return 16; }
 
-// p = U_c^T U~ in place in Uh [q][i] planes, class powers to Pc [C][M]
-int tc_project(Handle* H, float2* Uh, int Q, double* Pc, bool split, int* info, cudaStream_t st) {
+// p = U_c^T U~ in place in Uh (strides sp), class powers to Pc [C][M]
+int tc_project(Handle* H, float2* Uh, SpecStride sp, int Q, double* Pc, bool split, int* info, cudaStream_t st) {
   FR3D_TRY(ensure_tc_tables(H, 0, st));
   TcArgs a = base_args(H, 0, split, Q);
   a.R = H->M;
   a.K = H->M;
   a.in = Uh;
   a.out = Uh;
+  a.si = a.so = sp;
   a.scale = kScaleNone;
   a.Pc = Pc;
   a.info = info;
   return tc_run(a, TcAlphas{}, split, st);
 }
 
-// zeta~_j = sum_i W_c[i][j] g_i p_i / n^2 into Zs ([q][j] planes, or [j][q] when jq)
-int tc_solve(Handle* H, const float2* P, int Q, const int* aidx, const double* alphas, int na, int ra, int nb,
-             float2* Zs, int jq, bool split, int* info, cudaStream_t st) {
+// zeta~_j = sum_i W_c[i][j] g_i p_i / n^2 from P (strides sp) into Zs (strides sz)
+int tc_solve(Handle* H, const float2* P, SpecStride sp, int Q, const int* aidx, const double* alphas, int na, int ra,
+             int nb, float2* Zs, SpecStride sz, bool split, int* info, cudaStream_t st) {
   FR3D_TRY(ensure_tc_tables(H, 1, st));
   TcArgs a = base_args(H, 1, split, Q);
   a.R = H->Mp;
   a.K = H->M;
   a.in = P;
   a.out = Zs;
-  a.jq = jq;
+  a.si = sp;
+  a.so = sz;
   a.scale = kScaleSolve;
   a.lam = H->mlam;
   a.cband = H->cband;
@@ -515,6 +514,7 @@ int tc_forward(Handle* H, const float2* Zh, float2* Uh, bool split, cudaStream_t
   a.K = H->Mp;
   a.in = Zh;
   a.out = Uh;
+  a.si = a.so = SpecStride{1, 0, (long)(H->n / 2 + 1) * H->n};
   a.scale = kScaleConst;
   a.cscale = a.inv_n2;
   return tc_run(a, TcAlphas{}, split, st);
