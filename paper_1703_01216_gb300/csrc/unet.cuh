@@ -32,10 +32,9 @@ struct ConvArgs {
   int ngroups, nd, nchunks, stages, slog;   // set by conv3_launch (slog: log2 of the accumulator slots)
 };
 
-constexpr int kWgVox = 64;     // voxels (K) of a weight-gradient stage
+constexpr int kWgVox = 128;    // voxels (K) of a weight-gradient stage
 constexpr int kWgChain = 4096; // voxels at most that one FP32 accumulator of the weight gradient adds up
-// floats of one row of a weight-gradient partial: 27 / 3 taps x Cg input channels, the bias sum, padding
-__host__ __device__ constexpr int wgrad_row_floats(int Cg) { return 9 * Cg + 4; }
+constexpr int kWgCg = 16;      // input channels of a weight-gradient CTA
 
 // Weight gradient: partial sums per unit (sample, span of in-plane positions, depth chunk) and pair of
 // channel groups, then their ordered sum.
@@ -47,9 +46,10 @@ struct WgradArgs {
   int B, D, Wp;
   long HW, Vs, zero_pos;       // zero_pos: first voxel of the planes' zero guard
   int q_first, q_last;         // interior positions of a plane (with the halo between them)
-  float* partials;             // [units][pairs][3 Og][wgrad_row_floats(Cg)]
+  float* partials;             // [units][pairs][3 Og][9 kWgCg], then the bias sums [units][Cout]
   int* err;
-  int Og, Cg, n_og, n_cg, span, nspans, nd, nchunks, stages;   // wgrad_plan
+  int Og, n_og, n_cg, span, nspans, nd, nchunks, slots, gslots;   // wgrad_plan
+  float* bias_partials;        // set by wgrad3_launch
 };
 
 int conv_tiles(int q_first, int q_last);

@@ -26,10 +26,9 @@
 // Weight-gradient kernel (k_wgrad3): dW[tap][o][c] = sum_p G[p][o] X[p + s(tap)][c], a GEMM whose K is the
 // voxels: both operands come straight from CP planes, which hold 8 channels per 16 bytes, i.e. they are
 // MN-major operands (the instruction descriptor's transpose bits).  The rows stack the three f taps (the
-// output gradient shifted by one voxel) of Og <= 32 output channels, the columns the three e taps of Cg <= 48
-// input channels; the three a taps are three accumulators fed from the input planes d - 1, d, d + 1 of a ring,
-// so a plane sweep loads every input window once instead of once per a, and one CTA covers all 27 taps.  16
-// columns of ones behind the a = 1 windows make the bias gradient in the same MMAs.
+// output gradient shifted by one voxel) of Og <= 32 output channels, the columns the three a and three e taps of
+// 16 input channels; the a taps are the input planes d - 1, d, d + 1 of a ring, so a plane sweep loads every
+// input window once instead of once per a, and one CTA covers all 27 taps with one MMA per 16 voxels.
 #include <math.h>
 
 #include <algorithm>
@@ -71,12 +70,6 @@ __device__ __forceinline__ float lo16(uint32_t u) { return __uint_as_float(u << 
 __device__ __forceinline__ float hi16(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 
 __device__ __forceinline__ int flag(const int* f) { return *reinterpret_cast<const volatile int*>(f); }
-
-__host__ __device__ __forceinline__ uint32_t tmem_cols(int n) {
-  uint32_t c = 32;
-  while ((int)c < n) c <<= 1;
-  return c;
-}
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(bar)) : "memory");
@@ -348,31 +341,38 @@ __global__ void __launch_bounds__(PIPES* kPipeThreads, 1) k_conv3(ConvArgs a) {
 }
 
 // ------------------------------------------------------------------------------------------ k_wgrad3
-constexpr int kWgMaxStages = 8;
-constexpr int kWgThreads = 192;                 // warps 0-3 epilogue, 4 producer, 5 MMA
+constexpr int kWgMaxSlots = 16;                 // ring slots at most
+constexpr int kWgThreads = 192;                 // warps 0-3 bias sums and epilogue, 4 producer, 5 MMA
 constexpr int kWgPlane = kWgVox * 16;           // bytes of one window: kWgVox voxels of one channel chunk
+constexpr int kWgX = 3 * kWgCg / 8;             // input windows of a plane: [e][two chunks]
+static_assert(kWgCg == 16, "an input group is two chunks");
+constexpr int kWgCols = 9 * kWgCg;              // accumulator columns: [a][e][c]
+constexpr uint32_t kWgTmem = 256;
 
 // One CTA: the partial sums of one unit (sample, span of in-plane positions, depth chunk) for one pair of
-// channel groups.  A span is walked in sub-ranges of kWgVox positions, each swept through the depth.  Stage k
-// of a sweep holds the input plane g0 - 1 + k (three e windows per chunk, then 16 columns of ones) and, from
-// k = 2 on, the gradient plane g0 - 2 + k (three f windows per chunk): the MMAs of step k multiply that gradient
-// plane with the input planes of stages k - 2 (a = 0), k - 1 (a = 1, with the ones) and k (a = 2).  The 16 row
-// groups of an MMA reach past the 3 Og gradient rows into whatever lies behind them in shared memory: those
-// rows' accumulators are never read.
-// Bound (16 -> 16 channels at level 0): 12 window copies of 1 KB per 64 voxels from L2, and 3 x (4 KB + 1.5 KB)
-// of operand reads per 16 voxels, against 9 x 8 copies and 9 x 4.5 KB with one CTA per (a, e): 764 -> 223 us at
-// 128^2 x 32, batch 8, and the reduction, which used one thread per element, 224 -> 42 us.
+// channel groups.  A span is walked in sub-ranges of kWgVox positions, each swept through the depth.  Step k
+// of a sweep loads the input plane g0 - 1 + k (three e windows per chunk) and, from k = 2 on, the gradient plane
+// g0 - 2 + k (three f windows per chunk) and multiplies that gradient plane with the input planes of steps
+// k - 2, k - 1 and k: the taps a = 0, 1, 2.  The input planes lie in a ring of their own, so the three are
+// adjacent and one MMA of N = 144 columns takes them all (two where the ring wraps: 2 steps in 9 or 14).  The
+// idle epilogue warps add the bias gradient from the gradient windows meanwhile.  48 gradient rows (Og = 16) run
+// with M = 64, which reads half of the A operand; with M = 128 the rows past 3 Og are whatever lies behind them
+// in shared memory (the input ring follows) and their accumulators are never read.
+// Bound (16 -> 16 channels at 128^2 x 32, batch 8): the window copies, 57 cycles per KB and 83 per 2 KB and SM, hence
+// windows of 128 voxels (64: 173 us, 128: 122), then issue and operand reads of the MMAs, 2 KB + 4.5 KB per 16 voxels.
+// With windows of 64 voxels copied by a lane each and one MMA per a, of 48 to 160 columns: 225 us, and 568 us for
+// 48 -> 16 channels, now 322.
 __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
   extern __shared__ __align__(128) unsigned char sm[];
-  __shared__ __align__(8) uint64_t full[kWgMaxStages], empty[kWgMaxStages], done;
+  __shared__ __align__(8) uint64_t full[kWgMaxSlots], xempty[kWgMaxSlots], gempty[kWgMaxSlots], done;
   __shared__ uint32_t tbase;
   __shared__ int sabort, issued;
+  __shared__ float sb[4][32];
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-  const int S = a.stages;
-  const int nG = 3 * a.Og / 8, nX = 3 * a.Cg / 8;
-  const int stage = (nG + nX + 2) * kWgPlane;
-  const int N = 3 * a.Cg;
-  const uint32_t ncols = tmem_cols(3 * N + 16);
+  const int S = a.slots, SG = a.gslots;
+  const int gc = a.Og / 8, nG = 3 * gc;
+  const int gbytes = nG * kWgPlane;
+  unsigned char* xring = sm + SG * gbytes;
   const int npairs = a.n_og * a.n_cg;
   const int pair = blockIdx.x % npairs, unit = blockIdx.x / npairs;
   const int og = pair / a.n_cg, cg = pair - og * a.n_cg;
@@ -380,63 +380,66 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
   const int b = rest / a.nspans, sp = rest - b * a.nspans;
   const int g0 = 1 + ch * a.nd, cnt = min(a.nd, a.D + 1 - g0);
   const int v0 = a.q_first + sp * a.span, v1 = min(v0 + a.span, a.q_last + 1);   // in-plane positions [v0, v1)
-  // zeros everywhere once (the row groups past the gradient's), ones behind every stage's input windows
-  for (int e = tid; e < (S * stage + 2 * kWgPlane) / 16; e += kWgThreads) {
-    const int o = e * 16;
-    const uint32_t w = o < S * stage && o % stage >= (nG + nX) * kWgPlane ? 0x3F803F80u : 0u;
-    reinterpret_cast<uint4*>(sm)[e] = make_uint4(w, w, w, w);
-  }
-  tc::fence_proxy_async();
+  const bool bias = cg == 0;
   if (tid == 0) {
+    const uint32_t readers = bias ? 5 : 1;   // the MMA warp's commit, and the four bias warps
     for (int s = 0; s < S; ++s) {
       tc::mbar_init(&full[s], 1);
-      tc::mbar_init(&empty[s], 1);
+      tc::mbar_init(&xempty[s], readers);
     }
+    for (int s = 0; s < SG; ++s) tc::mbar_init(&gempty[s], readers);
     tc::mbar_init(&done, 1);
     tc::mbar_fence_init();
     sabort = 0;
     issued = 0;
   }
-  if (warp == 0) tc::tmem_alloc(&tbase, ncols);
+  if (warp == 0) tc::tmem_alloc(&tbase, kWgTmem);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tbase;
   if (warp == 4) {
-    // producer warp: lane 0 waits for the stage and posts its byte count, then each lane copies one window
-    // (the last K step of a span may end past it: the gradient's tail comes from the plane's zero guard)
-    const bool isg = lane < nG;
-    const int j = isg ? lane : lane - nG;
-    const int gc = (isg ? a.Og : a.Cg) / 8, t3 = j / gc, cc = j - t3 * gc;   // f or e, chunk in the group
-    const unsigned char* src = isg ? a.g + ((long)b * a.g_chunks + a.g_off + og * gc + cc) * a.Vs * 16
-                                   : a.x + ((long)b * a.x_chunks + a.x_off + cg * gc + cc) * a.Vs * 16;
-    const long shift = isg ? -(t3 - 1) : (long)(t3 - 1) * a.Wp;
-    int s = 0, use = 0, stop = 0;
-    for (int v = v0; v < v1 && !stop; v += kWgVox) {
+    // Producer warp.  Like the MMA warp it keeps every value the same in all lanes and lets one elected lane issue: the
+    // copy takes its operands from uniform registers, and a copy per lane is issued lane by lane (1 KB a lane: 77
+    // cycles per copy and SM; 16 -> 16 channels with the 2 KB windows: 135 instead of 122 us).
+    const unsigned char* gsrc = a.g + ((long)b * a.g_chunks + a.g_off + og * gc) * a.Vs * 16;
+    const unsigned char* xsrc = a.x + ((long)b * a.x_chunks + a.x_off + cg * (kWgCg / 8)) * a.Vs * 16;
+    int s = 0, use = 0, sg = 0, guse = 0;
+    bool ok = true;
+    for (int v = v0; v < v1 && ok; v += kWgVox) {
       const int rem = min(kWgVox, v1 - v), kv = (rem + 15) & ~15;
       for (int k = 0; k < cnt + 2; ++k) {
-        if (lane == 0) {
-          stop = flag(&sabort);
-          if (!stop && use > 0 && !tc::mbar_wait_sleep(&empty[s], (uint32_t)((use - 1) & 1), kPolls, kSleepNs)) {
-            sabort = 1;
-            stop = 1;
-          }
-          if (!stop) {
-            tc::mbar_arrive_expect_tx(&full[s], (uint32_t)((nX + (k >= 2 ? nG : 0)) * kv * 16));
-            ++issued;
+        ok = !flag(&sabort);
+        if (ok && use > 0) ok = tc::mbar_wait_sleep(&xempty[s], (uint32_t)((use - 1) & 1), kPolls, kSleepNs);
+        if (ok && k >= 2 && guse > 0) ok = tc::mbar_wait_sleep(&gempty[sg], (uint32_t)((guse - 1) & 1), kPolls, kSleepNs);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (tc::elect_one()) {
+          tc::mbar_arrive_expect_tx(&full[s], (uint32_t)((kWgX + (k >= 2 ? nG : 0)) * kv * 16));
+          ++issued;
+          const unsigned char* xs = xsrc + ((long)(g0 - 1 + k) * a.HW + v) * 16;
+          unsigned char* xd = xring + s * (kWgX * kWgPlane);
+#pragma unroll
+          for (int j = 0; j < kWgX; ++j)
+            tc::bulk_g2s(xd + j * kWgPlane, xs + ((j & 1) * a.Vs + ((j >> 1) - 1) * a.Wp) * 16, (uint32_t)(kv * 16), &full[s]);
+          if (k >= 2) {
+            // (the last K step of a span may end past it: the gradient's tail comes from the plane's zero guard)
+            const unsigned char* gs = gsrc + ((long)(g0 - 2 + k) * a.HW + v) * 16;
+            unsigned char* gd = sm + sg * gbytes;
+            for (int c = 0; c < gc; ++c) {
+#pragma unroll
+              for (int f = 0; f < 3; ++f) {
+                unsigned char* dst = gd + (f * gc + c) * kWgPlane;
+                tc::bulk_g2s(dst, gs + (c * a.Vs - (f - 1)) * 16, (uint32_t)(rem * 16), &full[s]);
+                if (kv > rem) tc::bulk_g2s(dst + rem * 16, gsrc + a.zero_pos * 16, (uint32_t)((kv - rem) * 16), &full[s]);
+              }
+            }
           }
         }
-        stop = __shfl_sync(0xffffffffu, stop, 0);
-        __syncwarp();   // the byte count is posted before any copy of the stage is issued
-        if (stop) break;
-        unsigned char* dst = sm + s * stage + lane * kWgPlane;
-        if (isg) {
-          if (k >= 2) {
-            tc::bulk_g2s(dst, src + ((long)(g0 - 2 + k) * a.HW + v + shift) * 16, (uint32_t)(rem * 16), &full[s]);
-            if (kv > rem) tc::bulk_g2s(dst + rem * 16, src + a.zero_pos * 16, (uint32_t)((kv - rem) * 16), &full[s]);
-          }
-        } else if (lane < nG + nX) {
-          tc::bulk_g2s(dst, src + ((long)(g0 - 1 + k) * a.HW + v + shift) * 16, (uint32_t)(kv * 16), &full[s]);
+        __syncwarp();
+        if (k >= 2 && ++sg == SG) {
+          sg = 0;
+          ++guse;
         }
         if (++s == S) {
           s = 0;
@@ -444,12 +447,13 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
         }
       }
     }
+    if (!ok) sabort = 1;
   } else if (warp == 5) {
     // MMA warp: uniform values, one elected lane issues (as in k_conv3)
-    const uint32_t idn = idesc_mn(128, N), id1 = idesc_mn(128, N + 16);
+    const int M = nG * 8 <= 64 ? 64 : 128;
     const uint64_t dh = desc_mn(0, kWgPlane, 128);
-    const uint32_t d0 = tc::smem_addr(sm) >> 4, xoff = nG * kWgPlane / 16, st16 = stage / 16;
-    int s = 0, ph = 0;
+    const uint32_t dg0 = tc::smem_addr(sm) >> 4, dx0 = tc::smem_addr(xring) >> 4;
+    int s = 0, ph = 0, sg = 0;
     bool ok = true, acc = false;
     for (int v = v0; v < v1 && ok; v += kWgVox) {
       const int ks = (min(kWgVox, v1 - v) + 15) / 16;
@@ -459,24 +463,27 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
         if (k >= 2) {
           tc::fence_after_sync();
           const int s1 = s >= 1 ? s - 1 : s - 1 + S, s2 = s >= 2 ? s - 2 : s - 2 + S;
-          const uint32_t da = d0 + s * st16;
-          const uint32_t x0 = d0 + s2 * st16 + xoff, x1 = d0 + s1 * st16 + xoff, x2 = da + xoff;
+          const int m0 = min(3, S - s2);   // planes of the first run; the rest start over at slot 0
+          const uint32_t da = dg0 + sg * (gbytes / 16), db0 = dx0 + s2 * (kWgX * kWgPlane / 16);
+          const uint32_t i0 = idesc_mn(M, m0 * 3 * kWgCg), i1 = idesc_mn(M, (3 - m0) * 3 * kWgCg);
+          const uint32_t c1 = tmem + m0 * 3 * kWgCg;
           if (tc::elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < kWgVox / 16; ++kk)
               if (kk < ks) {
-                tc::mma_bf16(tmem, dh | (da + 16 * kk), dh | (x0 + 16 * kk), idn, acc || kk > 0);
-                tc::mma_bf16(tmem + N, dh | (da + 16 * kk), dh | (x2 + 16 * kk), idn, acc || kk > 0);
-                tc::mma_bf16(tmem + 2 * N, dh | (da + 16 * kk), dh | (x1 + 16 * kk), id1, acc || kk > 0);
+                tc::mma_bf16(tmem, dh | (da + 16 * kk), dh | (db0 + 16 * kk), i0, acc || kk > 0);
+                if (m0 < 3) tc::mma_bf16(c1, dh | (da + 16 * kk), dh | (dx0 + 16 * kk), i1, acc || kk > 0);
               }
-            tc::mma_commit(&empty[s2]);
+            tc::mma_commit(&gempty[sg]);
+            tc::mma_commit(&xempty[s2]);
             if (k == cnt + 1) {
-              tc::mma_commit(&empty[s1]);
-              tc::mma_commit(&empty[s]);
+              tc::mma_commit(&xempty[s1]);
+              tc::mma_commit(&xempty[s]);
             }
           }
           acc = true;
           __syncwarp();
+          if (++sg == SG) sg = 0;
         }
         if (++s == S) {
           s = 0;
@@ -488,24 +495,71 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
     if (tc::elect_one()) tc::mma_commit(&done);
     __syncwarp();
   } else {
-    // epilogue: row tid = (f, o); columns [a = 0 | 2 | 1][e][c], then the ones
+    if (bias) {
+      // bias gradient: every thread adds its voxels of the unshifted (f = 1) windows
+      float acc[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) acc[k] = 0.f;
+      int s = 0, ph = 0, sg = 0;
+      bool ok = true;
+      for (int v = v0; v < v1 && ok; v += kWgVox) {
+        const int rem = min(kWgVox, v1 - v);
+        for (int k = 0; k < cnt + 2; ++k) {
+          ok = __all_sync(0xffffffffu, tc::mbar_wait_sleep(&full[s], (uint32_t)ph, kPolls, kSleepNs));
+          if (!ok) break;
+          if (k >= 2) {
+            for (int vx = tid; vx < rem; vx += 128) {
+              const unsigned char* w = sm + sg * gbytes + gc * kWgPlane + vx * 16;
+#pragma unroll
+              for (int h = 0; h < 4; ++h)
+                if (h < gc) {
+                  const uint4 q = *reinterpret_cast<const uint4*>(w + h * kWgPlane);
+                  const uint32_t qw[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                  for (int i = 0; i < 4; ++i) {
+                    acc[8 * h + 2 * i] += lo16(qw[i]);
+                    acc[8 * h + 2 * i + 1] += hi16(qw[i]);
+                  }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&gempty[sg]);
+            if (++sg == SG) sg = 0;
+          }
+          if (lane == 0) mbar_arrive(&xempty[s]);
+          if (++s == S) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+      }
+      if (!ok) sabort = 1;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], m);
+        if (lane == i) sb[warp][i] = acc[i];
+      }
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (tid < a.Og)
+        a.bias_partials[(long)unit * a.Cout + og * a.Og + tid] = (sb[0][tid] + sb[1][tid]) + (sb[2][tid] + sb[3][tid]);
+    }
+    // epilogue: accumulator row (f, o) is lane tid, with M = 64 the first 16 lanes of each warp
     const bool got = tc::mbar_wait_sleep(&done, 0u, kPolls, kSleepNs);
     if (!__all_sync(0xffffffffu, got)) sabort = 1;
     tc::fence_after_sync();
     const uint32_t tw = tmem + ((uint32_t)(warp * 32) << 16);
-    const int rs = wgrad_row_floats(a.Cg);
-    float* dst = a.partials + ((long)blockIdx.x * 3 * a.Og + tid) * rs;
-    for (int n = 0; n < 3 * N; n += 16) {
+    const bool half = nG * 8 <= 64;
+    const int row = half ? (lane < 16 ? warp * 16 + lane : nG * 8) : tid;
+    float* dst = a.partials + ((long)blockIdx.x * nG * 8 + row) * kWgCols;
+    for (int n = 0; n < kWgCols; n += 16) {
       float v[16];
       tc::tmem_ld16(tw + n, v);
-      if (tid < 3 * a.Og)
+      if (row < nG * 8)
 #pragma unroll
         for (int k = 0; k < 16; k += 4)
           *reinterpret_cast<float4*>(dst + n + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
     }
-    float v[16];
-    tc::tmem_ld16(tw + 3 * N, v);
-    if (tid < 3 * a.Og) dst[3 * N] = v[0];
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -516,39 +570,54 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
   }
   __syncthreads();
   tc::fence_after_sync();
-  if (warp == 0) tc::tmem_dealloc(tmem, ncols);
+  if (warp == 0) tc::tmem_dealloc(tmem, kWgTmem);
 }
 
-// dW[o][c][tap] (c < ci) and db[o]: the units' partial sums added in FP64 in a fixed order (8 threads per
-// element take every eighth unit, then the eight sums in order).  Bound by the partials' bytes.
-constexpr int kWgRedX = 32, kWgRedY = 8;
-__global__ void __launch_bounds__(kWgRedX* kWgRedY) k_wgrad_reduce(WgradArgs a, int nunits, int ci, float* __restrict__ dW,
-                                                                  float* __restrict__ db) {
-  __shared__ double red[kWgRedY][kWgRedX];
-  const int rs = wgrad_row_floats(a.Cg), N = 3 * a.Cg;
-  const int per = 3 * a.Og * rs, npairs = a.n_og * a.n_cg;
-  const int i = blockIdx.x * kWgRedX + threadIdx.x;
+// dW[o][c][tap] (c < ci) and db[o]: the units' partial sums added in a fixed order (blockDim.y threads per element
+// take every blockDim.y-th unit, then their sums in order).  A thread adds in FP32 with the rounding errors carried
+// along (Knuth's two-sum; what is lost is of order 2^-48): the FP64 conversions and additions were the bound.
+// 29 MB of partials: 42 -> 22 us, 86 MB: 98 -> 58 us, with four times the loads in flight.  Sums that are not finite
+// are added again in FP64, as a chain that leaves FP32's range on the way has to be.
+constexpr int kWgRedThreads = 512;
+__global__ void __launch_bounds__(kWgRedThreads) k_wgrad_reduce(WgradArgs a, int nunits, int ci, float* __restrict__ dW,
+                                                               float* __restrict__ db) {
+  __shared__ double red[kWgRedThreads];
+  const int per = 3 * a.Og * kWgCols, npairs = a.n_og * a.n_cg, nw = per * npairs;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool ok = i < nw + a.Cout;
   double s = 0.0;
-  if (i < per * npairs) {
-    const float* p = a.partials + i;
-    const long ustep = (long)per * npairs;
+  if (ok) {
+    const float* p = i < nw ? a.partials + i : a.bias_partials + (i - nw);
+    const long ustep = i < nw ? nw : a.Cout;
+    float hi = 0.f, lo = 0.f;
 #pragma unroll 8
-    for (int u = threadIdx.y; u < nunits; u += kWgRedY) s += (double)__ldg(p + u * ustep);
+    for (int u = threadIdx.y; u < nunits; u += blockDim.y) {
+      const float x = __ldg(p + u * ustep), t = __fadd_rn(hi, x), d = __fsub_rn(t, hi);
+      lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, d)), __fsub_rn(x, d)));
+      hi = t;
+    }
+    s = (double)hi + (double)lo;
+    if (!isfinite(hi) || !isfinite(lo)) {
+      s = 0.0;
+      for (int u = threadIdx.y; u < nunits; u += blockDim.y) s += (double)__ldg(p + u * ustep);
+    }
   }
-  red[threadIdx.y][threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.y != 0 || i >= per * npairs) return;
-  for (int y = 1; y < kWgRedY; ++y) s += red[y][threadIdx.x];
-  const int pair = i / per, m = (i - pair * per) / rs, n = i % rs;
+  if (blockDim.y > 1) {
+    red[threadIdx.y * blockDim.x + threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y != 0) return;
+    for (unsigned y = 1; y < blockDim.y; ++y) s += red[y * blockDim.x + threadIdx.x];
+  }
+  if (!ok) return;
+  if (i >= nw) {
+    db[i - nw] = (float)s;
+    return;
+  }
+  const int pair = i / per, m = (i - pair * per) / kWgCols, n = i % kWgCols;
   const int og = pair / a.n_cg, cg = pair - og * a.n_cg;
   const int f = m / a.Og, o = og * a.Og + m % a.Og;
-  if (n < 3 * N) {
-    const int part = n / N, e = (n % N) / a.Cg, c = cg * a.Cg + n % a.Cg;
-    const int ta = part == 0 ? 0 : 3 - part;
-    if (c < ci) dW[((long)o * ci + c) * 27 + ta * 9 + e * 3 + f] = (float)s;
-  } else if (n == 3 * N && f == 1 && cg == 0) {
-    db[o] = (float)s;
-  }
+  const int ta = n / (3 * kWgCg), e = n / kWgCg - 3 * ta, c = cg * kWgCg + n % kWgCg;
+  if (c < ci) dW[((long)o * ci + c) * 27 + ta * 9 + e * 3 + f] = (float)s;
 }
 
 int sm_count(int* sms) {
@@ -644,34 +713,33 @@ int conv3_launch(const ConvArgs& args, cudaStream_t st) {
   }
 }
 
-// Channel groups and units of a layer's weight gradient for batches up to B (fills Og .. nchunks, stages).
+// Channel groups and units of a layer's weight gradient for batches up to B (fills Og .. nchunks, slots).
 // A unit's accumulators see at most kWgChain voxels, as many as one FP32 chain of the partial sums may have.
 int wgrad_plan(WgradArgs* a, int B) {
-  if (a->Cin % 16 || a->Cout % 16) return FR3D_ERR_UNSUPPORTED_SIZE;
+  if (a->Cin % kWgCg || a->Cout % 16) return FR3D_ERR_UNSUPPORTED_SIZE;
   a->Og = a->Cout % 32 == 0 ? 32 : 16;
-  a->Cg = a->Cin % 48 == 0 ? 48 : (a->Cin % 32 == 0 ? 32 : 16);
   a->n_og = a->Cout / a->Og;
-  a->n_cg = a->Cin / a->Cg;
+  a->n_cg = a->Cin / kWgCg;
   a->nd = std::min(a->D, kWgChain / kWgVox);
   a->nchunks = (a->D + a->nd - 1) / a->nd;
   a->nd = (a->D + a->nchunks - 1) / a->nchunks;
-  const int stage = (3 * a->Og / 8 + 3 * a->Cg / 8 + 2) * kWgPlane;
-  const bool two = tmem_cols(9 * a->Cg + 16) <= kTmemCols / 2;   // two CTAs per SM share the tensor memory
-  const size_t room = (two ? 112 * 1024 : kMaxSmem) - kSmemSlack - 2 * kWgPlane;
-  a->stages = (int)std::min<size_t>(kWgMaxStages, room / stage);
-  if (a->stages < 4) return FR3D_ERR_UNSUPPORTED_SIZE;
+  const size_t room = 112 * 1024 - kSmemSlack;   // two CTAs per SM, which also share the tensor memory
+  // about half of the room for each ring: the input ring holds two more planes than the steps in flight
+  const int gplane = 3 * a->Og / 8 * kWgPlane, xplane = kWgX * kWgPlane;
+  a->gslots = std::min<int>(kWgMaxSlots - 3, (int)((room - 3 * xplane) / (gplane + xplane)));
+  a->slots = std::min<int>(kWgMaxSlots, (int)((room - (size_t)a->gslots * gplane) / xplane));
   int sms = 0;
   FR3D_TRY(sm_count(&sms));
-  const int slots = (two ? 2 : 1) * sms;
+  const int slots = 2 * sms;
   const int len = a->q_last - a->q_first + 1, npairs = a->n_og * a->n_cg;
   double bc = 0;
   a->span = 0;
   for (int span = kWgVox; span * a->nd <= std::max(kWgChain, kWgVox * a->nd) && span < len + kWgVox; span += kWgVox) {
     const long units = (long)B * a->nchunks * ((len + span - 1) / span);
     const long rounds = (units * npairs + slots - 1) / slots;
-    // MMA and copy time of a unit against the bytes of the partials (written and read once), in cycles
-    const double c = (double)rounds * ((span / kWgVox) * (a->nd + 2) * 12.0 * (32 + 3 * a->Cg / 4) + 3000) +
-                     (double)units * npairs * 3 * a->Og * wgrad_row_floats(a->Cg) * 8 / 2500.0;
+    // steps of a unit (two CTAs share an SM) against the bytes of the partials (written and read once), in cycles
+    const double c = (double)rounds * ((span / kWgVox) * (a->nd + 2) * 12.5 * kWgVox + 4000) +
+                     (double)units * npairs * 3 * a->Og * kWgCols * 8 / 2500.0;
     if (!a->span || c < bc) {
       a->span = span;
       bc = c;
@@ -682,17 +750,20 @@ int wgrad_plan(WgradArgs* a, int B) {
 }
 
 size_t wgrad_partial_floats(const WgradArgs& a, int B) {
-  return (size_t)B * a.nspans * a.nchunks * a.n_og * a.n_cg * 3 * a.Og * wgrad_row_floats(a.Cg);
+  return (size_t)B * a.nspans * a.nchunks * ((size_t)a.n_og * a.n_cg * 3 * a.Og * kWgCols + a.Cout);
 }
 
-int wgrad3_launch(const WgradArgs& a, int ci, float* dW, float* db, cudaStream_t st) {
-  const int stage = (3 * a.Og / 8 + 3 * a.Cg / 8 + 2) * kWgPlane;
-  const size_t smem = (size_t)a.stages * stage + 2 * kWgPlane;
+int wgrad3_launch(const WgradArgs& args, int ci, float* dW, float* db, cudaStream_t st) {
+  WgradArgs a = args;
+  const size_t smem = ((size_t)a.gslots * (3 * a.Og / 8) + (size_t)a.slots * kWgX) * kWgPlane;
   FR3D_TRY(smem_optin(reinterpret_cast<const void*>(k_wgrad3), smem));
   const int units = a.B * a.nspans * a.nchunks, npairs = a.n_og * a.n_cg;
+  const int total = npairs * 3 * a.Og * kWgCols;
+  a.bias_partials = a.partials + (size_t)units * total;
   k_wgrad3<<<units * npairs, kWgThreads, smem, st>>>(a);
-  const int total = npairs * 3 * a.Og * wgrad_row_floats(a.Cg);
-  k_wgrad_reduce<<<(total + kWgRedX - 1) / kWgRedX, dim3(kWgRedX, kWgRedY), 0, st>>>(a, units, ci, dW, db);
+  // threads per element: about eight units each, so that the loads of a layer with few elements fill the chip
+  const int ry = units >= 512 ? 32 : (units >= 128 ? 16 : (units >= 32 ? 4 : 1)), rx = kWgRedThreads / ry;
+  k_wgrad_reduce<<<(total + a.Cout + rx - 1) / rx, dim3(rx, ry), 0, st>>>(a, units, ci, dW, db);
   FR3D_CUDA_TRY(cudaGetLastError());
   return FR3D_OK;
 }
