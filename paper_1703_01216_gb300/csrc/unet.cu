@@ -276,43 +276,21 @@ __global__ void k_pool_backward(const unsigned char* __restrict__ gp, int p_chun
   }
 }
 
-// head: y_s = x_s + b + sum_c w_c h_c (FP32), optional prediction y_s / s in the caller's units, and
-// per-block partial sums of (y_s - t_s)^2 and t_s^2 for each sample (when t is given)
+// per-block partial sums of (y_s - t_s)^2 and t_s^2 for each sample.  The predictions come from the last
+// convolution, which applies the head to its outputs while it holds them.
 constexpr int kHeadThreads = 256;
-__global__ void __launch_bounds__(kHeadThreads) k_head_forward(const unsigned char* __restrict__ Hd, LevelArg L,
-                                                               const float* __restrict__ x, const float* __restrict__ t,
-                                                               const float* __restrict__ wb, float s, int B,
-                                                               float* __restrict__ ys, float* __restrict__ out,
-                                                               float* __restrict__ part) {
+__global__ void __launch_bounds__(kHeadThreads) k_loss_partial(const float* __restrict__ ys, const float* __restrict__ t,
+                                                               unsigned nvox, float s, float* __restrict__ part) {
   __shared__ float red[2][kHeadThreads];
-  const unsigned nvox = (unsigned)(L.D * L.H * L.W);
   const int b = blockIdx.y;
-  float w[16];
-#pragma unroll
-  for (int c = 0; c < 16; ++c) w[c] = bf16r(wb[c]);
-  const float bias = wb[16];
   float e2 = 0.f, t2 = 0.f;
+#pragma unroll 4
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < nvox; i += gridDim.x * blockDim.x) {
-    const unsigned r = i / L.W;
-    const int ww = (int)(i - r * L.W), h = (int)(r % L.H), d = (int)(r / L.H);
-    const long p = ppos(L, d, h, ww);
-    float a[8], c2[8];
-    unpack8(*reinterpret_cast<const uint4*>(Hd + (((long)b * 2) * L.Vs + p) * 16), a);
-    unpack8(*reinterpret_cast<const uint4*>(Hd + (((long)b * 2 + 1) * L.Vs + p) * 16), c2);
-    float acc = bias;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) acc = fmaf(w[k], a[k], fmaf(w[8 + k], c2[k], acc));
     const long gi = (long)b * nvox + i;
-    const float y = bf16r(s * x[gi]) + acc;
-    ys[gi] = y;
-    if (out) out[gi] = y / s;
-    if (t) {
-      const float tv = s * t[gi];
-      e2 += (y - tv) * (y - tv);
-      t2 += tv * tv;
-    }
+    const float tv = s * t[gi], e = ys[gi] - tv;
+    e2 += e * e;
+    t2 += tv * tv;
   }
-  if (!part) return;
   red[0][threadIdx.x] = e2;
   red[1][threadIdx.x] = t2;
   __syncthreads();
@@ -498,7 +476,7 @@ ConvArgs conv_args(const Unet* U, int lvl, int B) {
   return a;
 }
 
-int conv_forward(Unet* U, int k, int B, cudaStream_t st) {
+ConvArgs conv_forward_args(const Unet* U, int k, int B) {
   const Layer& Ly = U->layer[k];
   ConvArgs a = conv_args(U, Ly.lvl, B);
   a.x = U->t[Ly.in_t];
@@ -513,8 +491,9 @@ int conv_forward(Unet* U, int k, int B, cudaStream_t st) {
   a.y_off = Ly.out_off / 8;
   a.bias = U->params + Ly.woff + (long)Ly.co * Ly.ci * 27;
   a.mode = kConvFwd;
-  return conv3_launch(a, st);
+  return a;
 }
+int conv_forward(const Unet* U, int k, int B, cudaStream_t st) { return conv3_launch(conv_forward_args(U, k, B), st); }
 
 int conv_backward(Unet* U, int k, int B, cudaStream_t st) {
   const Layer& Ly = U->layer[k];
@@ -548,6 +527,8 @@ int conv_backward(Unet* U, int k, int B, cudaStream_t st) {
   return FR3D_OK;
 }
 
+constexpr int kLossBlocks = 128;   // per sample
+
 int forward(Unet* U, const float* x, int B, const float* t, float* out, cudaStream_t st) {
   const Level& L0 = U->lv[0];
   dim3 blk = row_block(L0.W);
@@ -575,18 +556,27 @@ int forward(Unet* U, const float* x, int B, const float* t, float* out, cudaStre
     FR3D_CUDA_TRY(cudaGetLastError());
     const int k = 9 + 2 * (kL - 2 - l);
     FR3D_TRY(conv_forward(U, k, B, st));
-    FR3D_TRY(conv_forward(U, k + 1, B, st));
+    if (l > 0) FR3D_TRY(conv_forward(U, k + 1, B, st));
   }
-  const int nblk = 128;
-  k_head_forward<<<dim3(nblk, B), kHeadThreads, 0, st>>>(U->t[T_D2], larg(L0), x, t, U->params + U->head_off,
-                                                         U->in_scale, B, U->y, out, t ? U->red : nullptr);
+  // the last convolution with the head; its own output is kept for the gradient only
+  ConvArgs a = conv_forward_args(U, kNumConv - 1, B);
+  a.mode = kConvHead;
+  a.hx = x;
+  a.hw = U->params + U->head_off;
+  a.hs = U->in_scale;
+  a.hout = out;
+  if (t) a.hys = U->y;
+  else a.y = nullptr;
+  FR3D_TRY(conv3_launch(a, st));
+  if (t)
+    k_loss_partial<<<dim3(kLossBlocks, B), kHeadThreads, 0, st>>>(U->y, t, (unsigned)(L0.D * L0.H * L0.W), U->in_scale, U->red);
   FR3D_CUDA_TRY(cudaGetLastError());
   return FR3D_OK;
 }
 
 int backward(Unet* U, const float* t, int B, float* loss, cudaStream_t st) {
   const Level& L0 = U->lv[0];
-  const int nblk = 128;
+  const int nblk = kLossBlocks;
   k_loss<<<1, kLossThreads, 0, st>>>(U->red, nblk, B, U->lossbuf, loss);
   k_head_backward<<<dim3(nblk, B), kHeadThreads, 0, st>>>(U->t[T_D2], larg(L0), U->y, t, U->params + U->head_off,
                                                           U->in_scale, B, U->lossbuf, U->g[T_D2], U->red);

@@ -7,7 +7,7 @@ namespace fr3d {
 
 constexpr float kLeaky = 0.01f;   // slope of leaky ReLU for negative inputs
 
-enum ConvMode { kConvFwd = 0, kConvDgradMask = 1, kConvDgradPlain = 2 };
+enum ConvMode { kConvFwd = 0, kConvDgradMask = 1, kConvDgradPlain = 2, kConvHead = 3 };
 
 // One 3 x 3 x 3 convolution (or its input gradient) over CP tensors (see unet_conv.cu).  Tensors are
 // byte pointers to [B][chunks][Vs][8] BF16; x_off / y_off / mask_off select a channel-chunk range of a
@@ -18,11 +18,16 @@ struct ConvArgs {
   // [N / Ng groups][3 (e)][Cin / 16][3 (f)][3 (a = 2, 1, 0)][Ng / 8][2 chunks][8][8] BF16, K-major core matrices
   const unsigned char* wimg;
   int N, Ng;                   // output channels, and those of one CTA (conv_group)
-  unsigned char* y;
+  unsigned char* y;            // kConvHead: may be null (the output is not kept)
   int y_chunks, y_off;
-  const float* bias;           // kConvFwd: [N] (may be null)
+  const float* bias;           // kConvFwd, kConvHead: [N] (may be null)
   const unsigned char* mask;   // kConvDgradMask: the tensor whose leaky derivative multiplies the result
   int mask_chunks, mask_off;
+  // kConvHead (N = Ng = 16): the network's 1 x 1 x 1 head on the 16 outputs of a voxel: ys = bf16(s x) + w h + b
+  // (any of ys and out = ys / s may be null), x, ys and out [B][D][H][W]
+  const float *hx, *hw;        // input, head weights and bias [17]
+  float *hys, *hout;
+  float hs;
   int mode;
   int B, D, H, W, Wp;
   long HW, Vs;                 // voxels of a padded (h, w) plane, and of a padded volume with its guard

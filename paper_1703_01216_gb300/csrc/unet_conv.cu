@@ -98,14 +98,15 @@ struct ConvPipe {
   int issued;
 };
 
-template <int PIPES>
+// HEAD: mode kConvHead, an instance of its own (as a branch of the others' epilogue it slowed the input gradients by 7 %)
+template <int PIPES, bool HEAD>
 __global__ void __launch_bounds__(PIPES* kPipeThreads, 1) k_conv3(ConvArgs a) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ __align__(8) ConvPipe pipes[PIPES];
   __shared__ __align__(8) uint64_t wfull;
   __shared__ uint32_t tbase;
   __shared__ int sabort;
-  __shared__ float sbias[64];
+  __shared__ float sbias[64], shead[17];
   // warps [0, 4 PIPES): epilogue (pipe = warp / 4; warp % 4 picks the 32 TMEM lanes it may read), then the
   // producers, then the MMA warps
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(PIPES* kPipeThreads, 1) k_conv3(ConvArgs a) {
     tc::mbar_fence_init();
   }
   if (tid < Ng) sbias[tid] = a.bias ? a.bias[grp * Ng + tid] : 0.f;
+  if (HEAD && tid < 17) shead[tid] = tid < 16 ? tc::bf16_val(tc::bf16_rn(a.hw[tid])) : a.hw[16];
   if (warp == 0) tc::tmem_alloc(&tbase, kTmemCols);
   tc::fence_before_sync();
   __syncthreads();
@@ -290,7 +292,7 @@ __global__ void __launch_bounds__(PIPES* kPipeThreads, 1) k_conv3(ConvArgs a) {
           }
           if (valid) {
             const long jc = (long)grp * (Ng / 8) + j;
-            if (a.mode == kConvFwd) {
+            if (HEAD || a.mode == kConvFwd) {
 #pragma unroll
               for (int k = 0; k < 16; ++k) {
                 const float z = v[k] + sbias[8 * j + k];
@@ -316,8 +318,19 @@ __global__ void __launch_bounds__(PIPES* kPipeThreads, 1) k_conv3(ConvArgs a) {
                 }
               }
             }
+            if constexpr (HEAD) {
+              // the head multiplies the stored (rounded) outputs, in the order of channel pairs (k, 8 + k)
+              const long gi = (((long)c.b * a.D + c.o0 + r - 1) * a.H + hh - 1) * a.W + ww - 1;
+              float h = shead[16];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+              for (int k = 0; k < 8; ++k)
+                h = fmaf(shead[k], tc::bf16_val(tc::bf16_rn(v[k])), fmaf(shead[8 + k], tc::bf16_val(tc::bf16_rn(v[8 + k])), h));
+              const float y = tc::bf16_val(tc::bf16_rn(a.hs * __ldg(a.hx + gi))) + h;
+              if (a.hys) a.hys[gi] = y;
+              if (a.hout) a.hout[gi] = y / a.hs;
+            }
+#pragma unroll
+            for (int h = 0; h < 2 && (!HEAD || a.y); ++h) {
               uint4 o;
               o.x = pack2(v[8 * h], v[8 * h + 1]);
               o.y = pack2(v[8 * h + 2], v[8 * h + 3]);
@@ -679,11 +692,11 @@ ConvPlan conv_plan(int Cin, int N, int D, int ntiles, int B, int ng, int sms) {
   return best;
 }
 
-template <int PIPES> int conv3_launch_t(const ConvArgs& a, int ctas, cudaStream_t st) {
+template <int PIPES, bool HEAD> int conv3_launch_t(const ConvArgs& a, int ctas, cudaStream_t st) {
   // all of the SM's tensor memory is one CTA's: ask for more than half of its shared memory
   const size_t smem = std::max(conv_weight_bytes(a.Cin, a.Ng) + (size_t)PIPES * a.stages * kConvStageBytes, (size_t)120 * 1024);
-  FR3D_TRY(smem_optin(reinterpret_cast<const void*>(k_conv3<PIPES>), smem));
-  k_conv3<PIPES><<<ctas, PIPES * kPipeThreads, smem, st>>>(a);
+  FR3D_TRY(smem_optin(reinterpret_cast<const void*>(k_conv3<PIPES, HEAD>), smem));
+  k_conv3<PIPES, HEAD><<<ctas, PIPES * kPipeThreads, smem, st>>>(a);
   FR3D_CUDA_TRY(cudaGetLastError());
   return FR3D_OK;
 }
@@ -701,6 +714,7 @@ int conv_group(int Cin, int N, int D, int ntiles, int B) {
 int conv3_launch(const ConvArgs& args, cudaStream_t st) {
   ConvArgs a = args;
   if (a.Cin % 16 || a.Ng % 16 || a.Ng < 16 || a.Ng > 64 || a.N % a.Ng) return FR3D_ERR_UNSUPPORTED_SIZE;
+  if (a.mode == kConvHead && (a.N != 16 || !a.hx || !a.hw)) return FR3D_ERR_UNSUPPORTED_SIZE;
   int sms = 0;
   FR3D_TRY(sm_count(&sms));
   const ConvPlan p = conv_plan(a.Cin, a.N, a.D, a.ntiles, a.B, a.Ng, sms);
@@ -713,10 +727,12 @@ int conv3_launch(const ConvArgs& args, cudaStream_t st) {
   while ((2 << a.slog) * a.Ng <= kTmemCols / p.pipes) ++a.slog;   // slots of a pipe's ring: a power of two
   const long units = (long)a.B * a.ntiles * a.nchunks;
   const long ctas = std::max<long>(1, std::min<long>(units, sms / a.ngroups));
+  const int nc = (int)ctas * a.ngroups;
+  const bool head = a.mode == kConvHead;
   switch (p.pipes) {
-    case 4: return conv3_launch_t<4>(a, (int)ctas * a.ngroups, st);
-    case 2: return conv3_launch_t<2>(a, (int)ctas * a.ngroups, st);
-    default: return conv3_launch_t<1>(a, (int)ctas * a.ngroups, st);
+    case 4: return head ? conv3_launch_t<4, true>(a, nc, st) : conv3_launch_t<4, false>(a, nc, st);
+    case 2: return head ? conv3_launch_t<2, true>(a, nc, st) : conv3_launch_t<2, false>(a, nc, st);
+    default: return head ? conv3_launch_t<1, true>(a, nc, st) : conv3_launch_t<1, false>(a, nc, st);
   }
 }
 
