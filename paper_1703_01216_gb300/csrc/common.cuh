@@ -151,10 +151,10 @@ __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.lau
 // the stream has released it or exited; it must call pdl_wait() in every thread before it touches what that kernel
 // (or, through that kernel's own wait, an earlier one) reads or writes.
 template <typename... P, typename... A>
-int launch_on(bool pdl, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, const A&... args) {
+int launch_on(bool pdl, void (*kern)(P...), dim3 grid, dim3 threads, size_t smem, cudaStream_t st, const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
+  cfg.blockDim = threads;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];

@@ -142,6 +142,11 @@ __device__ __forceinline__ long ppos(const LevelArg& L, int d, int h, int w) {
   return ((long)(d + 1) * L.Hp + (h + 1)) * L.Wp + (w + 1);
 }
 
+// Pooling, upsampling, their adjoints, the convolutions and the weight gradients are launched programmatically: their
+// set-up (barriers, tensor memory) and their launch run while the kernel before them leaves the SMs (24 and 62 launches:
+// 1024 -> 973 us forward and 3462 -> 3305 us gradient at 128^2 x 32, batch 8; 177 -> 117 and 600 -> 412 us at 24^2 x 8,
+// batch 1).  Each waits for that kernel before its first access to global memory; the others are launched as usual.
+//
 // The elementwise kernels below run one (chunk, depth, row) per blockDim.y lane group and consecutive w per
 // thread, so that the index divisions are per row and in 32 bits (per voxel and in 64 bits they cost more than
 // the memory traffic: the level-0 upsampling took 117 us for 310 MB).
@@ -188,6 +193,8 @@ __global__ void k_pack_input(const float* __restrict__ x, int B, LevelArg L, flo
 // average pooling by 2: dst (level l+1, chunks [0, nc)) from src (level l, chunks [soff, soff + nc))
 __global__ void k_pool(const unsigned char* __restrict__ src, int s_chunks, int soff, LevelArg Ls,
                        unsigned char* __restrict__ dst, int d_chunks, LevelArg Ld, int nc, int B) {
+  pdl_wait();
+  pdl_release();
   const Row q = row_of(B, nc, Ld.D, Ld.H);
   if (!q.ok) return;
   for (int w = threadIdx.x; w < Ld.W; w += blockDim.x) {
@@ -215,6 +222,8 @@ __global__ void k_pool(const unsigned char* __restrict__ src, int s_chunks, int 
 // (a parent per lane left 16 of every 32 bytes to a second store: 74 us to level 0 at 128^2 x 32, batch 8, now 51)
 __global__ void k_up(const unsigned char* __restrict__ src, int s_chunks, LevelArg Ls, unsigned char* __restrict__ dst,
                      int d_chunks, LevelArg Ld, int nc, int B) {
+  pdl_wait();
+  pdl_release();
   const Row q = row_of(B, nc, Ls.D, Ls.H);
   if (!q.ok) return;
   for (int w = threadIdx.x; w < Ld.W; w += blockDim.x) {
@@ -229,6 +238,8 @@ __global__ void k_up(const unsigned char* __restrict__ src, int s_chunks, LevelA
 __global__ void k_up_backward(const unsigned char* __restrict__ gd, int d_chunks, LevelArg Ld,
                               const unsigned char* __restrict__ s, unsigned char* __restrict__ gs, int s_chunks,
                               LevelArg Ls, int nc, int B) {
+  pdl_wait();
+  pdl_release();
   const Row q = row_of(B, nc, Ls.D, Ls.H);
   if (!q.ok) return;
   for (int w = threadIdx.x; w < Ls.W; w += blockDim.x) {
@@ -258,6 +269,8 @@ __global__ void k_up_backward(const unsigned char* __restrict__ gd, int d_chunks
 __global__ void k_pool_backward(const unsigned char* __restrict__ gp, int p_chunks, LevelArg Lp,
                                 const unsigned char* __restrict__ s, unsigned char* __restrict__ g, int c_chunks,
                                 int coff, LevelArg Lc, int nc, int B) {
+  pdl_wait();
+  pdl_release();
   const Row q = row_of(B, nc, Lc.D, Lc.H);
   if (!q.ok) return;
   for (int w = threadIdx.x; w < Lc.W; w += blockDim.x) {
@@ -542,9 +555,8 @@ int forward(Unet* U, const float* x, int B, const float* t, float* out, cudaStre
     const int src = T_CAT + l - 1;
     const int nc = kWidth[l - 1] / 8;
     blk = row_block(U->lv[l].W);
-    k_pool<<<row_grid(B, nc, U->lv[l].D, U->lv[l].H, blk), blk, 0, st>>>(U->t[src], U->td[src].C / 8, kWidth[l] / 8, larg(U->lv[l - 1]),
-                                         U->t[T_P + l - 1], nc, larg(U->lv[l]), nc, B);
-    FR3D_CUDA_TRY(cudaGetLastError());
+    FR3D_TRY(launch_on(true, k_pool, row_grid(B, nc, U->lv[l].D, U->lv[l].H, blk), blk, 0, st,
+                       U->t[src], U->td[src].C / 8, kWidth[l] / 8, larg(U->lv[l - 1]), U->t[T_P + l - 1], nc, larg(U->lv[l]), nc, B));
     FR3D_TRY(conv_forward(U, 2 * l, B, st));
     FR3D_TRY(conv_forward(U, 2 * l + 1, B, st));
     if (l == kL - 1) FR3D_TRY(conv_forward(U, 8, B, st));
@@ -553,9 +565,8 @@ int forward(Unet* U, const float* x, int B, const float* t, float* out, cudaStre
     const int src = l == kL - 2 ? T_B + 2 : T_D2 + l + 1;
     const int nc = kWidth[l + 1] / 8;
     blk = row_block(U->lv[l].W);
-    k_up<<<row_grid(B, nc, U->lv[l + 1].D, U->lv[l + 1].H, blk), blk, 0, st>>>(U->t[src], U->td[src].C / 8, larg(U->lv[l + 1]), U->t[T_CAT + l],
-                                       U->td[T_CAT + l].C / 8, larg(U->lv[l]), nc, B);
-    FR3D_CUDA_TRY(cudaGetLastError());
+    FR3D_TRY(launch_on(true, k_up, row_grid(B, nc, U->lv[l + 1].D, U->lv[l + 1].H, blk), blk, 0, st,
+                       U->t[src], U->td[src].C / 8, larg(U->lv[l + 1]), U->t[T_CAT + l], U->td[T_CAT + l].C / 8, larg(U->lv[l]), nc, B));
     const int k = 9 + 2 * (kL - 2 - l);
     FR3D_TRY(conv_forward(U, k, B, st));
     if (l > 0) FR3D_TRY(conv_forward(U, k + 1, B, st));
@@ -591,9 +602,8 @@ int backward(Unet* U, const float* t, int B, float* loss, cudaStream_t st) {
     const int dst = l == kL - 2 ? T_B + 2 : T_D2 + l + 1;
     const int nc = kWidth[l + 1] / 8;
     const dim3 blk = row_block(U->lv[l + 1].W);
-    k_up_backward<<<row_grid(B, nc, U->lv[l + 1].D, U->lv[l + 1].H, blk), blk, 0, st>>>(U->g[T_CAT + l], U->td[T_CAT + l].C / 8, larg(U->lv[l]), U->t[dst],
-                                                U->g[dst], U->td[dst].C / 8, larg(U->lv[l + 1]), nc, B);
-    FR3D_CUDA_TRY(cudaGetLastError());
+    FR3D_TRY(launch_on(true, k_up_backward, row_grid(B, nc, U->lv[l + 1].D, U->lv[l + 1].H, blk), blk, 0, st,
+                       U->g[T_CAT + l], U->td[T_CAT + l].C / 8, larg(U->lv[l]), U->t[dst], U->g[dst], U->td[dst].C / 8, larg(U->lv[l + 1]), nc, B));
   }
   FR3D_TRY(conv_backward(U, 8, B, st));
   FR3D_TRY(conv_backward(U, 7, B, st));
@@ -601,10 +611,8 @@ int backward(Unet* U, const float* t, int B, float* loss, cudaStream_t st) {
   for (int l = kL - 2; l >= 0; --l) {
     const int nc = kWidth[l] / 8;
     const dim3 blk = row_block(U->lv[l].W);
-    k_pool_backward<<<row_grid(B, nc, U->lv[l].D, U->lv[l].H, blk), blk, 0, st>>>(U->g[T_P + l], nc, larg(U->lv[l + 1]), U->t[T_CAT + l] +
-                                                  0, U->g[T_CAT + l], U->td[T_CAT + l].C / 8, kWidth[l + 1] / 8,
-                                                  larg(U->lv[l]), nc, B);
-    FR3D_CUDA_TRY(cudaGetLastError());
+    FR3D_TRY(launch_on(true, k_pool_backward, row_grid(B, nc, U->lv[l].D, U->lv[l].H, blk), blk, 0, st,
+                       U->g[T_P + l], nc, larg(U->lv[l + 1]), U->t[T_CAT + l] + 0, U->g[T_CAT + l], U->td[T_CAT + l].C / 8, kWidth[l + 1] / 8, larg(U->lv[l]), nc, B));
     FR3D_TRY(conv_backward(U, 2 * l + 1, B, st));
     FR3D_TRY(conv_backward(U, 2 * l, B, st));
   }

@@ -140,9 +140,11 @@ __global__ void __launch_bounds__(PIPES* kPipeThreads, 1) k_conv3(ConvArgs a) {
     }
     tc::mbar_fence_init();
   }
+  if (warp == 0) tc::tmem_alloc(&tbase, kTmemCols);
+  pdl_wait();
+  pdl_release();
   if (tid < Ng) sbias[tid] = a.bias ? a.bias[grp * Ng + tid] : 0.f;
   if (HEAD && tid < 17) shead[tid] = tid < 16 ? tc::bf16_val(tc::bf16_rn(a.hw[tid])) : a.hw[16];
-  if (warp == 0) tc::tmem_alloc(&tbase, kTmemCols);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -414,6 +416,8 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
     issued = 0;
   }
   if (warp == 0) tc::tmem_alloc(&tbase, kWgTmem);
+  pdl_wait();
+  pdl_release();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -602,12 +606,15 @@ constexpr int kWgRedThreads = 512;
 __global__ void __launch_bounds__(kWgRedThreads) k_wgrad_reduce(WgradArgs a, int nunits, int ci, float* __restrict__ dW,
                                                                float* __restrict__ db) {
   __shared__ double red[kWgRedThreads];
+  pdl_wait();
+  pdl_release();
   const int per = 3 * a.Og * kWgCols, npairs = a.n_og * a.n_cg, nw = per * npairs;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const bool ok = i < nw + a.Cout;
   double s = 0.0;
   if (ok) {
     const float* p = i < nw ? a.partials + i : a.bias_partials + (i - nw);
+    asm volatile("" : "+l"(p)::"memory");   // (no load of the partials is moved above the wait)
     const long ustep = i < nw ? nw : a.Cout;
     float hi = 0.f, lo = 0.f;
 #pragma unroll 8
@@ -696,9 +703,7 @@ template <int PIPES, bool HEAD> int conv3_launch_t(const ConvArgs& a, int ctas, 
   // all of the SM's tensor memory is one CTA's: ask for more than half of its shared memory
   const size_t smem = std::max(conv_weight_bytes(a.Cin, a.Ng) + (size_t)PIPES * a.stages * kConvStageBytes, (size_t)120 * 1024);
   FR3D_TRY(smem_optin(reinterpret_cast<const void*>(k_conv3<PIPES, HEAD>), smem));
-  k_conv3<PIPES, HEAD><<<ctas, PIPES * kPipeThreads, smem, st>>>(a);
-  FR3D_CUDA_TRY(cudaGetLastError());
-  return FR3D_OK;
+  return launch_on(true, k_conv3<PIPES, HEAD>, ctas, PIPES * kPipeThreads, smem, st, a);
 }
 
 }  // namespace
@@ -783,12 +788,10 @@ int wgrad3_launch(const WgradArgs& args, int ci, float* dW, float* db, cudaStrea
   const int units = a.B * a.nspans * a.nchunks, npairs = a.n_og * a.n_cg;
   const int total = npairs * 3 * a.Og * kWgCols;
   a.bias_partials = a.partials + (size_t)units * total;
-  k_wgrad3<<<units * npairs, kWgThreads, smem, st>>>(a);
+  FR3D_TRY(launch_on(true, k_wgrad3, units * npairs, kWgThreads, smem, st, a));
   // threads per element: about eight units each, so that the loads of a layer with few elements fill the chip
   const int ry = units >= 512 ? 32 : (units >= 128 ? 16 : (units >= 32 ? 4 : 1)), rx = kWgRedThreads / ry;
-  k_wgrad_reduce<<<(total + a.Cout + rx - 1) / rx, dim3(rx, ry), 0, st>>>(a, units, ci, dW, db);
-  FR3D_CUDA_TRY(cudaGetLastError());
-  return FR3D_OK;
+  return launch_on(true, k_wgrad_reduce, (total + a.Cout + rx - 1) / rx, dim3(rx, ry), 0, st, a, units, ci, dW, db);
 }
 
 }  // namespace fr3d
