@@ -601,7 +601,8 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
 // take every blockDim.y-th unit, then their sums in order).  A thread adds in FP32 with the rounding errors carried
 // along (Knuth's two-sum; what is lost is of order 2^-48): the FP64 conversions and additions were the bound.
 // 29 MB of partials: 42 -> 22 us, 86 MB: 98 -> 58 us, with four times the loads in flight.  Sums that are not finite
-// are added again in FP64, as a chain that leaves FP32's range on the way has to be.
+// are added again in FP64, as a chain that leaves FP32's range on the way has to be.  The partials are read with coherent
+// loads: k_wgrad3 may still be writing them when this kernel starts.
 constexpr int kWgRedThreads = 512;
 __global__ void __launch_bounds__(kWgRedThreads) k_wgrad_reduce(WgradArgs a, int nunits, int ci, float* __restrict__ dW,
                                                                float* __restrict__ db) {
@@ -614,19 +615,18 @@ __global__ void __launch_bounds__(kWgRedThreads) k_wgrad_reduce(WgradArgs a, int
   double s = 0.0;
   if (ok) {
     const float* p = i < nw ? a.partials + i : a.bias_partials + (i - nw);
-    asm volatile("" : "+l"(p)::"memory");   // (no load of the partials is moved above the wait)
     const long ustep = i < nw ? nw : a.Cout;
     float hi = 0.f, lo = 0.f;
 #pragma unroll 8
     for (int u = threadIdx.y; u < nunits; u += blockDim.y) {
-      const float x = __ldg(p + u * ustep), t = __fadd_rn(hi, x), d = __fsub_rn(t, hi);
+      const float x = __ldcg(p + u * ustep), t = __fadd_rn(hi, x), d = __fsub_rn(t, hi);
       lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, d)), __fsub_rn(x, d)));
       hi = t;
     }
     s = (double)hi + (double)lo;
     if (!isfinite(hi) || !isfinite(lo)) {
       s = 0.0;
-      for (int u = threadIdx.y; u < nunits; u += blockDim.y) s += (double)__ldg(p + u * ustep);
+      for (int u = threadIdx.y; u < nunits; u += blockDim.y) s += (double)__ldcg(p + u * ustep);
     }
   }
   if (blockDim.y > 1) {
