@@ -142,11 +142,11 @@ __global__ void __launch_bounds__(PIPES* kPipeThreads, 1) k_conv3(ConvArgs a) {
   }
   if (warp == 0) tc::tmem_alloc(&tbase, kTmemCols);
   pdl_wait();
-  pdl_release();
   if (tid < Ng) sbias[tid] = a.bias ? a.bias[grp * Ng + tid] : 0.f;
   if (HEAD && tid < 17) shead[tid] = tid < 16 ? tc::bf16_val(tc::bf16_rn(a.hw[tid])) : a.hw[16];
   tc::fence_before_sync();
   __syncthreads();
+  pdl_release();   // the CTA holds its tensor memory: a successor's CTA on this SM cannot take it while it waits for this one
   tc::fence_after_sync();
   const uint32_t tmem = tbase + pipe * (kTmemCols / PIPES);
   if (role == 1) {
@@ -417,9 +417,9 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
   }
   if (warp == 0) tc::tmem_alloc(&tbase, kWgTmem);
   pdl_wait();
-  pdl_release();
   tc::fence_before_sync();
   __syncthreads();
+  pdl_release();   // after the allocation, as in k_conv3
   tc::fence_after_sync();
   const uint32_t tmem = tbase;
   if (warp == 4) {
