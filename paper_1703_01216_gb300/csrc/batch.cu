@@ -125,9 +125,23 @@ int run_alpha(const AlphaPlan& a, const unsigned char* dev, cudaStream_t st) {
 
 }  // namespace
 
+// The info words that the alpha rule does not write (instances with a fixed or given alpha): cleared on every run, before
+// the inverse may report into them.
+std::vector<int*> unruled_info(const fr3d_instance* inst, int n) {
+  std::vector<int*> w;
+  for (int i = 0; i < n; ++i)
+    if (inst[i].opts->info && inst[i].opts->alpha_mode != FR3D_ALPHA_DISCREPANCY) w.push_back(inst[i].opts->info);
+  return w;
+}
+int clear_info(const std::vector<int*>& words, cudaStream_t st) {
+  for (int* w : words) FR3D_CUDA_TRY(cudaMemsetAsync(w, 0, sizeof(int), st));
+  return FR3D_OK;
+}
+
 struct Batch {
   std::vector<Group> groups;
   AlphaPlan alpha;
+  std::vector<int*> info;          // words to clear (unruled_info)
   unsigned char* dev = nullptr;
   unsigned char* qbuf = nullptr;   // the tile queue's counters and intermediates (zeroed once)
   int output = FR3D_OUT_XI;
@@ -234,6 +248,7 @@ void build_descriptors(const fr3d_instance* inst, const std::map<int, std::vecto
       }
       FusedArgs f;
       fused_args_f32(H, uh[idx], dd[idx], ai[idx], I.opts->n_bands > 1 ? I.opts->n_bands : 1, H->wtab, I.out, I.Q, &f);
+      f.info = I.opts->info;
       for (int j = 0; j < H->Mp; ++j) map.push_back(make_int2((int)fa.size(), j));
       fa.push_back(f);
     }
@@ -343,6 +358,7 @@ extern "C" int fr3d_batch_create(const fr3d_instance* inst, int n, fr3d_batch** 
       return FR3D_ERR_CUDA;
     }
   }
+  b.info = unruled_info(inst, n);
   b.launches = batch_launches(b.groups, b.alpha);
   fr3d_batch* h = new (std::nothrow) fr3d_batch();
   if (!h) {
@@ -362,6 +378,7 @@ extern "C" int fr3d_batch_run(fr3d_batch* h, void* stream) {
   const int mode = fused_tune_mode_get();
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   FR3D_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
+  FR3D_TRY(clear_info(h->b.info, st));
   for (auto& g : h->b.groups) FR3D_TRY(run_group_pre(g, h->b.dev, st));
   FR3D_TRY(run_alpha(h->b.alpha, h->b.dev, st));
   for (auto& g : h->b.groups) {
@@ -452,6 +469,7 @@ extern "C" int fr3d_invert_batched(const fr3d_instance* inst, int n, void* works
   FR3D_CUDA_TRY(cudaMemcpyAsync(tables, host.data(), host.size(), cudaMemcpyHostToDevice, st));
   const int mode = fused_tune_mode_get();
   const int v = mode >= 2 ? mode - 2 : 3;   // the forced tile, else the register-accumulator tile
+  FR3D_TRY(clear_info(unruled_info(inst, n), st));
   for (auto& g : groups) FR3D_TRY(run_group_pre(g, tables, st));
   FR3D_TRY(run_alpha(ap, tables, st));
   for (auto& g : groups)

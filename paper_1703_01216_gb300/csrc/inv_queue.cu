@@ -31,9 +31,9 @@
 // mbarriers.  64 depths and 8 sources: n = 192 57 us (the fused cluster tiles 120, spilling; the two passes
 // 107), n = 256 80 us; n = 96 and 128 have too few tiles alone (40 and 38 us, as the other variants) and gain in a
 // batch (49 and 51 sources' planes: 184 -> 81 us and 167 -> 118 us).  Every wait (on a stage or a counter) is
-// bounded: on expiry the kernel ORs
-// FR3D_INFO_TIMEOUT into the caller's info word and lets every other wait end at once, so the launch
-// always ends.
+// bounded: on expiry every other wait of the launch ends at once, so the launch always ends, and its last CTA ORs
+// FR3D_INFO_TIMEOUT into the info word of every instance (a batch's instances wait in one queue, and any of their tiles may
+// have run on incomplete data).
 // The arithmetic of every output (the solve weights, the radix passes and their twiddles, the split, the
 // order of the accumulation over q) is the fused kernel's, so all variants return the same bits.
 #include <string.h>
@@ -141,27 +141,26 @@ __device__ __forceinline__ void decode_ticket(int k, int nj, int lag, int& kind,
 // source parameters of the first half (the first dependency step of a row tile)
 __device__ __forceinline__ int half_q(int Q) { return Q > 1 ? Q / 2 : 1; }
 
-__device__ __forceinline__ void report_timeout(const QLaunch& ql, const QInst& qa) {
-  atomicExch(ql.ctl + 2, 1);
-  if (qa.f.info) atomicOr(qa.f.info, FR3D_INFO_TIMEOUT);
-}
+// A wait gave up.  Every other wait of the launch then ends at once, whichever instance it belongs to, so the last CTA
+// flags every instance of the launch.
+__device__ __forceinline__ void report_timeout(const QLaunch& ql) { atomicExch(ql.ctl + 2, 1); }
 
 // Wait until *c >= target (acquire), or a wait elsewhere has given up; false if this one gave up.
-__device__ __forceinline__ bool wait_count(const QLaunch& ql, const QInst& qa, const int* c, int target) {
+__device__ __forceinline__ bool wait_count(const QLaunch& ql, const int* c, int target) {
   const volatile int* gave_up = ql.ctl + 2;
   for (long it = 0; it < kSpinLimit; ++it) {
     int v;
     asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(c) : "memory");
     if (v >= target) return true;
-    if (*gave_up) return true;   // the results are flagged already; do not wait again
+    if (*gave_up) return true;   // the results will be flagged; do not wait again
     __nanosleep(128);
   }
-  report_timeout(ql, qa);
+  report_timeout(ql);
   return false;
 }
 
-__device__ __forceinline__ void stage_wait(const QLaunch& ql, const QInst& qa, uint64_t* bar, uint32_t& parity) {
-  if (!tc::mbar_wait(bar, parity, kSpinLimit)) report_timeout(ql, qa);
+__device__ __forceinline__ void stage_wait(const QLaunch& ql, uint64_t* bar, uint32_t& parity) {
+  if (!tc::mbar_wait(bar, parity, kSpinLimit)) report_timeout(ql);
   parity ^= 1u;
 }
 
@@ -261,7 +260,7 @@ __device__ __forceinline__ void column_tile(const QLaunch& ql, const QInst& qa, 
   float2* Tj = qa.T + (long)j * a.Q * N * L;
   for (int q = 0; q < a.Q; ++q) {
     const int sl = q & 1;
-    stage_wait(ql, qa, &bar[sl], par[sl]);
+    stage_wait(ql, &bar[sl], par[sl]);
     // first pass of the inverse column DFTs from the stage (butterfly jj of column c: bins jj + BC r)
     if (act) {
       const float2* sg = stage + sl * STG + c * N;
@@ -349,7 +348,7 @@ __device__ __forceinline__ void row_tile(const QLaunch& ql, const QInst& qa, int
   // q's rows once every column tile of depth j has finished the half of the source parameters q is in
   auto issue = [&](int q, int sl) {
     if (q == 0 || q == half_q(a.Q)) {
-      wait_count(ql, qa, qa.cnt + 2 * j + (q == 0 ? 0 : 1), NCT);
+      wait_count(ql, qa.cnt + 2 * j + (q == 0 ? 0 : 1), NCT);
       fence_proxy_global();
     }
     fence_proxy_smem();
@@ -390,7 +389,7 @@ __device__ __forceinline__ void row_tile(const QLaunch& ql, const QInst& qa, int
   __syncthreads();   // tables
   for (int q = 0; q < a.Q; ++q) {
     const int sl = q & 1;
-    stage_wait(ql, qa, &bar[sl], par[sl]);
+    stage_wait(ql, &bar[sl], par[sl]);
     // the rows of T are in shared memory now: drop their lines from L2 (one 128-byte line per thread)
     if (L == kQThreads || tid < L) l2_discard(Tj + ((long)q * (N / 16) + b) * L * 16 + tid * 16);
     float2* sg = stage + sl * STG;            // Z'[k][row], split by the column tiles
@@ -484,13 +483,17 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) k_inv_queue(QLaunch ql
     else row_tile<N>(ql, s_inst, j, t, stage, buf, tab, bar, par, pol, tid);
     __syncthreads();   // before thread 0 overwrites the ticket
   }
-  // the last CTA to finish resets the queue for the next launch
+  // the last CTA to finish reports waits that gave up and resets the queue for the next launch
   if (tid == 0) {
     __threadfence();
     if (atomicAdd(ql.ctl + 1, 1) == (int)gridDim.x - 1) {
       __threadfence();
       ql.ctl[0] = 0;
-      ql.ctl[2] = 0;
+      if (atomicExch(ql.ctl + 2, 0))
+        for (int i = 0; i < ql.ninst; ++i) {
+          int* info = (ql.tab ? ql.tab[i] : ql.inst0).f.info;
+          if (info) atomicOr(info, FR3D_INFO_TIMEOUT);
+        }
       for (int e = 0; e < ql.ncnt; ++e) ql.cnt_all[e] = 0;
       __threadfence();
       ql.ctl[1] = 0;
