@@ -368,69 +368,17 @@ int invert_impl(Handle* H, const T* U, int Q, const fr3d_invert_opts* o, T* out,
   C* Tb = reinterpret_cast<C*>((char*)H->ws + p.t_off);
   int launches = 0;
   prof_begin(H, st);
-  // step 1: 2D DFT of the data
-  FR3D_TRY(data_fft<T>(H, U, Q, Uh, st));
-  launches += 2;
-  // step 2 (parameter): alpha
-  const int* aidx;
-  const T* D;
   const int nb = o->n_bands > 1 ? o->n_bands : 1;
+  const bool fused = sizeof(T) == 4 && fused_supported(H->n);
+  // Tables that changed since the last call.  They come before the transform, so that they are complete before any
+  // kernel starts whose programmatic successor reads them (the inverse, through the read-only path).
   if (nb > 1) FR3D_TRY(ensure_bands(H, nb, nullptr));
-  if (o->alpha_mode == FR3D_ALPHA_DISCREPANCY) {
-    FR3D_TRY(alpha_tables(H, o->alphas, o->n_alpha, o->ra, st));
-    prof_mark(H, kStTable, st);
-    int* idx = o->alpha_idx ? o->alpha_idx : H->idx_scratch;
-    double thr2[FR3D_MAX_BANDS];
-    band_thresholds(H, o, nb, thr2);
-    FR3D_TRY(Ops<T>::alpha_choose(H, Uh, Q * H->M, o->n_alpha, thr2, nb, idx, o->residuals, o->info, st));
-    prof_mark(H, kStAlpha, st);
-    launches += 1;
-    aidx = idx;
-    if constexpr (sizeof(T) == 4) D = H->D32;
-    else D = H->D64;
-  } else if (o->alpha_mode == FR3D_ALPHA_LEARNED) {
-    FR3D_TRY(alpha_tables(H, o->alphas, o->n_alpha, o->ra, st));
-    prof_mark(H, kStTable, st);
-    int* idx = o->alpha_idx ? o->alpha_idx : H->idx_scratch;
-    if constexpr (sizeof(T) == 4) {
-      FR3D_TRY(learned_alpha(H, Uh, Q * H->M, nb, o->delta, o->alphas, o->n_alpha, o->net, idx, nullptr, o->info, st));
-      D = H->D32;
-    } else {
-      return FR3D_ERR_INVALID_ARG;   // excluded by check_invert_args
-    }
-    prof_mark(H, kStAlpha, st);
-    launches += 1;
-    aidx = idx;
-  } else if (o->alpha_mode == FR3D_ALPHA_GIVEN) {
-    FR3D_TRY(alpha_tables(H, o->alphas, o->n_alpha, o->ra, st));
-    prof_mark(H, kStTable, st);
-    aidx = o->alpha_idx;
-    if constexpr (sizeof(T) == 4) D = H->D32;
-    else D = H->D64;
-    if (o->info) FR3D_CUDA_TRY(cudaMemsetAsync(o->info, 0, sizeof(int), st));
-  } else {
-    FR3D_TRY(fixed_table(H, o->alpha, o->ra, st));
-    prof_mark(H, kStTable, st);
-    aidx = H->zero_idx;
-    if constexpr (sizeof(T) == 4) D = H->Dfix32;
-    else D = H->Dfix64;
-    if (o->alpha_idx) FR3D_CUDA_TRY(cudaMemsetAsync(o->alpha_idx, 0, sizeof(int), st));
-    if (o->info) FR3D_CUDA_TRY(cudaMemsetAsync(o->info, 0, sizeof(int), st));
-  }
-  if constexpr (sizeof(T) == 4) {
-    if (fused_supported(H->n)) {
-      // steps 2 (solve) + 3 (inverse DFT) + 4 (combination) fused, one launch for all depths
-      if (o->output == FR3D_OUT_XI) {
-        FR3D_TRY(ensure_wtab(H, o->sources, st));
-        prof_mark(H, kStTable, st);
-      }
-      const float* Dd = o->alpha_mode == FR3D_ALPHA_FIXED ? H->Ddfix32 : H->Dd32;
-      FR3D_TRY(inv_fused_f32(H, Uh, Dd, aidx, nb, H->wtab, out, Q, 0, H->Mp, o->output, st, out_host_mapped,
-                             o->info));
-      prof_mark(H, kStFused, st);
-      H->last_launches = launches + 1;
-      return FR3D_OK;
-    }
+  if (o->alpha_mode == FR3D_ALPHA_FIXED) FR3D_TRY(fixed_table(H, o->alpha, o->ra, st));
+  else FR3D_TRY(alpha_tables(H, o->alphas, o->n_alpha, o->ra, st));
+  const T* W = nullptr;
+  if (o->output == FR3D_OUT_XI) {
+    if (fused) FR3D_TRY(ensure_wtab(H, o->sources, st));
+    else FR3D_TRY(weights_or_null<T>(H, o->sources, &W, st));
   }
   const T* A;
   if constexpr (sizeof(T) == 4) A = H->A32;
@@ -438,10 +386,52 @@ int invert_impl(Handle* H, const T* U, int Q, const fr3d_invert_opts* o, T* out,
     FR3D_TRY(build_dense64(H, st));
     A = H->A64d;
   }
-  const T* W = nullptr;
-  if (o->output == FR3D_OUT_XI) {
-    FR3D_TRY(weights_or_null<T>(H, o->sources, &W, st));
-    prof_mark(H, kStTable, st);
+  prof_mark(H, kStTable, st);
+  // step 1: 2D DFT of the data
+  FR3D_TRY(data_fft<T>(H, U, Q, Uh, st));
+  launches += 2;
+  // step 2 (parameter): alpha
+  const int* aidx;
+  const T* D;
+  if (o->alpha_mode == FR3D_ALPHA_DISCREPANCY) {
+    int* idx = o->alpha_idx ? o->alpha_idx : H->idx_scratch;
+    double thr2[FR3D_MAX_BANDS];
+    band_thresholds(H, o, nb, thr2);
+    FR3D_TRY(Ops<T>::alpha_choose(H, Uh, Q * H->M, o->n_alpha, thr2, nb, idx, o->residuals, o->info, st));
+    prof_mark(H, kStAlpha, st);
+    launches += 1;
+    aidx = idx;
+  } else if (o->alpha_mode == FR3D_ALPHA_LEARNED) {
+    int* idx = o->alpha_idx ? o->alpha_idx : H->idx_scratch;
+    if constexpr (sizeof(T) == 4) {
+      FR3D_TRY(learned_alpha(H, Uh, Q * H->M, nb, o->delta, o->alphas, o->n_alpha, o->net, idx, nullptr, o->info, st));
+    } else {
+      return FR3D_ERR_INVALID_ARG;   // excluded by check_invert_args
+    }
+    prof_mark(H, kStAlpha, st);
+    launches += 1;
+    aidx = idx;
+  } else if (o->alpha_mode == FR3D_ALPHA_GIVEN) {
+    aidx = o->alpha_idx;
+    if (o->info) FR3D_CUDA_TRY(cudaMemsetAsync(o->info, 0, sizeof(int), st));
+  } else {
+    aidx = H->zero_idx;
+    if (o->alpha_idx) FR3D_CUDA_TRY(cudaMemsetAsync(o->alpha_idx, 0, sizeof(int), st));
+    if (o->info) FR3D_CUDA_TRY(cudaMemsetAsync(o->info, 0, sizeof(int), st));
+  }
+  const bool fixed = o->alpha_mode == FR3D_ALPHA_FIXED;
+  if constexpr (sizeof(T) == 4) {
+    D = fixed ? H->Dfix32 : H->D32;
+    if (fused) {
+      // steps 2 (solve) + 3 (inverse DFT) + 4 (combination) fused, one launch for all depths
+      FR3D_TRY(inv_fused_f32(H, Uh, fixed ? H->Ddfix32 : H->Dd32, aidx, nb, H->wtab, out, Q, 0, H->Mp, o->output, st,
+                             out_host_mapped, o->info));
+      prof_mark(H, kStFused, st);
+      H->last_launches = launches + 1;
+      return FR3D_OK;
+    }
+  } else {
+    D = fixed ? H->Dfix64 : H->D64;
   }
   // step 2 (solve) + step 3 (inverse DFT) + step 4 (xi = zeta / V0), by chunks of depths
   for (int j0 = 0; j0 < H->Mp; j0 += p.chunk) {

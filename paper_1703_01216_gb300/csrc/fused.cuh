@@ -121,6 +121,8 @@ struct FusedArgs {
 };
 
 // PRE: the column phase transforms the solved spectra a.Zs (M > 1 path) instead of weighting U~.
+// The kernel is launched programmatically, and its predecessor may be what wrote the spectra (with a fixed or given alpha no
+// kernel lies between them): those are read with coherent loads.  Every table was complete before the predecessor began.
 template <int N, int MODE, int V, bool PRE = false>
 __device__ __forceinline__ void inv_fused_body(const FusedArgs& a, int jl) {
   using G = FusedGeom<N, V>;
@@ -243,19 +245,19 @@ __device__ __forceinline__ void inv_fused_body(const FusedArgs& a, int jl) {
     auto ldc = [&](int col, int ky) -> float2 {
       const int e = col * N + ky;
       if constexpr (PRE) {        // solved spectrum of depth j (M > 1 path)
-        float2 v = __ldg(Zj + (long)c0 * N + e);
+        float2 v = __ldcg(Zj + (long)c0 * N + e);
         if (r == 0 && col == 0) {
-          const float2 un = __ldg(Zj + (long)L * N + ky);
+          const float2 un = __ldcg(Zj + (long)L * N + ky);
           v.x -= un.y;
           v.y += un.x;
         }
         return v;
       }
-      const float2 u = __ldg(Zq + (long)c0 * N + e);
+      const float2 u = __ldcg(Zq + (long)c0 * N + e);
       const float w = wsm[e];
       float2 v = make_float2(__fmul_rn(u.x, w), __fmul_rn(u.y, w));
       if (r == 0 && col == 0) {   // packed column 0: add i w(n/2, ky) U~(n/2, ky)
-        const float2 un = __ldg(Zq + (long)L * N + ky);
+        const float2 un = __ldcg(Zq + (long)L * N + ky);
         const float wl = wsm[CPC * N + ky];
         v.x = __fmaf_rn(-un.y, wl, v.x);
         v.y = __fmaf_rn(un.x, wl, v.y);
