@@ -488,13 +488,16 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) k_inv_queue(QLaunch ql
     __threadfence();
     if (atomicAdd(ql.ctl + 1, 1) == (int)gridDim.x - 1) {
       __threadfence();
+      const int gave_up = *(const volatile int*)(ql.ctl + 2);   // (its latency overlaps the stores)
       ql.ctl[0] = 0;
-      if (atomicExch(ql.ctl + 2, 0))
+      for (int e = 0; e < ql.ncnt; ++e) ql.cnt_all[e] = 0;
+      if (gave_up) {
+        ql.ctl[2] = 0;
         for (int i = 0; i < ql.ninst; ++i) {
-          int* info = (ql.tab ? ql.tab[i] : ql.inst0).f.info;
+          int* info = ql.tab ? ql.tab[i].f.info : ql.inst0.f.info;
           if (info) atomicOr(info, FR3D_INFO_TIMEOUT);
         }
-      for (int e = 0; e < ql.ncnt; ++e) ql.cnt_all[e] = 0;
+      }
       __threadfence();
       ql.ctl[1] = 0;
     }
