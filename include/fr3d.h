@@ -33,7 +33,10 @@
  * a new shape (so make that first call outside any stream capture).  Calls are
  * asynchronous on the given CUDA stream (NULL = legacy default stream); results
  * are valid once the stream has synchronised.  One handle serves one stream at a
- * time: concurrent calls on one handle share its workspace and race.
+ * time: concurrent calls on one handle share its workspace and race.  A handle that inverts to xi in FP64,
+ * or in FP32 at n = 512, also keeps its sources' combination weights (8 or 4 bytes x Q M' n^2, at most 4 GiB;
+ * larger, without room, or in a first xi call inside a capture: the weights are evaluated per voxel, slower and
+ * with other roundings).  They are given back when the workspace finds no room to grow.
  *
  * Errors.  Every call returns an int status: FR3D_OK (0) or a negative
  * FR3D_ERR_* code; argument and geometry checks happen on the host before any
@@ -324,6 +327,12 @@ int fr3d_autotune_query(fr3d_handle* h, int* variant, float* ms, int cap);
  * still returns, with FR3D_INFO_TIMEOUT set in the info word, and its xi is not valid.  No fault and no
  * hang is involved; the next call with the hook off is exact again.  Returns the previous setting. */
 int fr3d_test_withhold_queue_counts(int on);
+
+/* Test hook of the paths for a device without room: while bytes >= 0, the handles' workspaces, their tables of
+ * combination weights and the batched plans' queue buffers may take that many bytes more in all (what they give back
+ * counts again), and requests beyond it fail as if the device were full.  bytes < 0: no budget (the default).  attempts
+ * (may be NULL): how many such requests were made since the last call. */
+int fr3d_test_alloc_budget(long long bytes, int* attempts);
 
 /* ---- learned post-corrector: a 3D U-Net on the tensor cores (fr3d_unet) ----
  * The paper has no network.  This one post-corrects the reconstruction of fr3d_invert: with one observation

@@ -92,7 +92,7 @@ int ensure_wtab(Handle* H, const fr3d_sources* s, cudaStream_t st) {
 
 // Combination weights of the unfused row pass (FP64, and n = 512 in FP32): the same table in T, up to
 // kWeightBytes; *W = nullptr (V0 evaluated per voxel instead) when the table would be larger, cannot be
-// allocated, or is not there yet inside a stream capture.  A program that changes its sources on every call
+// allocated, or is not there yet inside a stream capture.  A workspace that finds no room takes the table's (ensure_ws).  A program that changes its sources on every call
 // rebuilds the table.  Microseconds per call with the per-voxel evaluation, with the table rebuilt on every call and with
 // an earlier call's table: FP64, 256^2 x 64, eight sources of five points 10558, 8788, 2851; FP64, 32^2 x 16, one source
 // 76, 62, 35; FP32, 512^2 x 32, four sources 415, 370, 277; FP32, 512^2 x 51, one source 203, 194, 138.
@@ -114,17 +114,15 @@ template <typename T> int weights_or_null(Handle* H, const fr3d_sources* s, cons
   FR3D_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
   if (need > kWeightBytes || cs != cudaStreamCaptureStatusNone) return FR3D_OK;
   if (cap < need) {
-    if (tab) cudaFree(tab);
+    dev_free(tab, cap);
     tab = nullptr;
     cap = 0;
     key.clear();
-    const cudaError_t e = cudaMalloc(&tab, need);
-    if (e == cudaErrorMemoryAllocation) {
-      cudaGetLastError();
-      tab = nullptr;
-      return FR3D_OK;
-    }
-    FR3D_CUDA_TRY(e);
+    void* p = nullptr;
+    const int rc = dev_alloc(&p, need);
+    if (rc == FR3D_ERR_OOM) return FR3D_OK;
+    FR3D_TRY(rc);
+    tab = static_cast<T*>(p);
     cap = need;
   }
   key.clear();

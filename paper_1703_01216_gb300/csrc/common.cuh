@@ -172,6 +172,11 @@ struct Launches {
 };
 
 int ensure_ws(Handle* H, size_t bytes);
+bool fused_supported(int n);
+// Device memory that may be short (workspaces, optional tables, plans' buffers): FR3D_OK, FR3D_ERR_OOM or FR3D_ERR_CUDA,
+// and its return.  Subject to fr3d_test_alloc_budget.
+int dev_alloc(void** p, size_t bytes);
+void dev_free(void* p, size_t bytes);
 
 // Opt a kernel in to `bytes` of dynamic shared memory (beyond the 48 KB default that static and
 // dynamic shared memory share) once per (kernel, device); later calls are a lookup, so launches

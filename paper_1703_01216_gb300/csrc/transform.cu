@@ -10,6 +10,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <new>
 #include <utility>
@@ -180,14 +181,59 @@ int smem_optin(const void* kernel, size_t bytes) {
   return FR3D_OK;
 }
 
+namespace {
+std::atomic<long long> g_budget{-1};   // fr3d_test_alloc_budget: bytes left, or -1: no budget
+std::atomic<int> g_attempts{0};
+}  // namespace
+
+int dev_alloc(void** p, size_t bytes) {
+  *p = nullptr;
+  ++g_attempts;
+  const bool limited = g_budget.load() >= 0;
+  if (limited && g_budget.load() < (long long)bytes) return FR3D_ERR_OOM;
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) {
+    *p = nullptr;
+    if (e != cudaErrorMemoryAllocation) return FR3D_ERR_CUDA;
+    cudaGetLastError();   // not sticky
+    return FR3D_ERR_OOM;
+  }
+  if (limited) g_budget -= (long long)bytes;
+  return FR3D_OK;
+}
+
+void dev_free(void* p, size_t bytes) {
+  if (!p) return;
+  cudaFree(p);
+  if (g_budget.load() >= 0) g_budget += (long long)bytes;
+}
+
+// Give back what the handle can do without: the combination weights of the unfused row pass, which then evaluates V0 per
+// voxel.  True if there was any.
+static bool drop_optional(Handle* H) {
+  bool any = H->wtab64 != nullptr;
+  dev_free(H->wtab64, H->wtab64_cap);
+  H->wtab64 = nullptr;
+  H->wtab64_cap = 0;
+  H->wtab64_key.clear();
+  if (!fused_supported(H->n) && H->wtab) {
+    any = true;
+    dev_free(H->wtab, H->wtab_cap);
+    H->wtab = nullptr;
+    H->wtab_cap = 0;
+    H->wtab_key.clear();
+  }
+  return any;
+}
+
 int ensure_ws(Handle* H, size_t bytes) {
   if (bytes <= H->ws_bytes) return FR3D_OK;
-  if (H->ws) {
-    cudaFree(H->ws);
-    H->ws = nullptr;
-    H->ws_bytes = 0;
-  }
-  FR3D_CUDA_TRY(cudaMalloc(&H->ws, bytes));
+  dev_free(H->ws, H->ws_bytes);
+  H->ws = nullptr;
+  H->ws_bytes = 0;
+  int rc = dev_alloc(&H->ws, bytes);
+  if (rc == FR3D_ERR_OOM && drop_optional(H)) rc = dev_alloc(&H->ws, bytes);
+  FR3D_TRY(rc);
   H->ws_bytes = bytes;
   return FR3D_OK;
 }
@@ -403,5 +449,11 @@ extern "C" int fr3d_handle_query(fr3d_handle* h, int* n, int* m, int* mp, double
   if (m) *m = h->h.M;
   if (mp) *mp = h->h.Mp;
   if (s2) *s2 = h->h.s2_host;
+  return FR3D_OK;
+}
+
+extern "C" int fr3d_test_alloc_budget(long long bytes, int* attempts) {
+  if (attempts) *attempts = fr3d::g_attempts.exchange(0);
+  fr3d::g_budget = bytes < 0 ? -1 : bytes;
   return FR3D_OK;
 }

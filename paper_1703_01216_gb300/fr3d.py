@@ -72,7 +72,7 @@ EXPORTS = ("fr3d_kernel_transform", "fr3d_handle_destroy", "fr3d_handle_query", 
            "fr3d_mlp_create", "fr3d_mlp_destroy", "fr3d_mlp_query", "fr3d_mlp_get_params", "fr3d_mlp_set_params",
            "fr3d_mlp_forward", "fr3d_mlp_gradient", "fr3d_mlp_train_step", "fr3d_band_features",
            "fr3d_band_alpha_targets", "fr3d_autotune_mode", "fr3d_autotune_query",
-           "fr3d_test_withhold_queue_counts", "fr3d_assemble_rhs",
+           "fr3d_test_withhold_queue_counts", "fr3d_test_alloc_budget", "fr3d_assemble_rhs",
            "fr3d_unet_create", "fr3d_unet_destroy", "fr3d_unet_query", "fr3d_unet_get_params", "fr3d_unet_set_params",
            "fr3d_unet_forward", "fr3d_unet_gradient", "fr3d_unet_train_step", "fr3d_unet_error_flags")
 
@@ -121,6 +121,7 @@ def load(path: str | None = None):
     lib.fr3d_autotune_mode.argtypes = [i]
     lib.fr3d_autotune_query.argtypes = [vp, ct.POINTER(i), ct.POINTER(ct.c_float), i]
     lib.fr3d_test_withhold_queue_counts.argtypes = [i]
+    lib.fr3d_test_alloc_budget.argtypes = [ct.c_longlong, ct.POINTER(i)]
     lib.fr3d_assemble_rhs.argtypes = [vp, vp, i, ct.POINTER(Sources), d, d, i, d, vp, vp]
     lib.fr3d_unet_create.argtypes = [i, i, i, i, ct.c_float, ct.c_ulonglong, ct.POINTER(vp)]
     lib.fr3d_unet_destroy.argtypes = [vp]
@@ -407,6 +408,13 @@ def test_withhold_queue_counts(on: bool) -> bool:
     """Test hook of the tile-queue variant's bounded waits (fr3d_test_withhold_queue_counts): while on, its
     row tiles' waits run out and the call reports FR3D_INFO_TIMEOUT.  Returns the previous setting."""
     return bool(load().fr3d_test_withhold_queue_counts(1 if on else 0))
+
+
+def test_alloc_budget(nbytes: int = -1) -> int:
+    """Test hook of the paths for a full device (fr3d_test_alloc_budget); the requests made since the last call."""
+    n = ct.c_int()
+    _check(load().fr3d_test_alloc_budget(int(nbytes), ct.byref(n)), "fr3d_test_alloc_budget")
+    return int(n.value)
 
 
 class Mlp:

@@ -1,0 +1,66 @@
+"""Calls on a device without room (fr3d_test_alloc_budget makes requests fail as if it were full): what a handle or a plan
+can do without is given up before a call fails, and results stay those of a call with room."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1703_01216_gb300 import inputs as I  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def F():
+    from paper_1703_01216_gb300 import fr3d
+    prev = fr3d.autotune_mode()
+    yield fr3d
+    fr3d.test_alloc_budget(-1)
+    fr3d.autotune_mode(prev)
+
+
+def least(F, call, step, top):
+    """The smallest budget (a multiple of step) with which call(budget) does not run out of memory."""
+    for b in range(0, top, step):
+        try:
+            call(b)
+            return b
+        except F.Fr3dError:
+            pass
+        finally:
+            F.test_alloc_budget(-1)
+    raise AssertionError("no budget was enough")
+
+
+@pytest.mark.parametrize("n,prec,mp", [(64, 1, 8), (512, 0, 3)])
+def test_weights_make_room_for_the_workspace(F, n, prec, mp):
+    dt = torch.float64 if prec == F.PREC_FP64 else torch.float32
+    w = I.make_workload(n, mp, q=3, n_incl=1, seed=71)
+    U = torch.as_tensor(w.noise, dtype=dt, device="cuda")
+    pts = np.asarray(w.sources)
+    ref = torch.empty((mp, n, n), dtype=dt, device="cuda")
+    F.invert(F.kernel_transform(n, w.x0, w.h, w.zr, w.zy, w.nu), U, 3, ref, F.Opts(alpha=1e-2, precision=prec, points=pts))
+    outs = []
+
+    def grow(first):
+        def call(budget):
+            H = F.kernel_transform(n, w.x0, w.h, w.zr, w.zy, w.nu)
+            if first == "xi":   # one source's weights are kept
+                F.invert(H, U[:1].contiguous(), 1, torch.empty_like(ref), F.Opts(alpha=1e-2, precision=prec, points=pts[:1]))
+            else:
+                z = torch.empty((1, mp, n, n), dtype=dt, device="cuda")
+                F.invert(H, U[:1].contiguous(), 1, z, F.Opts(alpha=1e-2, precision=prec, output=F.OUT_ZETA))
+            torch.cuda.synchronize()
+            F.test_alloc_budget(budget)
+            out = torch.empty_like(ref)
+            F.invert(H, U, 3, out, F.Opts(alpha=1e-2, precision=prec, points=pts))
+            torch.cuda.synchronize()
+            outs.append(out)
+        return call
+
+    table = U.element_size() * mp * n * n
+    step = table // 8
+    kept, none = (least(F, grow(first), step, 64 * table) for first in ("xi", "zeta"))
+    assert kept <= none - table + step, (kept, none, table)
+    for out in outs:   # (the weights may be evaluated per voxel: a few ulp)
+        assert float((out - ref).norm()) <= 32 * torch.finfo(dt).eps * float(ref.norm())
