@@ -104,6 +104,7 @@ template <typename T> int weights_or_null(Handle* H, const fr3d_sources* s, cons
   }();
   std::vector<double>& key = sizeof(T) == 4 ? H->wtab_key : H->wtab64_key;
   size_t& cap = sizeof(T) == 4 ? H->wtab_cap : H->wtab64_cap;
+  std::vector<double>& denied = sizeof(T) == 4 ? H->wtab_denied : H->wtab64_denied;
   *W = nullptr;
   if (tab && key == H->src_key) {
     *W = tab;
@@ -112,7 +113,7 @@ template <typename T> int weights_or_null(Handle* H, const fr3d_sources* s, cons
   const size_t need = sizeof(T) * (size_t)s->q * H->Mp * H->n * H->n;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   FR3D_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
-  if (need > kWeightBytes || cs != cudaStreamCaptureStatusNone) return FR3D_OK;
+  if (need > kWeightBytes || cs != cudaStreamCaptureStatusNone || denied == H->src_key) return FR3D_OK;
   if (cap < need) {
     dev_free(tab, cap);
     tab = nullptr;
@@ -120,7 +121,10 @@ template <typename T> int weights_or_null(Handle* H, const fr3d_sources* s, cons
     key.clear();
     void* p = nullptr;
     const int rc = dev_alloc(&p, need);
-    if (rc == FR3D_ERR_OOM) return FR3D_OK;
+    if (rc == FR3D_ERR_OOM) {   // every further call with these sources would only wait for the allocator
+      denied = H->src_key;
+      return FR3D_OK;
+    }
     FR3D_TRY(rc);
     tab = static_cast<T*>(p);
     cap = need;

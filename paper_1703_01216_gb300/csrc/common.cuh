@@ -82,6 +82,7 @@ struct Handle {
   double* wtab64 = nullptr;   // the same in FP64 (FP64 calls)
   std::vector<double> wtab64_key;
   size_t wtab64_cap = 0;
+  std::vector<double> wtab_denied, wtab64_denied;   // sources whose table found no room: not asked for again
   double* pts64 = nullptr;    // [Q*L*3]
   int src_cap = 0;
   // small device words

@@ -64,3 +64,26 @@ def test_weights_make_room_for_the_workspace(F, n, prec, mp):
     assert kept <= none - table + step, (kept, none, table)
     for out in outs:   # (the weights may be evaluated per voxel: a few ulp)
         assert float((out - ref).norm()) <= 32 * torch.finfo(dt).eps * float(ref.norm())
+
+
+def test_weights_without_room_are_asked_for_once_per_source_set(F):
+    n, mp = 48, 4
+    w = I.make_workload(n, mp, q=2, n_incl=1, seed=72)
+    pts = np.asarray(w.sources)
+    U = torch.as_tensor(w.noise, dtype=torch.float64, device="cuda")
+    out, z = torch.empty((mp, n, n), dtype=U.dtype, device="cuda"), torch.empty((2, mp, n, n), dtype=U.dtype, device="cuda")
+    H = F.kernel_transform(n, w.x0, w.h, w.zr, w.zy, w.nu)
+    F.invert(H, U, 2, z, F.Opts(alpha=1e-2, precision=F.PREC_FP64, output=F.OUT_ZETA))   # the workspace
+    F.test_alloc_budget(0)
+    for p in (pts, pts + 0.01):
+        for k in range(4):
+            F.invert(H, U, 2, out, F.Opts(alpha=1e-2, precision=F.PREC_FP64, points=p))
+            assert F.test_alloc_budget(0) == (1 if k == 0 else 0)
+    torch.cuda.synchronize()
+    voxel = out.clone()
+    F.test_alloc_budget(-1)
+    for p in (pts, pts + 0.01):   # other sources ask again, and then find room for these too
+        F.invert(H, U, 2, out, F.Opts(alpha=1e-2, precision=F.PREC_FP64, points=p))
+    torch.cuda.synchronize()
+    assert F.test_alloc_budget(-1) == 1
+    assert float((out - voxel).norm()) <= 32 * torch.finfo(U.dtype).eps * float(voxel.norm())
