@@ -113,8 +113,9 @@ template <typename T> int weights_or_null(Handle* H, const fr3d_sources* s, cons
   const size_t need = sizeof(T) * (size_t)s->q * H->Mp * H->n * H->n;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   FR3D_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
-  if (need > kWeightBytes || cs != cudaStreamCaptureStatusNone || denied == H->src_key) return FR3D_OK;
+  if (need > kWeightBytes || cs != cudaStreamCaptureStatusNone) return FR3D_OK;
   if (cap < need) {
+    if (denied == H->src_key) return FR3D_OK;
     dev_free(tab, cap);
     tab = nullptr;
     cap = 0;

@@ -86,4 +86,8 @@ def test_weights_without_room_are_asked_for_once_per_source_set(F):
         F.invert(H, U, 2, out, F.Opts(alpha=1e-2, precision=F.PREC_FP64, points=p))
     torch.cuda.synchronize()
     assert F.test_alloc_budget(-1) == 1
+    tabled = torch.empty_like(out)
+    F.invert(F.kernel_transform(n, w.x0, w.h, w.zr, w.zy, w.nu), U, 2, tabled, F.Opts(alpha=1e-2, precision=F.PREC_FP64, points=pts + 0.01))
+    torch.cuda.synchronize()
+    assert torch.equal(out, tabled)
     assert float((out - voxel).norm()) <= 32 * torch.finfo(U.dtype).eps * float(voxel.norm())
