@@ -306,10 +306,10 @@ int reserve_invert(Handle* H, int Q, bool host_io, int output, InvertPlan* p) {
   *p = plan_invert<T>(H, Q, host_io, output, bins);
   const int rc = ensure_ws(H, p->total);
   if (rc != FR3D_ERR_OOM || !bins) return rc;
-  cudaGetLastError();
-  H->no_bins = true;
   *p = plan_invert<T>(H, Q, host_io, output, false);
-  return ensure_ws(H, p->total);
+  FR3D_TRY(ensure_ws(H, p->total));
+  H->no_bins = true;   // (a call that fits in neither order says nothing about the next)
+  return FR3D_OK;
 }
 
 int check_invert_args(Handle* H, int Q, const fr3d_invert_opts* o) {

@@ -687,10 +687,9 @@ int choose_multi(Handle* H, const float* U, int Q, const double* alphas, int na,
   bool bins = multi_bins(H);
   int rc = ensure_ws(H, multi_layout(H, Q, bins, bins, nullptr).total);
   if (rc == FR3D_ERR_OOM && bins) {
-    cudaGetLastError();
-    H->no_bins = true;
     bins = false;
     rc = ensure_ws(H, multi_layout(H, Q, false, false, nullptr).total);
+    H->no_bins = rc == FR3D_OK;   // (a call that fits in neither order says nothing about the next)
   }
   FR3D_TRY(rc);
   const MultiWs w = multi_layout(H, Q, bins, bins, (char*)H->ws);

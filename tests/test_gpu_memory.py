@@ -91,3 +91,71 @@ def test_weights_without_room_are_asked_for_once_per_source_set(F):
     torch.cuda.synchronize()
     assert torch.equal(out, tabled)
     assert float((out - voxel).norm()) <= 32 * torch.finfo(U.dtype).eps * float(voxel.norm())
+
+
+def spectra(n, planes):
+    return 8 * planes * (n // 2 + 1) * n
+
+
+@pytest.mark.parametrize("n,m,mp,prec", [(192, 2, 5, 0), (192, 5, 2, 3), (256, 4, 7, 0), (384, 3, 1, 0), (512, 2, 6, 3)])
+def test_plane_order_where_bin_order_finds_no_room(F, n, m, mp, prec):
+    """Several observation depths: both orders project and solve the same spectra with the same kernels, so that what
+    differs is the rounding of the inverse transform (FP32, a few 1e-7; 1e-5 as between the inverse's other forms)."""
+    w = I.make_workload(n, mp, q=1, m_obs=m, n_incl=2, n_alpha=8, seed=73)
+    U = torch.as_tensor(w.noise, dtype=torch.float32, device="cuda")
+    opts = F.Opts(alpha=1e-2, output=F.OUT_ZETA, precision=prec)
+
+    def handle():
+        return F.kernel_transform(n, w.x0, w.h, w.zr, w.zy, w.nu)
+
+    def run(H):
+        out = torch.full((1, mp, n, n), float("nan"), device="cuda")
+        F.invert(H, U, 1, out, opts)
+        torch.cuda.synchronize()
+        return out
+
+    ref, got = run(handle()), []
+
+    def call(budget):
+        H = handle()
+        F.test_alloc_budget(budget)
+        got.append((run(H), H))
+
+    b = least(F, call, spectra(n, 1) // 2, 1 << 30)
+    assert b < spectra(n, 2 * max(m, mp))      # what bin order takes
+    out, H = got[0]
+    assert float((out - ref).norm()) <= 1e-5 * float(ref.norm())
+    again = run(H)                             # the layout stays
+    assert torch.equal(again, out)
+    idx, res = torch.zeros(1, dtype=torch.int32, device="cuda"), {}
+    for name, budget in (("plane", b), ("bin", -1)):   # the alpha rule alone, in both orders
+        H2 = handle()
+        F.test_alloc_budget(budget if name == "bin" else spectra(n, m) + 8 * m * (n // 2 + 1) * (n // 2 + 2) // 2 + 1024)
+        res[name] = torch.zeros(8, dtype=torch.float64, device="cuda")
+        F.choose_alpha(H2, U, 1, w.alphas, 0.5 * float(U.norm()), 1.1, idx, res[name], precision=prec)
+        torch.cuda.synchronize()
+        F.test_alloc_budget(-1)
+    assert torch.equal(res["plane"], res["bin"])
+
+
+def test_a_call_that_fits_in_no_order_leaves_the_handle_in_bin_order(F):
+    n, m, mp = 192, 3, 6
+    w = I.make_workload(n, mp, q=4, m_obs=m, n_incl=1, n_alpha=8, seed=74)
+    U = torch.as_tensor(w.noise, dtype=torch.float32, device="cuda")
+    out = {}
+    for name in ("fresh", "after"):
+        H = F.kernel_transform(n, w.x0, w.h, w.zr, w.zy, w.nu)
+        if name == "after":
+            F.test_alloc_budget(spectra(n, m + mp))
+            with pytest.raises(F.Fr3dError):
+                F.invert(H, U, 4, torch.empty((4, mp, n, n), device="cuda"), F.Opts(alpha=1e-2, output=F.OUT_ZETA))
+            F.test_alloc_budget(0)
+            with pytest.raises(F.Fr3dError):
+                F.choose_alpha(H, U, 4, w.alphas, 1.0, 1.1, torch.zeros(1, dtype=torch.int32, device="cuda"))
+            F.test_alloc_budget(-1)
+        out[name] = torch.empty((1, mp, n, n), device="cuda")
+        F.invert(H, U[:1].contiguous(), 1, out[name], F.Opts(alpha=1e-2, output=F.OUT_ZETA))
+        out[name + " launches"] = F.last_launch_count(H)
+    torch.cuda.synchronize()
+    assert out["fresh launches"] == out["after launches"]   # (plane order runs the fused inverse at this size)
+    assert torch.equal(out["fresh"], out["after"])
