@@ -144,6 +144,7 @@ struct Batch {
   std::vector<int*> info;          // words to clear (unruled_info)
   unsigned char* dev = nullptr;
   unsigned char* qbuf = nullptr;   // the tile queue's counters and intermediates (zeroed once)
+  size_t qbytes = 0;
   int output = FR3D_OUT_XI;
   int launches = 0;
 };
@@ -196,11 +197,11 @@ namespace fr3d {
 namespace {
 
 // Descriptor tables of the groups (host image; device offsets relative to the table's start).
-// qbuf: the plan's queue buffer (device), or null (no tile queue: the one-shot workspace form).
+// qbuf: the plan's queue buffer (device) for the groups from qmin on, or null (no tile queue: the one-shot form).
 void build_descriptors(const fr3d_instance* inst, const std::map<int, std::vector<int>>& by_n,
                        const std::vector<float2*>& uh, const std::vector<const float*>& dd,
                        const std::vector<const int*>& ai, std::vector<unsigned char>& host, std::vector<Group>& groups,
-                       AlphaPlan& ap, unsigned char* qbuf = nullptr) {
+                       AlphaPlan& ap, unsigned char* qbuf = nullptr, int qmin = 0) {
   std::vector<AlphaInst> alph;
   auto put = [&](const void* p, size_t bytes) {
     const size_t off = al(host.size());
@@ -254,7 +255,7 @@ void build_descriptors(const fr3d_instance* inst, const std::map<int, std::vecto
     }
     g.nplanes = (int)planes.size();
     g.nclusters = (int)map.size();
-    if (qbuf && queue_group(g.n, inst[kv.second[0]].opts->output)) {
+    if (qbuf && g.n >= qmin && queue_group(g.n, inst[kv.second[0]].opts->output)) {
       // [4 launch counters][2 M' depth counters per instance][intermediates, 256-byte aligned]
       int depths = 0;
       for (int idx : kv.second) depths += inst[idx].handle->h.Mp;
@@ -286,11 +287,11 @@ void build_descriptors(const fr3d_instance* inst, const std::map<int, std::vecto
   ap.off = alph.empty() ? 0 : put(alph.data(), alph.size() * sizeof(AlphaInst));
 }
 
-// bytes of the plan's queue buffer (the tile queues of its groups of a supported size, xi output), 0 if none
-size_t queue_bytes(const fr3d_instance* inst, const std::map<int, std::vector<int>>& by_n) {
+// bytes of the plan's queue buffer (the tile queues of its groups of a supported size from qmin on, xi output), 0 if none
+size_t queue_bytes(const fr3d_instance* inst, const std::map<int, std::vector<int>>& by_n, int qmin) {
   size_t b = 0;
   for (auto& kv : by_n) {
-    if (!queue_group(kv.first, inst[kv.second[0]].opts->output)) continue;
+    if (kv.first < qmin || !queue_group(kv.first, inst[kv.second[0]].opts->output)) continue;
     size_t ncnt = 0;
     for (int idx : kv.second) ncnt += 2 * (size_t)inst[idx].handle->h.Mp;
     b += al(sizeof(int) * (4 + ncnt));
@@ -327,26 +328,29 @@ extern "C" int fr3d_batch_create(const fr3d_instance* inst, int n, fr3d_batch** 
   FR3D_TRY(batch_prepare(inst, n, false, uh, dd, ai, by_n, &spectra, st));
   Batch b;
   b.output = inst[0].opts->output;
-  const size_t qb = queue_bytes(inst, by_n);
-  if (qb > 0) {
-    cudaError_t e = cudaMalloc(&b.qbuf, qb);
-    if (e == cudaErrorMemoryAllocation) {   // no room for the intermediates: the plan runs the fused tiles
-      cudaGetLastError();
-      b.qbuf = nullptr;
-      e = cudaSuccess;
-    } else if (e == cudaSuccess) {
-      e = cudaMemsetAsync(b.qbuf, 0, qb, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    }
+  // Where the intermediates of every group find no room, those of the larger grids alone (the fused tiles of the small
+  // ones lose least), else none: a group without them runs the fused tiles.
+  int qmin = 0;
+  for (auto it = by_n.begin(); it != by_n.end() && !b.qbuf; ++it) {
+    qmin = it->first;
+    b.qbytes = queue_bytes(inst, by_n, qmin);
+    if (b.qbytes == 0) break;
+    void* p = nullptr;
+    const int rc = dev_alloc(&p, b.qbytes);
+    if (rc == FR3D_ERR_OOM) continue;
+    FR3D_TRY(rc);
+    b.qbuf = static_cast<unsigned char*>(p);
+    cudaError_t e = cudaMemsetAsync(b.qbuf, 0, b.qbytes, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
-      cudaFree(b.qbuf);
+      dev_free(b.qbuf, b.qbytes);
       return FR3D_ERR_CUDA;
     }
   }
   std::vector<unsigned char> host;
-  build_descriptors(inst, by_n, uh, dd, ai, host, b.groups, b.alpha, b.qbuf);
+  build_descriptors(inst, by_n, uh, dd, ai, host, b.groups, b.alpha, b.qbuf, qmin);
   if (cudaMalloc(&b.dev, al(host.size())) != cudaSuccess) {
-    cudaFree(b.qbuf);
+    dev_free(b.qbuf, b.qbytes);
     return FR3D_ERR_OOM;
   }
   {
@@ -354,7 +358,7 @@ extern "C" int fr3d_batch_create(const fr3d_instance* inst, int n, fr3d_batch** 
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
       cudaFree(b.dev);
-      cudaFree(b.qbuf);
+      dev_free(b.qbuf, b.qbytes);
       return FR3D_ERR_CUDA;
     }
   }
@@ -363,7 +367,7 @@ extern "C" int fr3d_batch_create(const fr3d_instance* inst, int n, fr3d_batch** 
   fr3d_batch* h = new (std::nothrow) fr3d_batch();
   if (!h) {
     cudaFree(b.dev);
-    cudaFree(b.qbuf);
+    dev_free(b.qbuf, b.qbytes);
     return FR3D_ERR_OOM;
   }
   h->b = std::move(b);
@@ -421,7 +425,7 @@ extern "C" void fr3d_batch_destroy(fr3d_batch* h) {
   if (!h) return;
   cudaDeviceSynchronize();
   cudaFree(h->b.dev);
-  cudaFree(h->b.qbuf);
+  fr3d::dev_free(h->b.qbuf, h->b.qbytes);
   delete h;
 }
 

@@ -159,3 +159,40 @@ def test_a_call_that_fits_in_no_order_leaves_the_handle_in_bin_order(F):
     torch.cuda.synchronize()
     assert out["fresh launches"] == out["after launches"]   # (plane order runs the fused inverse at this size)
     assert torch.equal(out["fresh"], out["after"])
+
+
+def test_a_plan_keeps_the_queue_of_the_grids_that_find_room(F):
+    """Which groups run the queue shows in their info words while the queue's counts are withheld (its bounded waits give
+    up; the fused tiles of the other groups do not wait)."""
+    items, refs, infos = [], [], []
+    for k, (n, mp, q) in enumerate([(96, 5, 2), (256, 3, 1), (96, 2, 1), (256, 2, 2)]):
+        w = I.make_workload(n, mp, q=q, n_incl=1, n_alpha=12, seed=820 + k)
+        H = F.kernel_transform(n, w.x0, w.h, w.zr, w.zy, w.nu)
+        U = torch.as_tensor(w.noise, dtype=torch.float32, device="cuda")
+        infos.append(torch.zeros(1, dtype=torch.int32, device="cuda"))
+        opts = F.Opts(alphas=w.alphas, delta=0.3 * float(U.norm()), points=w.sources, info=infos[-1])
+        items.append((H, U, q, opts, torch.empty((mp, n, n), device="cuda")))
+    plan = F.Batch(items)
+    F.autotune_mode(2 + 3)
+    plan.run()
+    torch.cuda.synchronize()
+    refs = [it[4].clone() for it in items]
+    plan.close()
+    F.autotune_mode(2 + 5)
+    large = 4 * 256 * 256 * (3 * 1 + 2 * 2) + 4096
+    for budget, queued in ((1 << 30, {96, 256}), (large, {256}), (1 << 12, set())):
+        F.test_alloc_budget(budget)
+        plan = F.Batch(items)
+        F.test_alloc_budget(-1)
+        F.test_withhold_queue_counts(True)
+        plan.run()
+        torch.cuda.synchronize()
+        F.test_withhold_queue_counts(False)
+        for it, i in zip(items, infos):
+            assert bool(int(i) & F.INFO_TIMEOUT) == (it[0].n in queued), (budget, it[0].n)
+            it[4].fill_(float("nan"))
+        plan.run()
+        torch.cuda.synchronize()
+        for it, ref, i in zip(items, refs, infos):
+            assert torch.equal(it[4], ref) and not int(i) & F.INFO_TIMEOUT
+        plan.close()
