@@ -151,15 +151,39 @@ int fwd_impl(Handle* H, const T* zeta, int Q, T* U, cudaStream_t st) {
   const int n = H->n, M = H->M, Mp = H->Mp;
   const long ps = (long)(n / 2 + 1) * n;
   const size_t per = sizeof(C) * ps * Mp;
-  const int g = (int)std::max<size_t>(1, std::min<size_t>(std::min(Q, kMaxGridY / std::max(M, Mp)), kFwdBytes / per));
-  const int chunks = M == 1 ? Ops<T>::contract_chunks(H, g) : 0;
-  // sources per inverse pass: all of them, unless their partials or the launch grid say otherwise
-  const int gs = (int)std::max<size_t>(g, std::min<size_t>(std::min(Q, kMaxGridY / M), kFwdBytes / (sizeof(C) * ps * std::max(M, chunks))));
-  const size_t zb = align_up(per * g), pb = align_up(sizeof(C) * ps * gs * chunks), ub = align_up(sizeof(C) * ps * gs * M);
-  FR3D_TRY(ensure_ws(H, zb + pb + ub));
+  // sources per group and per inverse pass (all of them, unless their partials or the launch grid say otherwise), depth
+  // chunks, and the workspace: the group's planes, the partials, the data spectra
+  struct Plan {
+    int g, gs, chunks;
+    size_t zb, pb, total;
+  };
+  auto plan = [&](bool least) {
+    Plan p;
+    p.g = least ? 1 : (int)std::max<size_t>(1, std::min<size_t>(std::min(Q, kMaxGridY / std::max(M, Mp)), kFwdBytes / per));
+    p.chunks = M != 1 ? 0 : (least ? 1 : Ops<T>::contract_chunks(H, p.g));
+    const size_t room = kFwdBytes / (sizeof(C) * ps * std::max(M, p.chunks));
+    p.gs = least ? 1 : (int)std::max<size_t>(p.g, std::min<size_t>(std::min(Q, kMaxGridY / M), room));
+    p.zb = align_up(per * p.g);
+    p.pb = p.chunks > 1 ? align_up(sizeof(C) * ps * p.gs * p.chunks) : 0;   // (one chunk: summed in place)
+    p.total = p.zb + p.pb + align_up(sizeof(C) * ps * p.gs * M);
+    return p;
+  };
+  // One source at a time where the groups find no room, or inside a capture with the workspace of a smaller call
+  Plan pl = plan(false);
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  FR3D_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
+  const bool fixed = cs != cudaStreamCaptureStatusNone && pl.total > H->ws_bytes;
+  const int rc = fixed ? FR3D_ERR_OOM : ensure_ws(H, pl.total);
+  if (rc == FR3D_ERR_OOM) {
+    pl = plan(true);
+    FR3D_TRY(ensure_ws(H, pl.total));
+  } else {
+    FR3D_TRY(rc);
+  }
+  const int g = pl.g, gs = pl.gs, chunks = pl.chunks;
   C* Zh = reinterpret_cast<C*>(H->ws);
-  C* part = reinterpret_cast<C*>((char*)H->ws + zb);
-  C* Uh = reinterpret_cast<C*>((char*)H->ws + zb + pb);
+  C* Uh = reinterpret_cast<C*>((char*)H->ws + pl.zb + pl.pb);
+  C* part = chunks > 1 ? reinterpret_cast<C*>((char*)H->ws + pl.zb) : Uh;
   const T* A;
   if constexpr (sizeof(T) == 4) A = H->A32;
   else {

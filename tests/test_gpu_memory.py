@@ -196,3 +196,38 @@ def test_a_plan_keeps_the_queue_of_the_grids_that_find_room(F):
         for it, ref, i in zip(items, refs, infos):
             assert torch.equal(it[4], ref) and not int(i) & F.INFO_TIMEOUT
         plan.close()
+
+
+@pytest.mark.parametrize("n,m,mp,prec", [(64, 1, 6, 0), (96, 2, 5, 0), (48, 1, 16, 1), (256, 1, 9, 0)])
+def test_forward_operator_one_source_at_a_time(F, n, m, mp, prec):
+    """Without room for groups of sources the operator needs the planes of one source, M' + M half spectra, and a capture
+    after a call with fewer sources needs no more; other sums of FP32 terms in another order (1e-5 as in the parity
+    tests; FP64 1e-12)."""
+    dt, tol = (torch.float64, 1e-12) if prec == F.PREC_FP64 else (torch.float32, 1e-5)
+    q = 5
+    w = I.make_workload(n, mp, q=1, m_obs=m, n_incl=1, seed=75)
+    zeta = torch.as_tensor(np.random.default_rng(n).standard_normal((q, mp, n, n)), dtype=dt, device="cuda")
+
+    def handle():
+        return F.kernel_transform(n, w.x0, w.h, w.zr, w.zy, w.nu)
+
+    def out():
+        return torch.full((q, m, n, n), float("nan"), dtype=dt, device="cuda")
+
+    ref, got = out(), out()
+    F.fwd_apply(handle(), zeta, q, ref, prec)
+    one = spectra(n, 1) * zeta.element_size() // 4
+    F.test_alloc_budget((m + mp) * one + 1024)
+    F.fwd_apply(handle(), zeta, q, got, prec)
+    F.test_alloc_budget(-1)
+    torch.cuda.synchronize()
+    assert float((got - ref).norm()) <= tol * float(ref.norm())
+    H, got = handle(), out()
+    F.fwd_apply(H, zeta[:1].contiguous(), 1, torch.empty((1, m, n, n), dtype=dt, device="cuda"), prec)
+    torch.cuda.synchronize()
+    graph, st = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=st):
+        F.fwd_apply(H, zeta, q, got, prec, stream=st)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float((got - ref).norm()) <= tol * float(ref.norm())
