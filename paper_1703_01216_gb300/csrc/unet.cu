@@ -81,7 +81,7 @@ struct Layer {
   int dgrad = 0;                  // 0 none, 1 with the leaky derivative of the input, 2 plain
   size_t img_f = 0, img_b = 0;    // byte offsets of the weight images
   int ng_f = 0, ng_b = 0;         // output channels per CTA of the convolution and of its input gradient
-  WgradArgs wg{};                 // weight-gradient plan (the tensors are filled in per call)
+  WgradArgs wg{};                 // weight-gradient plan of Unet::wg_batch (the tensors are filled in per call)
 };
 
 }  // namespace
@@ -107,7 +107,8 @@ struct Unet {
   size_t img_bytes = 0;
   float* y = nullptr;             // scaled prediction [Bmax][D][H][W]
   float* partials = nullptr;      // weight-gradient partials
-  size_t partial_floats = 0;
+  size_t partial_floats = 0;      // for every batch up to Bmax
+  int wg_batch = 0;               // the batch size that the layers' weight-gradient plans are for
   float* red = nullptr;           // small reduction buffers
   size_t red_floats = 0;
   double* lossbuf = nullptr;      // [Bmax][2] sums, [1] loss
@@ -515,6 +516,16 @@ ConvArgs conv_forward_args(const Unet* U, int k, int B) {
 }
 int conv_forward(const Unet* U, int k, int B, cudaStream_t st) { return conv3_launch(conv_forward_args(U, k, B), st); }
 
+// The weight gradients' plans for batches of B: by the batch that is run, not the network's largest, so that the order of a
+// batch's sums does not depend on the network it runs in.
+int plan_wgrads(Unet* U, int B) {
+  if (U->wg_batch == B) return FR3D_OK;
+  U->wg_batch = 0;
+  for (Layer& Ly : U->layer) FR3D_TRY(wgrad_plan(&Ly.wg, B));
+  U->wg_batch = B;
+  return FR3D_OK;
+}
+
 int conv_backward(Unet* U, int k, int B, cudaStream_t st) {
   const Layer& Ly = U->layer[k];
   // weight and bias gradient: partial sums, then their ordered sum
@@ -595,6 +606,7 @@ int forward(Unet* U, const float* x, int B, const float* t, float* out, cudaStre
 int backward(Unet* U, const float* t, int B, float* loss, cudaStream_t st) {
   const Level& L0 = U->lv[0];
   const int nblk = kLossBlocks;
+  FR3D_TRY(plan_wgrads(U, B));
   k_loss<<<1, kLossThreads, 0, st>>>(U->red, nblk, B, U->lossbuf, loss);
   k_head_backward<<<dim3(nblk, B), kHeadThreads, 0, st>>>(U->t[T_D2], larg(L0), U->y, t, U->params + U->head_off,
                                                           U->in_scale, B, U->lossbuf, U->g[T_D2], U->red);
@@ -757,14 +769,19 @@ extern "C" int fr3d_unet_create(int depth, int height, int width, int max_batch,
       w.zero_pos = L.Vp;
       w.q_first = L.q_first;
       w.q_last = L.q_last;
-      if (!Ly.ng_f || !Ly.ng_b || wgrad_plan(&w, max_batch) != FR3D_OK) rc = FR3D_ERR_UNSUPPORTED_SIZE;
-      pmax = std::max(pmax, wgrad_partial_floats(w, max_batch));
+      // (the largest batch is planned last: its plan is the one that stays)
+      for (int b = 1; b <= max_batch; ++b) {
+        if (!Ly.ng_f || !Ly.ng_b || wgrad_plan(&w, b) != FR3D_OK) rc = FR3D_ERR_UNSUPPORTED_SIZE;
+        if (rc) break;
+        pmax = std::max(pmax, wgrad_partial_floats(w, b));
+      }
     }
     if (rc) break;
     U->head_off = off;
     U->n_params = off + kWidth[0] + 1;
     U->img_bytes = ioff;
     U->partial_floats = pmax;
+    U->wg_batch = max_batch;
     U->red_floats = (size_t)128 * 17 * max_batch;
     const size_t np = (size_t)U->n_params;
     if (cudaMalloc(&U->params, np * 4) != cudaSuccess || cudaMalloc(&U->grads, np * 4) != cudaSuccess ||
