@@ -37,6 +37,7 @@
 #include "ops.cuh"
 #include "tc.cuh"
 #include "unet.cuh"
+#include "wide_sum.cuh"
 
 namespace fr3d {
 
@@ -598,8 +599,8 @@ __global__ void __launch_bounds__(kWgThreads, 2) k_wgrad3(WgradArgs a) {
 }
 
 // dW[o][c][tap] (c < ci) and db[o]: the units' partial sums added in a fixed order (blockDim.y threads per element
-// take every blockDim.y-th unit, then their sums in order).  A thread adds in FP32 with the rounding errors carried
-// along (Knuth's two-sum; what is lost is of order 2^-48): the FP64 conversions and additions were the bound.
+// take every blockDim.y-th unit, then their sums in order).  A thread adds in three FP32 words, which lose less than FP64
+// additions (wide_sum.cuh): those and the conversions were the bound.
 // 29 MB of partials: 42 -> 22 us, 86 MB: 98 -> 58 us, with four times the loads in flight.  Sums that are not finite
 // are added again in FP64, as a chain that leaves FP32's range on the way has to be.  The partials are read with coherent
 // loads: k_wgrad3 may still be writing them when this kernel starts.
@@ -616,15 +617,11 @@ __global__ void __launch_bounds__(kWgRedThreads) k_wgrad_reduce(WgradArgs a, int
   if (ok) {
     const float* p = i < nw ? a.partials + i : a.bias_partials + (i - nw);
     const long ustep = i < nw ? nw : a.Cout;
-    float hi = 0.f, lo = 0.f;
+    WideSum sum;
 #pragma unroll 8
-    for (int u = threadIdx.y; u < nunits; u += blockDim.y) {
-      const float x = __ldcg(p + u * ustep), t = __fadd_rn(hi, x), d = __fsub_rn(t, hi);
-      lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, d)), __fsub_rn(x, d)));
-      hi = t;
-    }
-    s = (double)hi + (double)lo;
-    if (!isfinite(hi) || !isfinite(lo)) {
+    for (int u = threadIdx.y; u < nunits; u += blockDim.y) sum.add(__ldcg(p + u * ustep));
+    s = sum.value();
+    if (!sum.finite()) {
       s = 0.0;
       for (int u = threadIdx.y; u < nunits; u += blockDim.y) s += (double)__ldcg(p + u * ustep);
     }
