@@ -148,9 +148,10 @@ __device__ __forceinline__ long ppos(const LevelArg& L, int d, int h, int w) {
 // set-up (barriers, tensor memory) and their launch run while the kernel before them leaves the SMs (24 and 62 launches:
 // 1024 -> 973 us forward and 3462 -> 3305 us gradient at 128^2 x 32, batch 8; 177 -> 117 and 600 -> 412 us at 24^2 x 8,
 // batch 1).  Each waits for that kernel before its first access to global memory; the others are launched as usual.
-// What that kernel writes is read with coherent loads (__ldcg): the read-only path asks for data that no one writes while
-// the reader runs, and a reader launched programmatically runs before its predecessor has ended.  Tensors that were
-// complete before the predecessor began (the forward activations in the backward pass) keep __ldg.
+// What that kernel writes is read with coherent loads (__ldca: neighbouring lanes share sectors, and the second half of a
+// sector comes from L1): the read-only path asks for data that no one writes while the reader runs, and a reader
+// launched programmatically runs before its predecessor has ended.  Tensors that were complete before the predecessor
+// began (the forward activations in the backward pass) keep __ldg.
 //
 // The elementwise kernels below run one (chunk, depth, row) per blockDim.y lane group and consecutive w per
 // thread, so that the index divisions are per row and in 32 bits (per voxel and in 64 bits they cost more than
@@ -206,7 +207,7 @@ __global__ void k_pool(const unsigned char* __restrict__ src, int s_chunks, int 
     uint4 v[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c)
-      v[c] = __ldcg(vox(src, q.b, s_chunks, soff + q.j, Ls,
+      v[c] = __ldca(vox(src, q.b, s_chunks, soff + q.j, Ls,
                        ppos(Ls, 2 * q.d + (c >> 2), 2 * q.h + ((c >> 1) & 1), 2 * w + (c & 1))));
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
@@ -232,7 +233,7 @@ __global__ void k_up(const unsigned char* __restrict__ src, int s_chunks, LevelA
   const Row q = row_of(B, nc, Ls.D, Ls.H);
   if (!q.ok) return;
   for (int w = threadIdx.x; w < Ld.W; w += blockDim.x) {
-    const uint4 v = __ldcg(vox(src, q.b, s_chunks, q.j, Ls, ppos(Ls, q.d, q.h, w >> 1)));
+    const uint4 v = __ldca(vox(src, q.b, s_chunks, q.j, Ls, ppos(Ls, q.d, q.h, w >> 1)));
 #pragma unroll
     for (int c = 0; c < 4; ++c) *vox(dst, q.b, d_chunks, q.j, Ld, ppos(Ld, 2 * q.d + (c >> 1), 2 * q.h + (c & 1), w)) = v;
   }
@@ -251,7 +252,7 @@ __global__ void k_up_backward(const unsigned char* __restrict__ gd, int d_chunks
     uint4 v[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c)
-      v[c] = __ldcg(vox(gd, q.b, d_chunks, q.j, Ld,
+      v[c] = __ldca(vox(gd, q.b, d_chunks, q.j, Ld,
                        ppos(Ld, 2 * q.d + (c >> 2), 2 * q.h + ((c >> 1) & 1), 2 * w + (c & 1))));
     const long o = ppos(Ls, q.d, q.h, w);
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, m[8];
@@ -282,7 +283,7 @@ __global__ void k_pool_backward(const unsigned char* __restrict__ gp, int p_chun
     const long o = ppos(Lc, q.d, q.h, w);
     uint4* gq = vox(g, q.b, c_chunks, coff + q.j, Lc, o);
     float up[8], sk[8], m[8];
-    unpack8(__ldcg(vox(gp, q.b, p_chunks, q.j, Lp, ppos(Lp, q.d / 2, q.h / 2, w / 2))), up);
+    unpack8(__ldca(vox(gp, q.b, p_chunks, q.j, Lp, ppos(Lp, q.d / 2, q.h / 2, w / 2))), up);
     unpack8(*gq, sk);
     unpack8(__ldg(vox(s, q.b, c_chunks, coff + q.j, Lc, o)), m);
 #pragma unroll
