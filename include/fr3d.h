@@ -370,6 +370,9 @@ int fr3d_unet_gradient(fr3d_unet* net, const float* x, const float* t, int B, fl
 int fr3d_unet_train_step(fr3d_unet* net, const float* x, const float* t, int B, float lr, float* loss,
                          void* stream);
 int fr3d_unet_error_flags(fr3d_unet* net, int* flags);
+/* Test query: how the weight gradient of conv layer `layer` (0 .. 14) splits a batch of B: the units whose partial sums
+ * are added, and the in-plane positions each walks (either pointer may be NULL). */
+int fr3d_test_unet_wgrad_plan(fr3d_unet* net, int layer, int B, int* units, int* span);
 
 /* Right-hand side of Eq. (7) (the form Eq. (3) takes for point sources, Sec. 6) from the measured
  * z-derivative of V2 on the observation depths:

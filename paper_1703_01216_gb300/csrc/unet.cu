@@ -892,6 +892,15 @@ extern "C" int fr3d_unet_train_step(fr3d_unet* net, const float* x, const float*
   return fr3d::build_images(U, st);
 }
 
+extern "C" int fr3d_test_unet_wgrad_plan(fr3d_unet* net, int layer, int B, int* units, int* span) {
+  if (!net || layer < 0 || layer >= fr3d::kNumConv || B < 1 || B > net->u.Bmax) return FR3D_ERR_INVALID_ARG;
+  fr3d::WgradArgs w = net->u.layer[layer].wg;
+  FR3D_TRY(fr3d::wgrad_plan(&w, B));
+  if (units) *units = B * w.nspans * w.nchunks;
+  if (span) *span = w.span;
+  return FR3D_OK;
+}
+
 extern "C" int fr3d_unet_error_flags(fr3d_unet* net, int* flags) {
   if (!net || !flags) return FR3D_ERR_INVALID_ARG;
   FR3D_CUDA_TRY(cudaDeviceSynchronize());

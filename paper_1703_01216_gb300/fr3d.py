@@ -74,7 +74,8 @@ EXPORTS = ("fr3d_kernel_transform", "fr3d_handle_destroy", "fr3d_handle_query", 
            "fr3d_band_alpha_targets", "fr3d_autotune_mode", "fr3d_autotune_query",
            "fr3d_test_withhold_queue_counts", "fr3d_test_alloc_budget", "fr3d_assemble_rhs",
            "fr3d_unet_create", "fr3d_unet_destroy", "fr3d_unet_query", "fr3d_unet_get_params", "fr3d_unet_set_params",
-           "fr3d_unet_forward", "fr3d_unet_gradient", "fr3d_unet_train_step", "fr3d_unet_error_flags")
+           "fr3d_unet_forward", "fr3d_unet_gradient", "fr3d_unet_train_step", "fr3d_unet_error_flags",
+           "fr3d_test_unet_wgrad_plan")
 
 
 def load(path: str | None = None):
@@ -133,6 +134,7 @@ def load(path: str | None = None):
     lib.fr3d_unet_gradient.argtypes = [vp, vp, vp, i, vp, vp, vp]
     lib.fr3d_unet_train_step.argtypes = [vp, vp, vp, i, ct.c_float, vp, vp]
     lib.fr3d_unet_error_flags.argtypes = [vp, ct.POINTER(i)]
+    lib.fr3d_test_unet_wgrad_plan.argtypes = [vp, i, i, ct.POINTER(i), ct.POINTER(i)]
     lib.fr3d_status_string.argtypes = [i]
     lib.fr3d_status_string.restype = ct.c_char_p
     for name in EXPORTS:
@@ -576,6 +578,13 @@ class Unet:
         _need(loss, "loss", dtype=torch.float32, numel=1, optional=True)
         _check(load().fr3d_unet_train_step(self.ptr, _ptr(x), _ptr(t), int(x.shape[0]), float(lr), _ptr(loss),
                                            _stream(stream)), "fr3d_unet_train_step")
+
+    def test_wgrad_plan(self, layer: int, B: int):
+        """(units, span) of a conv layer's weight gradient for a batch of B (fr3d_test_unet_wgrad_plan)."""
+        u, s = ct.c_int(), ct.c_int()
+        _check(load().fr3d_test_unet_wgrad_plan(self.ptr, int(layer), int(B), ct.byref(u), ct.byref(s)),
+               "fr3d_test_unet_wgrad_plan")
+        return u.value, s.value
 
     def error_flags(self) -> int:
         f = ct.c_int()

@@ -1,4 +1,6 @@
-"""Gradients of a batch in networks made for larger batches: the same bits."""
+"""Gradients of a batch in networks made for larger batches (the same bits), and against those of its samples: every way
+of adding the units' partial sums (1, 4, 16 and 32 threads per element) and of walking a unit (one and several
+sub-ranges of 128 positions)."""
 import numpy as np
 import pytest
 
@@ -41,3 +43,30 @@ def test_gradient_bits_do_not_depend_on_the_largest_batch(shape, B, more):
             got = gradient(net, x, t)
             assert all(torch.equal(a, b) for a, b in zip(got, ref))
             gradient(net, xm, tm)
+
+
+@pytest.mark.parametrize("shape,threads", [((32, 64, 64), {1, 4, 16, 32}), ((8, 104, 104), {1, 4, 16})])
+def test_batch_gradient_is_the_mean_of_its_samples(shape, threads):
+    """A batch of 16: the loss is the mean over the samples, and 1 / 16 scales every stored value exactly, so the batch's
+    gradient is the mean of the samples' up to the order of FP32 sums: at most 256 chained accumulations of 2^-23 of the
+    running sum each, 2^-15 of the terms' magnitudes, times 16 for cancellation among them: 2^-11.  A sample alone has
+    fewer than 128 units of one sub-range, which the oracle tests cover.  A lost unit of 528 would be 2^-9 if all units
+    were alike, more if their signs differ."""
+    from paper_1703_01216_gb300 import fr3d as F
+    B = 16
+    net = network(F, shape, B)
+    plans = [net.test_wgrad_plan(k, B) for k in range(15)]
+    assert {32 if u >= 512 else 16 if u >= 128 else 4 if u >= 32 else 1 for u, _ in plans} == threads
+    assert max(s for _, s in plans) >= 384
+    assert all(u < 128 and s == 128 for u, s in (net.test_wgrad_plan(k, 1) for k in range(15)))
+    x, t = data((B, *shape), sum(shape))
+    got = gradient(net, x, t)[0].double()
+    ref = sum(gradient(net, x[b:b + 1].contiguous(), t[b:b + 1].contiguous())[0].double() for b in range(B)) / B
+    at, layers = 0, [(16, 1), (16, 16), (32, 16), (32, 32), (64, 32), (64, 64), (128, 64), (128, 128), (128, 128),
+                     (64, 192), (64, 64), (32, 96), (32, 32), (16, 48), (16, 16)]
+    for co, ci in layers:
+        for n in (co * ci * 27, co):
+            a, b = got[at:at + n], ref[at:at + n]
+            assert float((a - b).norm()) <= 2.0 ** -11 * float(b.norm()), (co, ci, n)
+            at += n
+    assert float((got[at:] - ref[at:]).norm()) <= 2.0 ** -11 * float(ref[at:].norm())
