@@ -319,9 +319,6 @@ __device__ __forceinline__ void class_pq(int c, int& p, int& q) {
   q = c - p * (p + 1) / 2;
 }
 
-__device__ __forceinline__ double sq_abs(float2 v) { return (double)fmaf(v.x, v.x, v.y * v.y); }
-__device__ __forceinline__ double sq_abs(double2 v) { return fma(v.x, v.x, v.y * v.y); }
-
 constexpr int kAlphaThreads = 256;
 constexpr int kAlphaCPB = 64;      // classes per block at most
 constexpr int kAlphaFill = 160;    // blocks that fill the chip (about one per SM)
