@@ -149,6 +149,12 @@ template <typename T>
 int fwd_impl(Handle* H, const T* zeta, int Q, T* U, cudaStream_t st) {
   using C = typename Ops<T>::C;
   const int n = H->n, M = H->M, Mp = H->Mp;
+  // One observation depth: the contraction is fused with the column pass, which saves the transformed columns' way through
+  // L2.  FP64 is bound by its arithmetic and by how many blocks share it instead: with more depths than chunks the separate
+  // passes are faster (us, n = 192: 64 depths, one source 257 fused, 203 separate; four sources 771, 646; 48^2 x 64 79,
+  // 41; 128^2 x 64 with four sources 265, 281), with a chunk per depth the fused one is (192^2 x 4: 54, 55; x 8: 65, 64;
+  // 128^2 x 8 with eight sources 89, 101).
+  const bool fuse = M == 1 && (sizeof(T) == 4 || Mp <= kMaxChunks);
   const long ps = (long)(n / 2 + 1) * n;
   const size_t per = sizeof(C) * ps * Mp;
   // sources per group and per inverse pass (all of them, unless their partials or the launch grid say otherwise), depth
@@ -160,7 +166,7 @@ int fwd_impl(Handle* H, const T* zeta, int Q, T* U, cudaStream_t st) {
   auto plan = [&](bool least) {
     Plan p;
     p.g = least ? 1 : (int)std::max<size_t>(1, std::min<size_t>(std::min(Q, kMaxGridY / std::max(M, Mp)), kFwdBytes / per));
-    p.chunks = M != 1 ? 0 : (least ? 1 : Ops<T>::contract_chunks(H, p.g));
+    p.chunks = !fuse ? 0 : (least ? 1 : Ops<T>::contract_chunks(H, p.g));
     const size_t room = kFwdBytes / (sizeof(C) * ps * std::max(M, p.chunks));
     p.gs = least ? 1 : (int)std::max<size_t>(p.g, std::min<size_t>(std::min(Q, kMaxGridY / M), room));
     p.zb = align_up(per * p.g);
@@ -196,7 +202,7 @@ int fwd_impl(Handle* H, const T* zeta, int Q, T* U, cudaStream_t st) {
     for (int q = 0; q < ns; q += g) {
       const int nq = std::min(g, ns - q);
       FR3D_TRY(Ops<T>::row_r2c(H, zeta + (long)(q0 + q) * Mp * n * n, (long)n * n, Zh, nq * Mp, st));
-      if (M == 1) {
+      if (fuse) {
         FR3D_TRY(Ops<T>::col_contract(H, Zh, part + q * ps, ps * ns, A, nq, chunks, st));
         launches += 2;
       } else {
@@ -205,7 +211,7 @@ int fwd_impl(Handle* H, const T* zeta, int Q, T* U, cudaStream_t st) {
         launches += 3;
       }
     }
-    if (M == 1) FR3D_TRY(Ops<T>::col_sum(H, part, ps * ns, Uh, ns, chunks, st));
+    if (fuse) FR3D_TRY(Ops<T>::col_sum(H, part, ps * ns, Uh, ns, chunks, st));
     else FR3D_TRY(Ops<T>::col_plain(H, Uh, Uh, ns * M, true, st));
     FR3D_TRY(Ops<T>::row_c2r_plain(H, Uh, U + (long)q0 * M * n * n, ns * M, 1, 0, 1, st));
     launches += 2;

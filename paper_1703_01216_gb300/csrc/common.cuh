@@ -172,6 +172,7 @@ struct Launches {
   void add(int k = 1) { n += k; }
 };
 
+constexpr int kMaxChunks = 8;   // depth chunks of the forward contraction at most
 int ensure_ws(Handle* H, size_t bytes);
 bool fused_supported(int n);
 // Device memory that may be short (workspaces, optional tables, plans' buffers): FR3D_OK, FR3D_ERR_OOM or FR3D_ERR_CUDA,

@@ -217,7 +217,6 @@ struct ColTable {
   __device__ float2 load(int, int, int, float2 v) const { return v; }
 };
 
-constexpr int kMaxChunks = 8;   // depth chunks of the forward contraction at most
 // inverse column pass over the sum of S <= kMaxChunks partial spectra, p and p + stride, ..., scaled by `scale`
 template <typename T> struct ColSum {
   using C = typename cpx<T>::t;

@@ -242,14 +242,15 @@ static int col_contract_n(const Handle* H, const typename cpx<T>::t* Zh, typenam
                    tw_of<T>(H, N));
 }
 
-// Depth chunks of the contraction: enough CTAs to fill the SMs (five each at n = 256), at least four depths each, no
+// Depth chunks of the contraction: enough CTAs to fill the SMs (five each at n = 256), at least four depths each (FP64: one;
+// a depth in FP64 takes as long as four; 192^2 x 8: 95 -> 65 us), no
 // empty chunk; more partials than kMaxChunks cost the sum more than the extra CTAs give (16 chunks: 17 us).
 template <typename T>
 int Ops<T>::contract_chunks(const Handle* H, int Q) {
   int tc = (sizeof(T) == 4 ? 2048 : 1024) / H->n;
   tc = std::max(1, std::min(tc, H->n / 2 + 1));
   const int ctas = ((H->n / 2 + tc) / tc) * Q;
-  const int want = std::max(1, std::min({(5 * 152 + ctas - 1) / ctas, H->Mp / 4, kMaxChunks}));
+  const int want = std::max(1, std::min({(5 * 152 + ctas - 1) / ctas, sizeof(T) == 8 ? H->Mp : H->Mp / 4, kMaxChunks}));
   const int per = (H->Mp + want - 1) / want;
   return (H->Mp + per - 1) / per;
 }
