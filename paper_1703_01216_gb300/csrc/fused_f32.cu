@@ -67,7 +67,7 @@ std::map<TuneKey, int> g_tuned;
 
 // variants 0-3: the fused cluster kernel's tiles; 4: the two-pass inverse (inv2p.cu), whose intermediate
 // lives in the handle's inv2 buffer (grown outside stream captures only); 5: the persistent tile queue
-// (inv_queue.cu: n = 256, xi output), through the same intermediate and the handle's queue counters
+// (inv_queue.cu: n = 96, 128, 192, 256, xi output), through the same intermediate and the handle's queue counters
 constexpr int kInvVariants = kFusedVariants + 2;
 
 int ensure_inv2(Handle* H, int Q, int nj, cudaStream_t st, bool* ok) {

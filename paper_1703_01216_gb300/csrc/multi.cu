@@ -519,7 +519,9 @@ size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 // whole records instead of 8-byte values a plane apart, each of which cost a 32-byte sector.  Below it the fused
 // inverse on plane-ordered spectra saves two launches.  Whole inversions: 512^2, M = M' = 51, 516 us in plane order
 // and 449 in bin order (projection 169 -> 131, solve 168 -> 120, the column passes + 6 each); 256^2, M = 40,
-// M' = 64, split BF16, 187 -> 167.
+// M' = 64, split BF16, 187 -> 167.  From n = 192 on it is the faster order with few planes too, where the column passes of
+// 8 to 21 planes per block are mostly empty (M = 2 to 24, M' = 16 to 48, one and two sources, n = 192 to 512, FP32 and split
+// BF16: between 1.005 times at n = 192 with two observation and 32 result depths and 1.5 at 512).
 constexpr int kBinsMinN = 192;
 
 struct MultiWs {

@@ -16,7 +16,8 @@
 // for its maximum batch).  Convolutions and their gradients run on the tensor cores (unet_conv.cu; the last
 // convolution applies the head); pooling, upsampling, the head's gradient, loss, reductions and Adam are the CUDA-core
 // kernels below.  Every reduction
-// has a fixed order (block partials, then one ordered pass), so results do not depend on the run.
+// has a fixed order (block partials, then one ordered pass), so results do not depend on the run, nor on the largest batch
+// a network was made for.
 #include <math.h>
 #include <string.h>
 
