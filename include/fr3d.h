@@ -75,7 +75,8 @@ extern "C" {
                                             the discrepancy rule is the fallback to run) */
 #define FR3D_INFO_TIMEOUT 16             /* a bounded device wait (a tensor-core copy or MMA completion,
                                             or the tile-queue inverse's wait on a release) gave up: the
-                                            outputs of this call are incomplete */
+                                            outputs of this call are incomplete (a batched plan: those of
+                                            every instance whose word has the bit) */
 
 /* ---- enums ---- */
 #define FR3D_K_DZ_INV_R 0 /* K = d/dz (1/r), Eq. (4) (the equation the paper solves) */
@@ -235,7 +236,7 @@ int fr3d_invert_host(fr3d_handle* h, const void* U_host, int Q, const fr3d_inver
  * device pointers and options of the instances are fixed at creation.  fr3d_batch_run only
  * launches kernels (it can be captured in a CUDA graph); with the autotuner on (mode 1, below) its
  * first call outside a capture also times the fused variants and synchronises `stream`, so make
- * that call before capturing.  The paper has no batch form: this is
+ * that call before capturing.  Every run overwrites the instances' info words.  The paper has no batch form: this is
  * Algorithm 1 applied to many independent problems at once. */
 typedef struct fr3d_instance {
   fr3d_handle* handle;            /* geometry and kernel tables (fr3d_kernel_transform) */
