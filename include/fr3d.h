@@ -311,7 +311,7 @@ int fr3d_band_alpha_targets(fr3d_handle* h, const float* U, const float* zeta_tr
  * written once); 4: two streaming passes through an intermediate in a handle-owned buffer; 5: one
  * persistent launch over a queue of column and row tiles through the same intermediate, served from L2
  * (n = 96, 128, 192 and 256 with xi output; other shapes run variant 3).  Variants 4 and 5 allocate their buffer on the
- * first call outside a stream capture (inside a capture before that, they run variant 3).  Modes: 0 = always variant 0; 1 (default) = on the first fr3d_invert of a
+ * first call outside a stream capture (inside a capture before that, and on a handle that found no room for it, they run variant 3).  Modes: 0 = always variant 0; 1 (default) = on the first fr3d_invert of a
  * shape (device, n, M', Q, output) made outside a stream capture, time every variant on that
  * call's own arguments (1 warm-up + 3 timed launches each, synchronising the stream once) and use
  * the fastest from then on, process-wide; 2 + v = always variant v.  A batched plan (mode 1) times

@@ -127,6 +127,7 @@ struct Handle {
   // grown outside captures; the tile queue's counters (zeroed at allocation, left zeroed by every launch)
   float2* inv2_buf = nullptr;
   size_t inv2_cap = 0;
+  size_t inv2_denied = 0;     // size for which the buffer found no room (0: none): not asked for again
   int* qctl = nullptr;
   size_t qctl_n = 0;
   // stage profiling: events recorded between consecutive launches of one call

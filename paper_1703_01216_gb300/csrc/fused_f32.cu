@@ -70,6 +70,7 @@ std::map<TuneKey, int> g_tuned;
 // (inv_queue.cu: n = 96, 128, 192, 256, xi output), through the same intermediate and the handle's queue counters
 constexpr int kInvVariants = kFusedVariants + 2;
 
+// Without room for them (ok = false) the register-accumulator tile runs, with the same bits.
 int ensure_inv2(Handle* H, int Q, int nj, cudaStream_t st, bool* ok) {
   const size_t need = inv2_scratch_bytes(H->n, Q, nj);
   *ok = H->inv2_cap >= need;
@@ -77,11 +78,19 @@ int ensure_inv2(Handle* H, int Q, int nj, cudaStream_t st, bool* ok) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   FR3D_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
   if (cs != cudaStreamCaptureStatusNone) return FR3D_OK;   // no allocation inside a capture
+  if (H->inv2_denied && need >= H->inv2_denied) return FR3D_OK;
   FR3D_CUDA_TRY(cudaStreamSynchronize(st));
-  if (H->inv2_buf) cudaFree(H->inv2_buf);
+  dev_free(H->inv2_buf, H->inv2_cap);
   H->inv2_buf = nullptr;
   H->inv2_cap = 0;
-  FR3D_CUDA_TRY(cudaMalloc(&H->inv2_buf, need));
+  void* p = nullptr;
+  const int rc = dev_alloc(&p, need);
+  if (rc == FR3D_ERR_OOM) {
+    H->inv2_denied = need;
+    return FR3D_OK;
+  }
+  FR3D_TRY(rc);
+  H->inv2_buf = static_cast<float2*>(p);
   H->inv2_cap = need;
   *ok = true;
   return FR3D_OK;
@@ -96,10 +105,14 @@ int ensure_qctl(Handle* H, int nj, int Q, cudaStream_t st, bool* ok) {
   FR3D_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
   if (cs != cudaStreamCaptureStatusNone) return FR3D_OK;
   FR3D_CUDA_TRY(cudaStreamSynchronize(st));
-  if (H->qctl) cudaFree(H->qctl);
+  dev_free(H->qctl, H->qctl_n * sizeof(int));
   H->qctl = nullptr;
   H->qctl_n = 0;
-  FR3D_CUDA_TRY(cudaMalloc(&H->qctl, need * sizeof(int)));
+  void* p = nullptr;
+  const int rc = dev_alloc(&p, need * sizeof(int));
+  if (rc == FR3D_ERR_OOM) return FR3D_OK;
+  FR3D_TRY(rc);
+  H->qctl = static_cast<int*>(p);
   FR3D_CUDA_TRY(cudaMemset(H->qctl, 0, need * sizeof(int)));
   H->qctl_n = need;
   *ok = true;
@@ -115,15 +128,15 @@ int launch_variant(Handle* H, int v, int n, bool xi, const FusedArgs& a, int nj,
     case 4: {
       bool ok = false;
       FR3D_TRY(ensure_inv2(H, a.Q, nj, st, &ok));
-      if (!ok) return fused_launch<3>(n, xi, a, nj, st);   // inside a capture without the buffer
+      if (!ok) return fused_launch<3>(n, xi, a, nj, st);   // no room, or inside a capture without the buffer
       return inv2_launch(n, xi, a, nj, H->inv2_buf, st);
     }
     case 5: {
-      // other sizes and outputs, and a first call inside a capture: the register-accumulator tile
+      // other sizes and outputs, no room, and a first call inside a capture: the register-accumulator tile
       if (!inv_queue_supported(n, xi) || a.Zs) return fused_launch<3>(n, xi, a, nj, st);
       bool ok = false, okc = false;
       FR3D_TRY(ensure_inv2(H, a.Q, nj, st, &ok));
-      FR3D_TRY(ensure_qctl(H, nj, a.Q, st, &okc));
+      if (ok) FR3D_TRY(ensure_qctl(H, nj, a.Q, st, &okc));
       if (!ok || !okc) return fused_launch<3>(n, xi, a, nj, st);
       return inv_queue_launch(n, a, nj, H->inv2_buf, H->qctl, st);
     }
@@ -172,6 +185,10 @@ int choose_variant(Handle* H, const FusedArgs& a, int nj, bool xi, bool once, cu
     float ms = 0.f;
     if (st_ok == FR3D_OK && cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) st_ok = FR3D_ERR_CUDA;
     if (st_ok != FR3D_OK) break;
+    if (v >= kFusedVariants && H->inv2_cap < inv2_scratch_bytes(H->n, a.Q, nj)) {   // no room: variant 3 ran instead
+      H->fused_tune_ms[v] = 0.f;
+      continue;
+    }
     ms /= 3.f;
     H->fused_tune_ms[v] = ms;
     if (ms < best_ms) {

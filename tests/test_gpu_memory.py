@@ -231,3 +231,41 @@ def test_forward_operator_one_source_at_a_time(F, n, m, mp, prec):
     graph.replay()
     torch.cuda.synchronize()
     assert float((got - ref).norm()) <= tol * float(ref.norm())
+
+
+@pytest.mark.parametrize("n,v", [(96, 5), (192, 5), (256, 5), (192, 4)])
+def test_inverse_without_room_for_its_intermediate(F, n, v):
+    """The two-pass and the queue form run the register tile instead, with the same bits; the buffer is asked for once.
+    A tuner that cannot time them picks another."""
+    mp, q = 6, 2
+    w = I.make_workload(n, mp, q=q, n_incl=1, n_alpha=8, seed=76)
+    U = torch.as_tensor(w.noise, dtype=torch.float32, device="cuda")
+    opts = F.Opts(alphas=w.alphas, delta=0.3 * float(U.norm()), points=w.sources)
+    zeta = torch.empty((q, mp, n, n), device="cuda")
+
+    def handle():
+        H = F.kernel_transform(n, w.x0, w.h, w.zr, w.zy, w.nu)
+        F.autotune_mode(0)
+        F.invert(H, U, q, zeta, F.Opts(alphas=w.alphas, delta=0.3 * float(U.norm()), output=F.OUT_ZETA))   # the workspace
+        torch.cuda.synchronize()
+        return H
+
+    ref = torch.empty((mp, n, n), device="cuda")
+    H = handle()
+    F.autotune_mode(2 + 3)
+    F.invert(H, U, q, ref, opts)
+    H = handle()
+    F.autotune_mode(2 + v)
+    F.test_alloc_budget(0)
+    for asked in (1, 0, 0):
+        out = torch.full((mp, n, n), float("nan"), device="cuda")
+        F.invert(H, U, q, out, opts)
+        torch.cuda.synchronize()
+        assert F.test_alloc_budget(0) == asked and torch.equal(out, ref)
+    F.test_alloc_budget(-1)
+    H = handle()
+    F.test_alloc_budget(0)
+    F.autotune_mode(1)
+    F.invert(H, U, q, out.fill_(float("nan")), opts)   # (a shape no other test uses: the tuner runs)
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref) and F.autotune_query(H)[0] < 4
