@@ -31,9 +31,8 @@
 // mbarriers.  64 depths and 8 sources: n = 192 57 us (the fused cluster tiles 120, spilling; the two passes
 // 107), n = 256 80 us; n = 96 and 128 have too few tiles alone (40 and 38 us, as the other variants) and gain in a
 // batch (49 and 51 sources' planes: 184 -> 81 us and 167 -> 118 us).  Every wait (on a stage or a counter) is
-// bounded: on expiry every other wait of the launch ends at once, so the launch always ends, and its last CTA ORs
-// FR3D_INFO_TIMEOUT into the info word of every instance (a batch's instances wait in one queue, and any of their tiles may
-// have run on incomplete data).
+// bounded: on expiry every other wait of the launch ends at once, so the launch always ends, and every tile that waited in
+// vain ORs FR3D_INFO_TIMEOUT into its instance's info word.
 // The arithmetic of every output (the solve weights, the radix passes and their twiddles, the split, the
 // order of the accumulation over q) is the fused kernel's, so all variants return the same bits.
 #include <string.h>
@@ -96,7 +95,7 @@ struct QInst {
 // The launch: the instances (one in the arguments, or a device table of several), the ticket counter and
 // the flags that every instance shares.
 struct QLaunch {
-  int* ctl;          // [0] ticket, [1] CTAs finished (and kGaveUp), [2] a wait gave up
+  int* ctl;          // [0] ticket, [1] CTAs finished, [2] a wait gave up
   int* cnt_all;      // every instance's counters, contiguous (reset with ctl by the last CTA)
   int ncnt, total;   // counter ints; tickets of the launch
   int depths, lag;   // depths of all instances; depths between column and row tiles (at most `depths`)
@@ -141,25 +140,24 @@ __device__ __forceinline__ void decode_ticket(int k, int nj, int lag, int& kind,
 // source parameters of the first half (the first dependency step of a row tile)
 __device__ __forceinline__ int half_q(int Q) { return Q > 1 ? Q / 2 : 1; }
 
-// A wait gave up: the tile's own instance is flagged here.  Every other wait of the launch then ends at once, whichever
-// instance it belongs to, so the last CTA flags the others.  It learns of it from a bit of the counter of finished CTAs,
-// whose value it has in hand (a load of the flag in the launch's tail, or this report without the instance, which
-// takes the compiler two registers more, cost 0.3 us).
-constexpr int kGaveUp = 1 << 30;
 __device__ __forceinline__ void report_timeout(const QLaunch& ql, const QInst& qa) {
   atomicExch(ql.ctl + 2, 1);
-  atomicOr(ql.ctl + 1, kGaveUp);
   if (qa.f.info) atomicOr(qa.f.info, FR3D_INFO_TIMEOUT);
 }
 
-// Wait until *c >= target (acquire), or a wait elsewhere has given up; false if this one gave up.
+// Wait until *c >= target (acquire), or a wait elsewhere has given up; false if this one gave up.  Either way the tile runs
+// on incomplete data, and its instance is flagged: in a batch the wait elsewhere may have been another instance's.
+// (Flagging every instance from the launch's last CTA instead cost 0.4 us of each launch.)
 __device__ __forceinline__ bool wait_count(const QLaunch& ql, const QInst& qa, const int* c, int target) {
   const volatile int* gave_up = ql.ctl + 2;
   for (long it = 0; it < kSpinLimit; ++it) {
     int v;
     asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(c) : "memory");
     if (v >= target) return true;
-    if (*gave_up) return true;   // the results will be flagged; do not wait again
+    if (*gave_up) {   // do not wait again
+      if (qa.f.info) atomicOr(qa.f.info, FR3D_INFO_TIMEOUT);
+      return true;
+    }
     __nanosleep(128);
   }
   report_timeout(ql, qa);
@@ -490,21 +488,14 @@ __global__ void __launch_bounds__(kQThreads, kQMinBlocks) k_inv_queue(QLaunch ql
     else row_tile<N>(ql, s_inst, j, t, stage, buf, tab, bar, par, pol, tid);
     __syncthreads();   // before thread 0 overwrites the ticket
   }
-  // the last CTA to finish reports waits that gave up and resets the queue for the next launch
+  // the last CTA to finish resets the queue for the next launch
   if (tid == 0) {
     __threadfence();
-    const int finished = atomicAdd(ql.ctl + 1, 1);
-    if ((finished & (kGaveUp - 1)) == (int)gridDim.x - 1) {
+    if (atomicAdd(ql.ctl + 1, 1) == (int)gridDim.x - 1) {
       __threadfence();
       ql.ctl[0] = 0;
       ql.ctl[2] = 0;
       for (int e = 0; e < ql.ncnt; ++e) ql.cnt_all[e] = 0;
-      if (finished & kGaveUp) {
-        for (int i = 0; i < ql.ninst; ++i) {
-          int* info = ql.tab ? ql.tab[i].f.info : ql.inst0.f.info;
-          if (info) atomicOr(info, FR3D_INFO_TIMEOUT);
-        }
-      }
       __threadfence();
       ql.ctl[1] = 0;
     }
